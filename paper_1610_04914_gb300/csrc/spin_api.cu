@@ -93,6 +93,7 @@ Layout layout_for(const spin_params* p) {
     const bool generic = !tb.chain || p->path == 1 || !(tb.stages == 2 || tb.stages == 4);
     L.tmp = off;
     if (generic) off += align_up(elt * (size_t)(tb.stages + 1) * 3 * (size_t)g.N());
+    else if (elt == 8) off += align_up(elt * (size_t)stage64_scratch(tb.stages) * (size_t)g.N());
     L.partials = off;
     off += align_up(sizeof(double) * 5 * (size_t)observables_blocks(g));
     L.out_sample = off;

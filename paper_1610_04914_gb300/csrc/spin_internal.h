@@ -71,6 +71,10 @@ cudaError_t launch_step_patch(const StepLaunch<float>& L);
 cudaError_t prepare_patch_kernels();
 // The noise rotation of Eq. (s_rotation) over every site of L.out, in place.
 cudaError_t launch_pulse_lattice(const StepLaunch<float>& L);
+// FP64 chain tableaus, one kernel per stage; L.tmp holds stage64_scratch(S) N
+// doubles.
+cudaError_t launch_step_stage64(const StepLaunch<double>& L);
+int stage64_scratch(int stages);
 // FP32 fused six-stage (Butcher RK5) step in two three-stage segments; needs
 // L.tmp with 12N floats (the four carried vectors) and no per-site field.
 bool rk5_fused_supports(const StepLaunch<float>& L);

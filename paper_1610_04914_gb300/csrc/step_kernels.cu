@@ -1,20 +1,13 @@
 // One integration step delta t of the noiseless Landau-Lifshitz equation,
-// Eq. (LLL), on the periodic simple-cubic lattice, followed by
-// renormalisation and, on pulse steps, the noise rotation of Eq. (s_rotation).
-//
-// Two paths:
-//  * chain tableaus (RK4, RK2 midpoint, Heun: stage j needs only K_{j-1}):
-//    one fused kernel per step.  Each CTA owns an (x, y) tile plus a halo of
-//    S sites (S = number of stages) and marches along z.  At wavefront
-//    iteration t it loads spin plane t+S from HBM, evaluates stage j on plane
-//    t+S-j for j = 1..S (x-y neighbours of each stage input through shared
-//    memory, z neighbours from per-thread register rings) and writes the
-//    finished plane t.  Stage states never leave the SM: one read and one
-//    write of the state per step.
+// Eq. (LLL), on the simple-cubic lattice, followed by renormalisation and, on
+// pulse steps, the noise rotation of Eq. (s_rotation).  The paths:
+//  * chain tableaus (RK4, RK2 midpoint, Heun: stage j needs only K_{j-1}) in
+//    FP32: one fused kernel per step, all stages on chip (patch_tile.cuh);
+//  * chain tableaus in FP64: one kernel per stage (step_stage64.cu);
 //  * Butcher RK5 in FP32 without a per-site field: two fused three-stage
-//    segments (step_rk5.cu).
+//    segments (step_rk5.cu);
 //  * any tableau, any precision: one stencil kernel per stage plus a combine
-//    kernel, stage states in the workspace.
+//    kernel, stage states in the workspace (below).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -23,11 +16,6 @@
 #include "spin_internal.h"
 
 namespace spin {
-
-__host__ __device__ inline int wrap_index(int v, int n) {
-    int r = v % n;
-    return r < 0 ? r + n : r;
-}
 
 Tableau tableau_for(int integrator) {
     Tableau t{};
@@ -81,308 +69,14 @@ Tableau tableau_for(int integrator) {
     return t;
 }
 
-// ---------------------------------------------------------------------------
-// Fused chain-tableau step
-// ---------------------------------------------------------------------------
-
-template <typename real>
-struct ChainArgs {
-    const real* __restrict__ in0;
-    const real* __restrict__ in1;
-    const real* __restrict__ in2;
-    real* __restrict__ out0;
-    real* __restrict__ out1;
-    real* __restrict__ out2;
-    const real* __restrict__ hs0;
-    const real* __restrict__ hs1;
-    const real* __restrict__ hs2;
-    int nx, ny, nz, tz, n_iter;
-    real J, twoD, Hx, Hy, Hz, lambda;
-    real cdt[4];  // x_{j+1} = s + cdt[j-1] f_j   (dt folded in)
-    real bdt[4];  // s' = s + sum_j bdt[j-1] f_j
-    int renorm;
-    uint64_t seed, replica;
-    real sigma;
-    const long long* interval;
-    int bc;  // 1: free boundaries (outside columns and planes are zero spins)
-};
-
-// Register rings, indexed by (local plane index) & 3.
-template <typename real, int S, bool HSITE>
-struct Rings {
-    real s[4][3];
-    real x[S > 1 ? S - 1 : 1][4][3];  // x_j for j = 2..S
-    real y[4][3];
-    real h[HSITE ? 4 : 1][3];
-};
-
-template <typename real, int S, int BX, int BY, bool PREC, bool HSITE, bool PULSE, int P>
-__device__ __forceinline__ void chain_iteration(const ChainArgs<real>& a, Rings<real, S, HSITE>& r,
-                                                real* __restrict__ sh, int i, int t0, int z0, int col,
-                                                int plane, bool out_col, int tx, int ty, int xm, int xp,
-                                                int ym, int yp, long long k, real cmask) {
-    constexpr int TILE = BX * BY;
-    const int buf = P & 1;
-    real* shb = sh + buf * (S * 3 * TILE);
-    const int me = ty * BX + tx;
-
-    // 1. publish this iteration's stage inputs for the x-y neighbours
-#pragma unroll
-    for (int j = 1; j <= S; ++j) {
-        const int slot = (P + S - j) & 3;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const real v = (j == 1) ? r.s[slot][c] : r.x[j - 2][slot][c];
-            shb[((j - 1) * 3 + c) * TILE + me] = v;
-        }
-    }
-
-    // 2. stream in spin plane t+S (and the site field one plane behind)
-    const int t = i + t0;
-    {
-        const int gz = wrap_index(t + S, a.nz);
-        const long long off = (long long)gz * plane + col;
-        const int slot = (P + S) & 3;
-        r.s[slot][0] = __ldg(a.in0 + off);
-        r.s[slot][1] = __ldg(a.in1 + off);
-        r.s[slot][2] = __ldg(a.in2 + off);
-        if (a.bc) {
-            const real m = (t + S >= 0 && t + S < a.nz) ? cmask : real(0);
-            r.s[slot][0] *= m;
-            r.s[slot][1] *= m;
-            r.s[slot][2] *= m;
-        }
-        if (HSITE) {
-            const int gzh = wrap_index(t + S - 1, a.nz);
-            const long long offh = (long long)gzh * plane + col;
-            const int sl = (P + S - 1) & 3;
-            r.h[sl][0] = __ldg(a.hs0 + offh);
-            r.h[sl][1] = __ldg(a.hs1 + offh);
-            r.h[sl][2] = __ldg(a.hs2 + offh);
-        }
-    }
-    __syncthreads();
-
-    // 3. stage j on plane t+S-j, j = 1..S
-#pragma unroll
-    for (int j = 1; j <= S; ++j) {
-        const int slot = (P + S - j) & 3;
-        const int sm = (slot + 3) & 3, sp = (slot + 1) & 3;
-        const real* shj = shb + (j - 1) * 3 * TILE;
-        real cen[3], sum[3];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const real* q = shj + c * TILE;
-            cen[c] = (j == 1) ? r.s[slot][c] : r.x[j - 2][slot][c];
-            const real zmv = (j == 1) ? r.s[sm][c] : r.x[j - 2][sm][c];
-            const real zpv = (j == 1) ? r.s[sp][c] : r.x[j - 2][sp][c];
-            // neighbour order x-1, x+1, y-1, y+1, z-1, z+1
-            sum[c] = q[ty * BX + xm] + q[ty * BX + xp] + q[ym * BX + tx] + q[yp * BX + tx] + zmv + zpv;
-        }
-        real hx = a.J * sum[0] + a.Hx;
-        real hy = a.J * sum[1] + a.Hy;
-        real hz = a.J * sum[2] + a.Hz;
-        if (HSITE) {
-            hx += r.h[slot][0];
-            hy += r.h[slot][1];
-            hz += r.h[slot][2];
-        }
-        hz += a.twoD * cen[2];
-        real f[3];
-        llg_rhs<real, PREC>(cen[0], cen[1], cen[2], hx, hy, hz, a.lambda, f[0], f[1], f[2]);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            if (j == 1)
-                r.y[slot][c] = r.s[slot][c] + a.bdt[0] * f[c];
-            else
-                r.y[slot][c] = r.y[slot][c] + a.bdt[j - 1] * f[c];
-            if (j < S) r.x[j - 1][slot][c] = r.s[slot][c] + a.cdt[j - 1] * f[c];
-        }
-        if (j == S) {
-            // finished plane t
-            if (out_col && t >= z0 && t < z0 + a.tz && t < a.nz) {
-                real ox = r.y[slot][0], oy = r.y[slot][1], oz = r.y[slot][2];
-                if (a.renorm) {
-                    const real inv = Math<real>::rsqrt_(ox * ox + oy * oy + oz * oz);
-                    ox *= inv;
-                    oy *= inv;
-                    oz *= inv;
-                }
-                const long long site = (long long)t * plane + col;
-                if (PULSE) pulse_site<real>(ox, oy, oz, a.seed, (uint64_t)site, (uint64_t)k, a.replica, a.sigma);
-                a.out0[site] = ox;
-                a.out1[site] = oy;
-                a.out2[site] = oz;
-            }
-        }
-    }
-}
-
-template <typename real, int S, int BX, int BY, bool PREC, bool HSITE, bool PULSE>
-__global__ void __launch_bounds__(BX* BY, 1) k_step_chain(ChainArgs<real> a) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    real* sh = reinterpret_cast<real*>(smem_raw);
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const int gxu = (int)blockIdx.x * (BX - 2 * S) - S + tx;
-    const int gyu = (int)blockIdx.y * (BY - 2 * S) - S + ty;
-    const int gx = wrap_index(gxu, a.nx), gy = wrap_index(gyu, a.ny);
-    const bool out_col = tx >= S && tx < BX - S && ty >= S && ty < BY - S && gxu < a.nx && gyu < a.ny;
-    const int col = gy * a.nx + gx;
-    const int plane = a.nx * a.ny;
-    const int xm = tx > 0 ? tx - 1 : tx, xp = tx < BX - 1 ? tx + 1 : tx;
-    const int ym = ty > 0 ? ty - 1 : ty, yp = ty < BY - 1 ? ty + 1 : ty;
-    const int z0 = (int)blockIdx.z * a.tz;
-    const int t0 = z0 - 2 * S + 2;
-    const long long k = PULSE ? *a.interval : 0;
-    const real cmask = (a.bc && (gxu < 0 || gxu >= a.nx || gyu < 0 || gyu >= a.ny)) ? real(0) : real(1);
-
-    Rings<real, S, HSITE> r;
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            r.s[q][c] = real(0);
-            r.y[q][c] = real(0);
-#pragma unroll
-            for (int j = 0; j < (S > 1 ? S - 1 : 1); ++j) r.x[j][q][c] = real(0);
-            if (HSITE) r.h[q][c] = real(0);
-        }
-    // preload s at local planes S-2 and S-1
-#pragma unroll
-    for (int L = S - 2; L <= S - 1; ++L) {
-        const long long off = (long long)wrap_index(t0 + L, a.nz) * plane + col;
-        r.s[L & 3][0] = __ldg(a.in0 + off);
-        r.s[L & 3][1] = __ldg(a.in1 + off);
-        r.s[L & 3][2] = __ldg(a.in2 + off);
-        if (a.bc) {
-            const real m = (t0 + L >= 0 && t0 + L < a.nz) ? cmask : real(0);
-            r.s[L & 3][0] *= m;
-            r.s[L & 3][1] *= m;
-            r.s[L & 3][2] *= m;
-        }
-    }
-
-    for (int i = 0; i < a.n_iter; i += 4) {
-        chain_iteration<real, S, BX, BY, PREC, HSITE, PULSE, 0>(a, r, sh, i + 0, t0, z0, col, plane, out_col, tx, ty, xm, xp, ym, yp, k, cmask);
-        chain_iteration<real, S, BX, BY, PREC, HSITE, PULSE, 1>(a, r, sh, i + 1, t0, z0, col, plane, out_col, tx, ty, xm, xp, ym, yp, k, cmask);
-        chain_iteration<real, S, BX, BY, PREC, HSITE, PULSE, 2>(a, r, sh, i + 2, t0, z0, col, plane, out_col, tx, ty, xm, xp, ym, yp, k, cmask);
-        chain_iteration<real, S, BX, BY, PREC, HSITE, PULSE, 3>(a, r, sh, i + 3, t0, z0, col, plane, out_col, tx, ty, xm, xp, ym, yp, k, cmask);
-    }
-}
-
-template <typename real, int S, int BX, int BY, bool PREC, bool HSITE, bool PULSE>
-static cudaError_t launch_chain_t(const ChainArgs<real>& a, dim3 grid, cudaStream_t st) {
-    const size_t smem = sizeof(real) * 2 * S * 3 * BX * BY;
-    k_step_chain<real, S, BX, BY, PREC, HSITE, PULSE><<<grid, dim3(BX, BY), smem, st>>>(a);
-    return cudaGetLastError();
-}
-
-template <typename real, int S, int BX, int BY, bool PREC, bool HSITE, bool PULSE>
-static cudaError_t prepare_chain_t() {
-    const size_t smem = sizeof(real) * 2 * S * 3 * BX * BY;
-    return cudaFuncSetAttribute(k_step_chain<real, S, BX, BY, PREC, HSITE, PULSE>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-}
-
-template <typename real, int S, int BX, int BY>
-static cudaError_t dispatch_chain(const ChainArgs<real>& a, dim3 grid, cudaStream_t st, bool prec, bool hsite,
-                                  bool pulse, bool prepare) {
-#define SPIN_CHAIN_CASE(P_, H_, U_)                                                     \
-    if (prepare) {                                                                      \
-        cudaError_t e = prepare_chain_t<real, S, BX, BY, P_, H_, U_>();                 \
-        if (e != cudaSuccess) return e;                                                 \
-    } else if (prec == P_ && hsite == H_ && pulse == U_) {                              \
-        return launch_chain_t<real, S, BX, BY, P_, H_, U_>(a, grid, st);                \
-    }
-    SPIN_CHAIN_CASE(true, false, false)
-    SPIN_CHAIN_CASE(true, false, true)
-    SPIN_CHAIN_CASE(true, true, false)
-    SPIN_CHAIN_CASE(true, true, true)
-    SPIN_CHAIN_CASE(false, false, false)
-    SPIN_CHAIN_CASE(false, false, true)
-    SPIN_CHAIN_CASE(false, true, false)
-    SPIN_CHAIN_CASE(false, true, true)
-#undef SPIN_CHAIN_CASE
-    return prepare ? cudaSuccess : cudaErrorInvalidValue;
-}
-
-// CTA shape of the fused step: 32x16 columns for float, 16x16 for double
-// (the double register rings need up to 255 registers per thread).
-template <typename real>
-struct ChainShape;
-template <>
-struct ChainShape<float> {
-    static constexpr int BX = 32, BY = 16;
-};
-template <>
-struct ChainShape<double> {
-    static constexpr int BX = 16, BY = 16;
-};
-
 template <typename real>
 cudaError_t prepare_step_kernels() {
-    constexpr int BX = ChainShape<real>::BX, BY = ChainShape<real>::BY;
-    ChainArgs<real> a{};
-    cudaError_t e = dispatch_chain<real, 4, BX, BY>(a, dim3(1), 0, false, false, false, true);
-    if (e != cudaSuccess) return e;
-    e = dispatch_chain<real, 2, BX, BY>(a, dim3(1), 0, false, false, false, true);
-    if (e != cudaSuccess || sizeof(real) != 4) return e;
-    if ((e = prepare_patch_kernels()) != cudaSuccess) return e;
-    return prepare_rk5_kernels();
+    if (sizeof(real) != 4) return cudaSuccess;   // the FP64 kernels use no dynamic shared memory
+    const cudaError_t e = prepare_patch_kernels();
+    return e == cudaSuccess ? prepare_rk5_kernels() : e;
 }
 template cudaError_t prepare_step_kernels<float>();
 template cudaError_t prepare_step_kernels<double>();
-
-template <typename real>
-static cudaError_t launch_chain(const StepLaunch<real>& L) {
-    constexpr int BX = ChainShape<real>::BX, BY = ChainShape<real>::BY;
-    const Tableau& tb = *L.tab;
-    const int S = tb.stages;
-    ChainArgs<real> a{};
-    a.in0 = L.in[0];
-    a.in1 = L.in[1];
-    a.in2 = L.in[2];
-    a.out0 = L.out[0];
-    a.out1 = L.out[1];
-    a.out2 = L.out[2];
-    a.hs0 = L.hs[0];
-    a.hs1 = L.hs[1];
-    a.hs2 = L.hs[2];
-    a.nx = L.g.nx;
-    a.ny = L.g.ny;
-    a.nz = L.g.nz;
-    a.J = L.ph.J;
-    a.twoD = L.ph.twoD;
-    a.Hx = L.ph.H[0];
-    a.Hy = L.ph.H[1];
-    a.Hz = L.ph.H[2];
-    a.lambda = L.ph.lambda;
-    for (int j = 0; j < 4; ++j) {
-        a.cdt[j] = (j + 1 < S) ? (real)(tb.a[j + 1][j] * L.dt) : real(0);
-        a.bdt[j] = (j < S) ? (real)(tb.b[j] * L.dt) : real(0);
-    }
-    a.renorm = L.renorm;
-    a.seed = L.seed;
-    a.replica = L.replica;
-    a.sigma = L.sigma;
-    a.interval = L.d_interval;
-    a.bc = L.bc;
-    const int tiles_x = (L.g.nx + (BX - 2 * S) - 1) / (BX - 2 * S);
-    const int tiles_y = (L.g.ny + (BY - 2 * S) - 1) / (BY - 2 * S);
-    // z chunk: enough CTAs to fill the GPU twice over, chunks of >= 8 planes
-    int zc = L.g.nz;
-    const int want = 2 * 152;
-    while (zc > 8 && (long long)tiles_x * tiles_y * ((L.g.nz + zc - 1) / zc) < want) zc = (zc + 1) / 2;
-    a.tz = zc;
-    const int iters = zc + 2 * S - 2;
-    a.n_iter = (iters + 3) & ~3;
-    dim3 grid(tiles_x, tiles_y, (L.g.nz + zc - 1) / zc);
-    const bool hs = L.hs[0] != nullptr;
-    const bool prec = L.precession != 0;
-    if (S == 4) return dispatch_chain<real, 4, BX, BY>(a, grid, L.stream, prec, hs, L.pulse != 0, false);
-    if (S == 2) return dispatch_chain<real, 2, BX, BY>(a, grid, L.stream, prec, hs, L.pulse != 0, false);
-    return cudaErrorInvalidValue;
-}
 
 // ---------------------------------------------------------------------------
 // Generic tableau: stencil-per-stage kernels
@@ -564,7 +258,7 @@ template <typename real>
 cudaError_t launch_step(const StepLaunch<real>& L) {
     if (L.tab->chain && !L.force_generic && (L.tab->stages == 4 || L.tab->stages == 2)) {
         if (sizeof(real) == 4) return launch_step_patch(reinterpret_cast<const StepLaunch<float>&>(L));
-        return launch_chain<real>(L);
+        return launch_step_stage64(reinterpret_cast<const StepLaunch<double>&>(L));
     }
     if (sizeof(real) == 4 && !L.force_generic && rk5_fused_supports(reinterpret_cast<const StepLaunch<float>&>(L)))
         return launch_step_rk5(reinterpret_cast<const StepLaunch<float>&>(L));
