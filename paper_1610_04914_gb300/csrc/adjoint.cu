@@ -328,7 +328,7 @@ __device__ __forceinline__ void top_body(const TopArgs<real>& a, const AdjGeom<r
         const Words4 wd = noise_words(a.seed, (uint64_t)i, (uint64_t)a.k, a.replica);
         real g0, g1, g2;
         Gauss<real>::draw(wd, g0, g1, g2);
-        pulse_rotate<real>(l0, l1, l2, -a.sigma * g0, -a.sigma * g1, -a.sigma * g2);
+        pulse_rotate<real>(l0, l1, l2, -a.sigma * g0, -a.sigma * g1, -a.sigma * g2, a.sigma);
     }
     if (a.renorm) {
         real y0, y1, y2;

@@ -59,41 +59,62 @@ struct Gauss;
 
 template <>
 struct Gauss<double> {
+    // (k + 1/2) 2^-53, k = w >> 11, correctly rounded: k + 1/2 = m/2 with the
+    // 54-bit odd integer m, exact in a double unless its top bit is set, when
+    // the dropped last bit is a tie (to even).  Integer operations only: the
+    // conversion, the addition and the scaling would take three instructions
+    // of the FP64 pipe, which bounds the FP64 kernels.
+    __device__ __forceinline__ static double u01(uint64_t w) {
+        uint64_t m = (w >> 10) | 1ULL;
+        if (m >> 53) m = ((m >> 1) + ((m >> 1) & 1ULL)) << 1;
+        const int lz = __clzll((long long)m);
+        // value m 2^-54: exponent 63 - lz - 54, mantissa below the leading bit
+        return __longlong_as_double((long long)(((uint64_t)(1023 + 9 - lz) << 52) + ((m << lz) << 1 >> 12)));
+    }
     __device__ __forceinline__ static void draw(const Words4& w, double& g0, double& g1, double& g2) {
-        const double scale = 1.0 / 9007199254740992.0;  // 2^-53
-        const double u0 = ((double)(w.w[0] >> 11) + 0.5) * scale;
-        const double u1 = ((double)(w.w[1] >> 11) + 0.5) * scale;
-        const double u2 = ((double)(w.w[2] >> 11) + 0.5) * scale;
-        const double u3 = ((double)(w.w[3] >> 11) + 0.5) * scale;
-        const double r0 = sqrt(-2.0 * log(u0));
-        const double r2 = sqrt(-2.0 * log(u2));
-        double s1, c1, s3, c3;
-        sincospi(2.0 * u1, &s1, &c1);
-        sincospi(2.0 * u3, &s3, &c3);
+        const double r0 = sqrt(-2.0 * log(u01(w.w[0])));
+        const double r2 = sqrt(-2.0 * log(u01(w.w[2])));
+        double s1, c1;
+        sincospi(2.0 * u01(w.w[1]), &s1, &c1);
         g0 = r0 * c1;
         g1 = r0 * s1;
-        g2 = r2 * c3;
+        g2 = r2 * cospi(2.0 * u01(w.w[3]));
     }
 };
 
 template <>
 struct Gauss<float> {
     // Same real numbers as the double path, each rounded once to float: the
-    // 54-bit odd integer 2(w>>11)+1 converts with relative error 2^-24 at any
-    // magnitude, so small u keep their relative precision in the logarithm.
+    // 54-bit odd integer m = 2(w>>11)+1 to 24 bits.  From 2^34 on, m's bits
+    // above 2^32 (hi) and the 23 below them with the last one set (sticky: m is
+    // odd, and the rounding boundary lies at least one bit higher) convert
+    // exactly by exponent tricks, so one addition rounds like m itself.  Below
+    // (one word in 2^20), m shifted to 32 bits with the same sticky bit goes
+    // through the 32-bit conversion.  The 64-bit conversion instruction is
+    // avoided: it runs on GB300's narrow FP64 pipe.
     __device__ __forceinline__ static float u01(uint64_t w) {
-        return __ull2float_rn(((w >> 11) << 1) | 1ULL) * 5.5511151231257827e-17f;  // 2^-54
+        const unsigned wh = (unsigned)(w >> 32);
+        const unsigned hi = wh >> 10;
+        const unsigned b = __funnelshift_r((unsigned)w, wh, 19) & 0x7FFFFFu;
+        const float h = __fmaf_rn(__uint_as_float(0x4B000000u | hi), 2.384185791015625e-07f, -2.0f);   // hi 2^-22
+        const float l = __fmaf_rn(__uint_as_float(0x4B000001u | b), 2.8421709430404007e-14f,
+                                  -2.384185791015625e-07f);                                            // b 2^-45
+        float u = __fadd_rn(h, l);
+        if (hi < 4u) {
+            const unsigned lo = __funnelshift_r((unsigned)w, wh, 10) | 1u;   // m's low 32 bits
+            u = hi ? __uint2float_rn((hi << 30) | (lo >> 2) | 1u) * 2.2204460492503131e-16f   // 2^-52
+                   : __uint2float_rn(lo) * 5.5511151231257827e-17f;                           // 2^-54
+        }
+        return u;
     }
     __device__ __forceinline__ static void draw(const Words4& w, float& g0, float& g1, float& g2) {
-        const float u0 = u01(w.w[0]), u1 = u01(w.w[1]), u2 = u01(w.w[2]), u3 = u01(w.w[3]);
-        const float r0 = sqrtf(-2.0f * logf(u0));
-        const float r2 = sqrtf(-2.0f * logf(u2));
-        float s1, c1, s3, c3;
-        sincospif(2.0f * u1, &s1, &c1);
-        sincospif(2.0f * u3, &s3, &c3);
+        const float r0 = sqrtf(-2.0f * logf(u01(w.w[0])));
+        const float r2 = sqrtf(-2.0f * logf(u01(w.w[2])));
+        float s1, c1;
+        sincospif(2.0f * u01(w.w[1]), &s1, &c1);
         g0 = r0 * c1;
         g1 = r0 * s1;
-        g2 = r2 * c3;
+        g2 = r2 * cospif(2.0f * u01(w.w[3]));
     }
 };
 
@@ -112,12 +133,76 @@ struct Math<double> {
     __device__ __forceinline__ static void sincos_(double x, double* s, double* c) { sincos(x, s, c); }
 };
 
+// sin(phi)/phi and (1 - cos(phi))/phi^2 for p = phi^2 <= kSmallPhi2: the Taylor
+// series in p, truncated below the type's rounding (the first omitted terms are
+// p^7/15! = 1.3e-8 and p^11/23! = 1.6e-16 at p = 4).
+constexpr float kSmallPhi2 = 4.0f;
+__device__ __forceinline__ void rotation_series(float p, float& sinc, float& cosc) {
+    sinc = 1.0f / 6227020800.0f;
+    sinc = __fmaf_rn(sinc, p, -1.0f / 39916800.0f);
+    sinc = __fmaf_rn(sinc, p, 1.0f / 362880.0f);
+    sinc = __fmaf_rn(sinc, p, -1.0f / 5040.0f);
+    sinc = __fmaf_rn(sinc, p, 1.0f / 120.0f);
+    sinc = __fmaf_rn(sinc, p, -1.0f / 6.0f);
+    sinc = __fmaf_rn(sinc, p, 1.0f);
+    cosc = 1.0f / 87178291200.0f;
+    cosc = __fmaf_rn(cosc, p, -1.0f / 479001600.0f);
+    cosc = __fmaf_rn(cosc, p, 1.0f / 3628800.0f);
+    cosc = __fmaf_rn(cosc, p, -1.0f / 40320.0f);
+    cosc = __fmaf_rn(cosc, p, 1.0f / 720.0f);
+    cosc = __fmaf_rn(cosc, p, -1.0f / 24.0f);
+    cosc = __fmaf_rn(cosc, p, 0.5f);
+}
+__device__ __forceinline__ void rotation_series(double p, double& sinc, double& cosc) {
+    sinc = 1.0 / 51090942171709440000.0;              // 21!
+    sinc = fma(sinc, p, -1.0 / 121645100408832000.0);  // 19!
+    sinc = fma(sinc, p, 1.0 / 355687428096000.0);      // 17!
+    sinc = fma(sinc, p, -1.0 / 1307674368000.0);       // 15!
+    sinc = fma(sinc, p, 1.0 / 6227020800.0);
+    sinc = fma(sinc, p, -1.0 / 39916800.0);
+    sinc = fma(sinc, p, 1.0 / 362880.0);
+    sinc = fma(sinc, p, -1.0 / 5040.0);
+    sinc = fma(sinc, p, 1.0 / 120.0);
+    sinc = fma(sinc, p, -1.0 / 6.0);
+    sinc = fma(sinc, p, 1.0);
+    cosc = 1.0 / 1124000727777607680000.0;             // 22!
+    cosc = fma(cosc, p, -1.0 / 2432902008176640000.0);  // 20!
+    cosc = fma(cosc, p, 1.0 / 6402373705728000.0);      // 18!
+    cosc = fma(cosc, p, -1.0 / 20922789888000.0);       // 16!
+    cosc = fma(cosc, p, 1.0 / 87178291200.0);
+    cosc = fma(cosc, p, -1.0 / 479001600.0);
+    cosc = fma(cosc, p, 1.0 / 3628800.0);
+    cosc = fma(cosc, p, -1.0 / 40320.0);
+    cosc = fma(cosc, p, 1.0 / 720.0);
+    cosc = fma(cosc, p, -1.0 / 24.0);
+    cosc = fma(cosc, p, 0.5);
+}
+
 // Rotation of s by the angle vector phi = sigma G, Eq. (s_rotation):
 //   s' = s cos(phi) + (n x s) sin(phi) + n (n.s)(1 - cos(phi)),  n = phi/|phi|.
+// Small angles (almost every pulse within the method's applicability
+// condition sigma^2 <= 0.2) need no n: with the two even functions of phi
+// above, s' = s (1 - phi^2 B) + (phi x s) A + phi (phi.s) B, which saves the
+// square root, the division and the sine and cosine.
+// kSeriesSigma: sigma up to which the series is tried.  There phi^2 passes
+// kSmallPhi2 with probability below 1e-6 (chi-squared, three degrees), so the
+// warp does not diverge; for larger sigma every site takes the general form.
+constexpr float kSeriesSigma = 0.35f;
 template <typename real>
-__device__ __forceinline__ void pulse_rotate(real& sx, real& sy, real& sz, real px, real py, real pz) {
+__device__ __forceinline__ void pulse_rotate(real& sx, real& sy, real& sz, real px, real py, real pz, real sigma) {
     const real phi2 = px * px + py * py + pz * pz;
-    if (phi2 > real(0)) {
+    if (sigma <= real(kSeriesSigma) && phi2 <= real(kSmallPhi2)) {
+        real A, B;
+        rotation_series(phi2, A, B);
+        const real C = real(1) - phi2 * B;
+        const real ps = (px * sx + py * sy + pz * sz) * B;
+        const real cx = py * sz - pz * sy;
+        const real cy = pz * sx - px * sz;
+        const real cz = px * sy - py * sx;
+        sx = sx * C + cx * A + px * ps;
+        sy = sy * C + cy * A + py * ps;
+        sz = sz * C + cz * A + pz * ps;
+    } else if (phi2 > real(0)) {
         const real phi = Math<real>::sqrt_(phi2);
         const real inv = real(1) / phi;
         const real nx = px * inv, ny = py * inv, nz = pz * inv;
@@ -144,7 +229,7 @@ __device__ __forceinline__ void pulse_site(real& sx, real& sy, real& sz, uint64_
     const Words4 w = noise_words(seed, site, k, replica);
     real g0, g1, g2;
     Gauss<real>::draw(w, g0, g1, g2);
-    pulse_rotate<real>(sx, sy, sz, sigma * g0, sigma * g1, sigma * g2);
+    pulse_rotate<real>(sx, sy, sz, sigma * g0, sigma * g1, sigma * g2, sigma);
 }
 
 // Exact float -> double for FP64 accumulation of FP32 terms: sign, exponent

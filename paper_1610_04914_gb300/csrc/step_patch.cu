@@ -206,14 +206,19 @@ cudaError_t patch_dispatch(const PatchArgs& a, dim3 grid, cudaStream_t st, bool 
 }
 
 // The noise pulse on its own, over every site of the lattice (all threads
-// busy): on pulse steps of a single lattice the step kernel runs without its
-// epilogue rotation and this kernel rotates the finished state in place.  The
+// busy; bound by instruction issue, about half of it the 64-bit products of
+// Philox4x64-10: 34.8 us at 128^3, 257 us at 256^3, 37.2 and 280 before the
+// series rotation and the conversions without the FP64 pipe; four rounds of
+// resident blocks rather than one even out the tail, 256^3 260 -> 257 us): on
+// pulse steps of a single lattice the step kernel runs without its epilogue
+// rotation and this kernel rotates the finished state in place.  The
 // arithmetic per site is the fused epilogue's, so the results are identical.
 __global__ void __launch_bounds__(256) k_pulse_f32(float* __restrict__ sx, float* __restrict__ sy, float* __restrict__ sz,
-                                                   long long N, uint64_t seed, const long long* __restrict__ interval,
+                                                   unsigned N, uint64_t seed, const long long* __restrict__ interval,
                                                    uint64_t replica, float sigma) {
     const uint64_t k = (uint64_t)*interval;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
+    // N < 2^31 and the stride is far below 2^31, so the index cannot wrap
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
         float x = sx[i], y = sy[i], z = sz[i];
         pulse_site<float>(x, y, z, seed, (uint64_t)i, k, replica, sigma);
         sx[i] = x;
@@ -359,9 +364,9 @@ cudaError_t launch_step_patch(const StepLaunch<float>& L) {
 
 cudaError_t launch_pulse_lattice(const StepLaunch<float>& L) {
     const long long N = L.g.N();
-    const int blocks = (int)std::max<long long>(1, std::min<long long>((N + 255) / 256, 152LL * 8));
-    k_pulse_f32<<<blocks, 256, 0, L.stream>>>(L.out[0], L.out[1], L.out[2], N, L.seed, L.d_interval, L.replica,
-                                              L.sigma);
+    const int blocks = (int)std::max<long long>(1, std::min<long long>((N + 255) / 256, 152LL * 32));
+    k_pulse_f32<<<blocks, 256, 0, L.stream>>>(L.out[0], L.out[1], L.out[2], (unsigned)N, L.seed, L.d_interval,
+                                              L.replica, L.sigma);
     return cudaGetLastError();
 }
 

@@ -91,10 +91,10 @@ __global__ void __launch_bounds__(256) k_pulse_batch(float* __restrict__ sx, flo
     const ObsBlock ob = blocks[blockIdx.x];
     const BatchRep rp = reps[ob.rep];
     const uint64_t k = (uint64_t)*interval;
-    const long long first = (long long)ob.row0 * rp.L;
-    const long long count = (long long)ob.nrows * rp.L;
-    for (long long q = threadIdx.x; q < count; q += blockDim.x) {
-        const long long i = first + q;          // site index within the replica
+    const unsigned first = (unsigned)ob.row0 * rp.L;
+    const unsigned count = (unsigned)ob.nrows * rp.L;
+    for (unsigned q = threadIdx.x; q < count; q += blockDim.x) {
+        const unsigned i = first + q;           // site index within the replica (below 2^31)
         const long long g = rp.off + i;
         float x = sx[g], y = sy[g], z = sz[g];
         pulse_site<float>(x, y, z, seed, (uint64_t)i, k, (uint64_t)ob.rep, rp.sigma);

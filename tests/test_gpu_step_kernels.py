@@ -3,6 +3,7 @@ the FP64 oracle on the same inputs and noise (tolerances of the parity tests:
 one step agrees to 1e-13 in FP64 and 2e-6 in FP32, three steps run here)."""
 import numpy as np
 import pytest
+import torch
 
 import spin_inputs
 from gpu_helpers import run_gpu, run_oracle
@@ -34,3 +35,32 @@ def _compare(gpu, orc, shape, tol, hsite=False, **kw):
 def test_fp64_stage_kernels(gpu, orc, integ, shape, precession, hsite, bc):
     _compare(gpu, orc, shape, 1e-13, hsite=hsite, precision=64, integrator=getattr(gpu, integ),
              precession=precession, bc=bc)
+
+
+# free spins (J = D = H = 0): three pulses with sigma at both sides of the
+# series limit 0.35, far above it (general form), and angles from ~0 to beyond
+# phi^2 = 4.  FP32: the angle carries ~4 roundings of G (5e-7 at phi = 2), the
+# rotation ~10 more, per pulse.
+@pytest.mark.parametrize("prec,tol", [(32, 5e-6), (64, 1e-13)])
+@pytest.mark.parametrize("sigma", [0.01, 0.3499, 0.3501, 1.55])
+def test_pulse_rotation_forms(gpu, orc, prec, tol, sigma):
+    n = (33, 17, 40)
+    p = gpu.Params(*n, J=0.0, D=0.0, H=(0.0, 0.0, 0.0), lam=0.5, T=sigma ** 2, dt=1.0, R=1, seed=5, precision=prec)
+    s0 = spin_inputs.random_spins(*n, seed=3)
+    got, _ = run_gpu(gpu, p, s0, 3)
+    ref, _ = run_oracle(orc, p, s0, 3)
+    assert np.max(np.abs(got - ref)) < tol
+
+
+def test_noise_uniforms_small_words(gpu):
+    """2^22 draws, so that words below 2^44 (the conversion's other branch, one
+    in 2^20) occur: Gaussians against numpy's from the same words."""
+    words, g32 = gpu.spin_noise_draw(9, 3, 1, 1 << 22, precision=32)
+    torch.cuda.synchronize()
+    w = words.cpu().numpy().view(np.uint64)
+    assert int((w < np.uint64(1 << 44)).sum()) > 0
+    u = ((w >> np.uint64(11)).astype(np.float64) + 0.5) * 2.0 ** -53
+    r0, r2 = np.sqrt(-2 * np.log(u[:, 0])), np.sqrt(-2 * np.log(u[:, 2]))
+    a, b = 2 * np.pi * u[:, 1], 2 * np.pi * u[:, 3]
+    ref = np.stack([r0 * np.cos(a), r0 * np.sin(a), r2 * np.cos(b)], 1)
+    assert np.max(np.abs(g32.cpu().numpy() - ref)) < 1e-5
