@@ -3,20 +3,30 @@
 //   M = (1/N) sum_i s_i
 //   E = (1/N) [ -J sum_<ij> s_i.s_j - D sum_i s_iz^2 - sum_i (H + h_i).s_i ]
 // each bond counted once through the three forward neighbours of every site.
-// Pass 1: grid-stride FP64 partial sums, warp-shuffle then shared-memory
-// reduction, one 5-double record per block.  Pass 2: one block adds the block
-// records in a fixed order, so the result is bitwise reproducible.
+// Pass 1: one warp per lattice row, FP64 sums per lane, one 5-double record per
+// block.  Pass 2: one block adds the block records in a fixed order, so the
+// result is bitwise reproducible.
+//
+// What bounds it: GB300's FP64 pipe (a warp's FP64 instruction holds it for 16
+// cycles of the SM) and, in pass 2, its latency.  So float terms convert to
+// double by integer operations (to_f64), the block's sums are formed from
+// shared memory with every lane busy (4 x 512 values by four warps: 80
+// instructions; shuffle trees in every warp took 25 per warp, 400 per block),
+// and 1/N comes from the host.  The two passes at 128^3, cold: FP32 25.5 + 9.7
+// -> 16.0 + 7.3 us, FP64 121 -> 77 us for the first.
 #include <cuda_runtime.h>
 
 #include <algorithm>
 
+#include "spin_device.cuh"
 #include "spin_internal.h"
 
 namespace spin {
 
 namespace {
 
-constexpr int kObsThreads = 256;
+constexpr int kObsThreads = 512;
+constexpr int kObsWarps = kObsThreads / 32;
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
@@ -24,221 +34,237 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
+// Sums of one lane over its share of rows: M and E in FP64, non-finite spins.
+struct ObsLane {
+    double m[3], e;
+    int bad;
+};
+
+// Add one row's terms: row arrays at a, b, c (this row), their y+1 and z+1
+// rows, weights wy, wz of those bonds and of the bond across the row's end.
+// FP32: the terms are formed and summed over the lane's sites of the row in
+// FP32, then added in FP64.  FP64: the sums of bonds and s_z^2 are kept apart
+// and combined once per row, 13 FP64 operations a site.
 template <typename real, bool HSITE>
-__global__ void __launch_bounds__(kObsThreads) k_obs_partial(const real* __restrict__ sx, const real* __restrict__ sy,
-                                                             const real* __restrict__ sz, const real* __restrict__ hx,
-                                                             const real* __restrict__ hy, const real* __restrict__ hz,
-                                                             int nx, int ny, int nz, double J, double D, double H0,
-                                                             double H1, double H2, double* __restrict__ partials,
-                                                             int bc) {
-    // one warp per lattice row (y, z); lanes stride along x, so no per-site
-    // index division and the row's loads are coalesced
-    const long long P = (long long)nx * ny;
-    const int rows = ny * nz;
-    const int lane = threadIdx.x & 31;
-    const int warps_total = gridDim.x * (blockDim.x >> 5);
-    double m0 = 0, m1 = 0, m2 = 0, e = 0, bad = 0;
-    for (int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); row < rows; row += warps_total) {
-        const int y = row % ny;
-        const int z = row / ny;
-        const long long rb = (long long)z * P + (long long)y * nx;
-        const long long rby = (long long)z * P + (long long)(y + 1 == ny ? 0 : y + 1) * nx;
-        const long long rbz = (long long)(z + 1 == nz ? 0 : z + 1) * P + (long long)y * nx;
-        // per-site terms in the state's precision, summed over this lane's
-        // sites of the row, then added into the FP64 accumulators
-        real rm0 = 0, rm1 = 0, rm2 = 0, re = 0;
-        int rbad = 0;
-        const real Jr = (real)J, Dr = (real)D, H0r = (real)H0, H1r = (real)H1, H2r = (real)H2;
-        for (int x = lane; x < nx; x += 32) {
-            const long long i = rb + x;
-            const long long ix = rb + (x + 1 == nx ? 0 : x + 1);
-            const long long iy = rby + x;
-            const long long iz = rbz + x;
-            const real a = sx[i], b = sy[i], c = sz[i];
-            if (!isfinite(a) || !isfinite(b) || !isfinite(c)) rbad += 1;
-            rm0 += a;
-            rm1 += b;
-            rm2 += c;
-            // forward bonds; with free boundaries none crosses the last face
-            const real wx = (bc && x + 1 == nx) ? real(0) : real(1);
-            const real wy = (bc && y + 1 == ny) ? real(0) : real(1);
-            const real wz = (bc && z + 1 == nz) ? real(0) : real(1);
-            const real bond = a * (wx * sx[ix] + wy * sx[iy] + wz * sx[iz]) + b * (wx * sy[ix] + wy * sy[iy] + wz * sy[iz]) +
-                              c * (wx * sz[ix] + wy * sz[iy] + wz * sz[iz]);
+__device__ __forceinline__ void obs_row(ObsLane& o, const real* __restrict__ sx, const real* __restrict__ sy,
+                                        const real* __restrict__ sz, const real* __restrict__ hx,
+                                        const real* __restrict__ hy, const real* __restrict__ hz, long long rb,
+                                        long long rby, long long rbz, int nx, bool openx, bool openy, bool openz,
+                                        double J, double D, double H0, double H1, double H2, int lane) {
+    real m0 = 0, m1 = 0, m2 = 0, e = 0, sq = 0, hs = 0;
+    const real Jr = (real)J, Dr = (real)D, H0r = (real)H0, H1r = (real)H1, H2r = (real)H2;
+#pragma unroll 2
+    for (int x = lane; x < nx; x += 32) {
+        const long long i = rb + x;
+        const bool last = x + 1 == nx;
+        const long long ix = rb + (last ? 0 : x + 1), iy = rby + x, iz = rbz + x;
+        const real a = sx[i], b = sy[i], c = sz[i];
+        if (!finite_bits(a) || !finite_bits(b) || !finite_bits(c)) o.bad += 1;
+        m0 += a;
+        m1 += b;
+        m2 += c;
+        // forward bonds; with free boundaries none crosses the last face
+        const bool ox = openx && last;
+        const real x0 = ox ? real(0) : sx[ix], x1 = ox ? real(0) : sy[ix], x2 = ox ? real(0) : sz[ix];
+        const real y0 = openy ? real(0) : sx[iy], y1 = openy ? real(0) : sy[iy], y2 = openy ? real(0) : sz[iy];
+        const real z0 = openz ? real(0) : sx[iz], z1 = openz ? real(0) : sy[iz], z2 = openz ? real(0) : sz[iz];
+        if (sizeof(real) == 8) {
+            e += a * (x0 + y0 + z0);
+            e += b * (x1 + y1 + z1);
+            e += c * (x2 + y2 + z2);
+            sq += c * c;
+            if (HSITE) hs += hx[i] * a + hy[i] * b + hz[i] * c;
+        } else {
+            // contractions written out: the single-lattice and the batched
+            // kernel then round alike
+            const real bond = fma(a, x0 + y0 + z0, fma(b, x1 + y1 + z1, c * (x2 + y2 + z2)));
             real f0 = H0r, f1 = H1r, f2 = H2r;
             if (HSITE) {
                 f0 += hx[i];
                 f1 += hy[i];
                 f2 += hz[i];
             }
-            re += -Jr * bond - Dr * c * c - (f0 * a + f1 * b + f2 * c);
+            e += fma(-Jr, bond, fma(-Dr * c, c, -fma(f0, a, fma(f1, b, f2 * c))));
         }
-        m0 += (double)rm0;
-        m1 += (double)rm1;
-        m2 += (double)rm2;
-        e += (double)re;
-        bad += (double)rbad;
     }
-    __shared__ double red[kObsThreads / 32][5];
-    m0 = warp_sum(m0);
-    m1 = warp_sum(m1);
-    m2 = warp_sum(m2);
-    e = warp_sum(e);
-    bad = warp_sum(bad);
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    if (l == 0) {
-        red[w][0] = m0;
-        red[w][1] = m1;
-        red[w][2] = m2;
-        red[w][3] = e;
-        red[w][4] = bad;
-    }
-    __syncthreads();
-    if (threadIdx.x < 5) {
-        double acc = 0;
-        for (int q = 0; q < kObsThreads / 32; ++q) acc += red[q][threadIdx.x];
-        partials[(long long)blockIdx.x * 5 + threadIdx.x] = acc;
-    }
+    o.m[0] += to_f64(m0);
+    o.m[1] += to_f64(m1);
+    o.m[2] += to_f64(m2);
+    if (sizeof(real) == 8)
+        o.e += -J * (double)e - D * (double)sq - (H0 * (double)m0 + H1 * (double)m1 + H2 * (double)m2) - (double)hs;
+    else
+        o.e += to_f64(e);
 }
 
-__global__ void __launch_bounds__(kObsThreads) k_obs_final(const double* __restrict__ partials, int nblocks, long long N,
+// The block's record (5 doubles) from its lanes' sums, in a fixed order.
+__device__ __forceinline__ void obs_block(const ObsLane& o, double* __restrict__ rec) {
+    __shared__ double red[4][kObsThreads];
+    __shared__ int bad;
+    const int t = threadIdx.x, w = t >> 5, l = t & 31;
+    if (t == 0) bad = 0;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) red[q][t] = o.m[q];
+    red[3][t] = o.e;
+    __syncthreads();
+    const unsigned nb = __reduce_add_sync(0xffffffffu, (unsigned)o.bad);
+    if (l == 0 && nb) atomicAdd(&bad, (int)nb);
+    if (w < 4) {
+        double v[kObsWarps];
+#pragma unroll
+        for (int q = 0; q < kObsWarps; ++q) v[q] = red[w][q * 32 + l];
+#pragma unroll
+        for (int s = kObsWarps / 2; s > 0; s >>= 1)
+#pragma unroll
+            for (int q = 0; q < s; ++q) v[q] += v[q + s];
+        const double r = warp_sum(v[0]);
+        if (l == 0) rec[w] = r;
+    }
+    __syncthreads();
+    if (t == 0) rec[4] = (double)bad;
+}
+
+// Pass 2 is launched while pass 1 drains and waits for it here.
+__device__ __forceinline__ void obs_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+__device__ __forceinline__ void obs_go() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+
+template <typename real, bool HSITE>
+__global__ void __launch_bounds__(kObsThreads, 2)
+    k_obs_partial(const real* __restrict__ sx, const real* __restrict__ sy, const real* __restrict__ sz,
+                  const real* __restrict__ hx, const real* __restrict__ hy, const real* __restrict__ hz, int nx,
+                  int ny, int nz, double J, double D, double H0, double H1, double H2, double* __restrict__ partials,
+                  int bc) {
+    // one warp per lattice row (y, z); lanes stride along x, so no per-site
+    // index division and the row's loads are coalesced
+    obs_go();
+    const long long P = (long long)nx * ny;
+    const int rows = ny * nz;
+    const int lane = threadIdx.x & 31;
+    ObsLane o{};
+    for (int row = blockIdx.x * kObsWarps + (threadIdx.x >> 5); row < rows; row += gridDim.x * kObsWarps) {
+        const int z = row / ny, y = row - z * ny;
+        obs_row<real, HSITE>(o, sx, sy, sz, hx, hy, hz, (long long)row * nx,
+                             (long long)z * P + (long long)(y + 1 == ny ? 0 : y + 1) * nx,
+                             (long long)(z + 1 == nz ? 0 : z + 1) * P + (long long)y * nx, nx, bc, bc && y + 1 == ny,
+                             bc && z + 1 == nz, J, D, H0, H1, H2, lane);
+    }
+    obs_block(o, partials + (long long)blockIdx.x * 5);
+}
+
+__global__ void __launch_bounds__(kObsThreads) k_obs_final(const double* __restrict__ partials, int nblocks, double invN,
                                                            double* __restrict__ out5, double* __restrict__ ring, int ring_len,
                                                            long long* __restrict__ interval,
                                                            long long* __restrict__ sample_count, int R) {
-    __shared__ double red[kObsThreads / 32][5];
-    double acc[5] = {0, 0, 0, 0, 0};
-    for (int b = threadIdx.x; b < nblocks; b += blockDim.x)
-        for (int q = 0; q < 5; ++q) acc[q] += partials[(long long)b * 5 + q];
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    for (int q = 0; q < 5; ++q) {
-        const double v = warp_sum(acc[q]);
-        if (l == 0) red[w][q] = v;
+    __shared__ double tot[5];
+    obs_wait();
+    long long m = 0, count = 0;
+    if (ring && threadIdx.x == 0) {
+        m = *interval;
+        count = *sample_count;
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t[5] = {0, 0, 0, 0, 0};
-        for (int ww = 0; ww < kObsThreads / 32; ++ww)
-            for (int q = 0; q < 5; ++q) t[q] += red[ww][q];
-        const double invN = 1.0 / (double)N;
-        out5[0] = t[0] * invN;
-        out5[1] = t[1] * invN;
-        out5[2] = t[2] * invN;
-        out5[3] = t[3] * invN;
-        out5[4] = t[4];
-        if (ring) {
-            const long long m = *interval;
-            double* rec = ring + (*sample_count % ring_len) * 5;
-            rec[0] = (double)((m + 1) * (long long)R);
-            rec[1] = out5[0];
-            rec[2] = out5[1];
-            rec[3] = out5[2];
-            rec[4] = out5[3];
-            *interval = m + 1;
-            *sample_count = *sample_count + 1;
+    // warp w < 5 adds value w over the blocks
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+    if (w < 5) {
+        double a0 = 0, a1 = 0, a2 = 0, a3 = 0;   // four chains: the additions' latency, not their number, counts here
+        int b = l;
+        for (; b + 96 < nblocks; b += 128) {
+            a0 += partials[(long long)b * 5 + w];
+            a1 += partials[(long long)(b + 32) * 5 + w];
+            a2 += partials[(long long)(b + 64) * 5 + w];
+            a3 += partials[(long long)(b + 96) * 5 + w];
+        }
+        for (; b < nblocks; b += 32) a0 += partials[(long long)b * 5 + w];
+        const double r = warp_sum((a0 + a1) + (a2 + a3));
+        if (l == 0) {
+            tot[w] = w < 4 ? r * invN : r;
+            out5[w] = tot[w];
         }
     }
+    __syncthreads();
+    if (ring && threadIdx.x == 0) {
+        double* rec = ring + (count % ring_len) * 5;
+        rec[0] = (double)((m + 1) * (long long)R);
+        rec[1] = tot[0];
+        rec[2] = tot[1];
+        rec[3] = tot[2];
+        rec[4] = tot[3];
+        *interval = m + 1;
+        *sample_count = count + 1;
+    }
+}
+
+// Launch pass 2 as a programmatic dependent of pass 1.
+template <typename Kern, typename... Args>
+cudaError_t launch_final(Kern kernel, int threads, cudaStream_t st, Args... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(1);
+    cfg.blockDim = dim3(threads);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
 // Batched replicas: the same row-wise reduction, each block on a row range
 // of one replica; the final pass gives one record per replica.
-__global__ void __launch_bounds__(kObsThreads) k_obs_batch_partial(const float* __restrict__ sx, const float* __restrict__ sy,
-                                                                   const float* __restrict__ sz,
-                                                                   const BatchRep* __restrict__ reps,
-                                                                   const ObsBlock* __restrict__ blocks, double J, double D,
-                                                                   double H0, double H1, double H2,
-                                                                   double* __restrict__ partials) {
+__global__ void __launch_bounds__(kObsThreads, 2)
+    k_obs_batch_partial(const float* __restrict__ sx, const float* __restrict__ sy, const float* __restrict__ sz,
+                        const BatchRep* __restrict__ reps, const ObsBlock* __restrict__ blocks, double J, double D,
+                        double H0, double H1, double H2, double* __restrict__ partials) {
+    obs_go();
     const ObsBlock ob = blocks[blockIdx.x];
     const BatchRep rp = reps[ob.rep];
     const int L = rp.L;
     const long long P = (long long)L * L;
-    const float* ax = sx + rp.off;
-    const float* ay = sy + rp.off;
-    const float* az = sz + rp.off;
     const int lane = threadIdx.x & 31;
-    double m0 = 0, m1 = 0, m2 = 0, e = 0, bad = 0;
-    const float Jr = (float)J, Dr = (float)D, H0r = (float)H0, H1r = (float)H1, H2r = (float)H2;
-    for (int row = ob.row0 + (threadIdx.x >> 5); row < ob.row0 + ob.nrows; row += (blockDim.x >> 5)) {
-        const int y = row % L, z = row / L;
-        const long long rb = (long long)z * P + (long long)y * L;
-        const long long rby = (long long)z * P + (long long)(y + 1 == L ? 0 : y + 1) * L;
-        const long long rbz = (long long)(z + 1 == L ? 0 : z + 1) * P + (long long)y * L;
-        float rm0 = 0, rm1 = 0, rm2 = 0, re = 0;
-        int rbad = 0;
-        for (int x = lane; x < L; x += 32) {
-            const long long i = rb + x, ix = rb + (x + 1 == L ? 0 : x + 1), iy = rby + x, iz = rbz + x;
-            const float a = ax[i], b = ay[i], c = az[i];
-            if (!isfinite(a) || !isfinite(b) || !isfinite(c)) rbad += 1;
-            rm0 += a;
-            rm1 += b;
-            rm2 += c;
-            const float bond = a * (ax[ix] + ax[iy] + ax[iz]) + b * (ay[ix] + ay[iy] + ay[iz]) + c * (az[ix] + az[iy] + az[iz]);
-            re += -Jr * bond - Dr * c * c - (H0r * a + H1r * b + H2r * c);
-        }
-        m0 += (double)rm0;
-        m1 += (double)rm1;
-        m2 += (double)rm2;
-        e += (double)re;
-        bad += (double)rbad;
+    ObsLane o{};
+    for (int row = ob.row0 + (threadIdx.x >> 5); row < ob.row0 + ob.nrows; row += kObsWarps) {
+        const int z = row / L, y = row - z * L;
+        obs_row<float, false>(o, sx + rp.off, sy + rp.off, sz + rp.off, nullptr, nullptr, nullptr, (long long)row * L,
+                              (long long)z * P + (long long)(y + 1 == L ? 0 : y + 1) * L,
+                              (long long)(z + 1 == L ? 0 : z + 1) * P + (long long)y * L, L, false, false, false, J, D,
+                              H0, H1, H2, lane);
     }
-    __shared__ double red[kObsThreads / 32][5];
-    m0 = warp_sum(m0);
-    m1 = warp_sum(m1);
-    m2 = warp_sum(m2);
-    e = warp_sum(e);
-    bad = warp_sum(bad);
-    const int w = threadIdx.x >> 5;
-    if (lane == 0) {
-        red[w][0] = m0;
-        red[w][1] = m1;
-        red[w][2] = m2;
-        red[w][3] = e;
-        red[w][4] = bad;
-    }
-    __syncthreads();
-    if (threadIdx.x < 5) {
-        double acc = 0;
-        for (int q = 0; q < kObsThreads / 32; ++q) acc += red[q][threadIdx.x];
-        partials[(long long)blockIdx.x * 5 + threadIdx.x] = acc;
-    }
+    obs_block(o, partials + (long long)blockIdx.x * 5);
 }
 
-__global__ void __launch_bounds__(kObsThreads) k_obs_batch_final(const double* __restrict__ partials,
-                                                                 const int* __restrict__ first_block,
-                                                                 const BatchRep* __restrict__ reps, int nrep,
-                                                                 double* __restrict__ out, double* __restrict__ ring,
-                                                                 int ring_len, long long* __restrict__ interval,
-                                                                 long long* __restrict__ sample_count, int R) {
+// one warp per replica at a time, 32 warps
+constexpr int kObsFinalThreads = 1024;
+__global__ void __launch_bounds__(kObsFinalThreads) k_obs_batch_final(const double* __restrict__ partials,
+                                                                      const int* __restrict__ first_block,
+                                                                      const BatchRep* __restrict__ reps, int nrep,
+                                                                      double* __restrict__ out, double* __restrict__ ring,
+                                                                      int ring_len, long long* __restrict__ interval,
+                                                                      long long* __restrict__ sample_count, int R) {
+    obs_wait();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const long long m = ring ? *interval : 0;
-    const long long slot = ring ? (*sample_count % ring_len) : 0;
-    for (int r = w; r < nrep; r += blockDim.x >> 5) {
+    const long long count = ring ? *sample_count : 0;
+    const long long slot = ring ? count % ring_len : 0;
+    for (int r = w; r < nrep; r += kObsFinalThreads >> 5) {
+        const double L = (double)reps[r].L;
+        const double invN = 1.0 / (L * L * L);
         double acc[5] = {0, 0, 0, 0, 0};
         for (int b = first_block[r] + lane; b < first_block[r + 1]; b += 32)
             for (int q = 0; q < 5; ++q) acc[q] += partials[(long long)b * 5 + q];
         for (int q = 0; q < 5; ++q) acc[q] = warp_sum(acc[q]);
         if (lane == 0) {
-            const double L = (double)reps[r].L;
-            const double invN = 1.0 / (L * L * L);
             double* o = out + (long long)r * 5;
-            o[0] = acc[0] * invN;
-            o[1] = acc[1] * invN;
-            o[2] = acc[2] * invN;
-            o[3] = acc[3] * invN;
+            for (int q = 0; q < 4; ++q) o[q] = acc[q] * invN;
             o[4] = acc[4];
             if (ring) {
                 double* rec = ring + (slot * nrep + r) * 5;
                 rec[0] = (double)((m + 1) * (long long)R);
-                rec[1] = o[0];
-                rec[2] = o[1];
-                rec[3] = o[2];
-                rec[4] = o[3];
+                for (int q = 0; q < 4; ++q) rec[1 + q] = acc[q] * invN;
             }
         }
     }
     __syncthreads();
     if (ring && threadIdx.x == 0) {
         *interval = m + 1;
-        *sample_count = *sample_count + 1;
+        *sample_count = count + 1;
     }
 }
 
@@ -246,8 +272,7 @@ __global__ void __launch_bounds__(kObsThreads) k_obs_batch_final(const double* _
 
 int observables_blocks(Geom g) {
     const long long rows = (long long)g.ny * g.nz;
-    const long long warps_per_block = kObsThreads / 32;
-    return (int)std::max<long long>(1, std::min<long long>((rows + warps_per_block - 1) / warps_per_block, 152LL * 4));
+    return (int)std::max<long long>(1, std::min<long long>((rows + kObsWarps - 1) / kObsWarps, 152LL * 2));
 }
 
 template <typename real>
@@ -263,9 +288,10 @@ cudaError_t launch_observables(const real* s[3], const real* hs[3], Geom g, Phys
         k_obs_partial<real, false><<<nblocks, kObsThreads, 0, stream>>>(s[0], s[1], s[2], nullptr, nullptr, nullptr, g.nx, g.ny,
                                                                         g.nz, (double)ph.J, D, (double)ph.H[0],
                                                                         (double)ph.H[1], (double)ph.H[2], partials, bc);
-    k_obs_final<<<1, kObsThreads, 0, stream>>>(partials, nblocks, g.N(), out5, sample_ring, ring, d_interval,
-                                               d_sample_count, R);
-    return cudaGetLastError();
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    return launch_final(k_obs_final, 160, stream, (const double*)partials, nblocks, 1.0 / (double)g.N(), out5,
+                        sample_ring, ring, d_interval, d_sample_count, R);
 }
 
 cudaError_t launch_observables_batch(const float* s[3], const BatchRep* reps, const ObsBlock* blocks, int nblocks,
@@ -274,9 +300,10 @@ cudaError_t launch_observables_batch(const float* s[3], const BatchRep* reps, co
                                      long long* d_sample_count, int R, cudaStream_t stream) {
     k_obs_batch_partial<<<nblocks, kObsThreads, 0, stream>>>(s[0], s[1], s[2], reps, blocks, ph.J, 0.5 * ph.twoD,
                                                              ph.H[0], ph.H[1], ph.H[2], partials);
-    k_obs_batch_final<<<1, kObsThreads, 0, stream>>>(partials, first_block, reps, nrep, out, ring, ring_len, d_interval,
-                                                     d_sample_count, R);
-    return cudaGetLastError();
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    return launch_final(k_obs_batch_final, kObsFinalThreads, stream, (const double*)partials, first_block, reps, nrep, out,
+                        ring, ring_len, d_interval, d_sample_count, R);
 }
 
 template cudaError_t launch_observables<float>(const float* s[3], const float* hs[3], Geom, Phys<double>, double*, int,

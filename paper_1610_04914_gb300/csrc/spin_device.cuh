@@ -232,22 +232,28 @@ __device__ __forceinline__ void pulse_site(real& sx, real& sy, real& sz, uint64_
     pulse_rotate<real>(sx, sy, sz, sigma * g0, sigma * g1, sigma * g2, sigma);
 }
 
-// Exact float -> double for FP64 accumulation of FP32 terms: sign, exponent
-// rebased from 127 to 1023, mantissa shifted into the top of the 52-bit field
-// -- integer operations only, because this GPU's FP64 pipe, which the
-// hardware conversion uses, runs at ~1/76 of the FP32 rate and is needed for
-// the FP64 additions themselves.  Zeros keep their sign; subnormal, infinite
-// and NaN floats take the hardware conversion.
+// Exact float -> double for FP64 accumulation of FP32 terms, with 32-bit integer
+// operations only: the hardware conversion uses this GPU's FP64 pipe, which
+// runs at ~1/64 of the FP32 rate and is needed for the FP64 additions
+// themselves.  The exponent is rebased from 127 to 1023; subnormals are first
+// scaled by 2^24; zeros, infinities and NaNs keep their sign and payload.
+// (Every case is selected, none branched to: a conversion instruction in a
+// rare branch would be executed always, with its result discarded.)
 __device__ __forceinline__ double to_f64(float f) {
     const unsigned b = __float_as_uint(f);
-    const unsigned e = (b >> 23) & 0xFFu;
-    const unsigned long long sign = (unsigned long long)(b & 0x80000000u) << 32;
-    if ((b & 0x7FFFFFFFu) == 0u) return __longlong_as_double((long long)sign);
-    if (e == 0u || e == 0xFFu) return (double)f;
-    return __longlong_as_double(
-        (long long)(sign | ((unsigned long long)(e + 896u) << 52) | ((unsigned long long)(b & 0x7FFFFFu) << 29)));
+    const bool sub = (b & 0x7F800000u) == 0u;
+    const unsigned m = sub ? __float_as_uint(f * 16777216.0f) : b;
+    const unsigned e = (m >> 23) & 0xFFu;
+    const unsigned x = e == 0u ? 0u : e == 0xFFu ? 2047u : e + (sub ? 872u : 896u);
+    return __hiloint2double((int)((b & 0x80000000u) | (x << 20) | ((m & 0x7FFFFFu) >> 3)), (int)(m << 29));
 }
 __device__ __forceinline__ double to_f64(double d) { return d; }
+
+// isfinite without the FP64 pipe (its comparison would run there)
+__device__ __forceinline__ bool finite_bits(float f) { return (__float_as_uint(f) & 0x7F800000u) != 0x7F800000u; }
+__device__ __forceinline__ bool finite_bits(double d) {
+    return ((unsigned)__double2hiint(d) & 0x7FF00000u) != 0x7FF00000u;
+}
 
 // Right-hand side of Eq. (LLL) with a rectangular-noise field zeta, which
 // enters the precession term only:  f = s x (H + zeta) - lambda s x (s x H).

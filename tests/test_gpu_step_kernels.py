@@ -39,28 +39,60 @@ def test_fp64_stage_kernels(gpu, orc, integ, shape, precession, hsite, bc):
 
 # free spins (J = D = H = 0): three pulses with sigma at both sides of the
 # series limit 0.35, far above it (general form), and angles from ~0 to beyond
-# phi^2 = 4.  FP32: the angle carries ~4 roundings of G (5e-7 at phi = 2), the
-# rotation ~10 more, per pulse.
-@pytest.mark.parametrize("prec,tol", [(32, 5e-6), (64, 1e-13)])
+# phi^2 = 4.  Per pulse the angle carries about four roundings of G, relative,
+# so phi times that, and the rotation about ten more; |G| < 6 here.
+@pytest.mark.parametrize("prec", [32, 64])
 @pytest.mark.parametrize("sigma", [0.01, 0.3499, 0.3501, 1.55])
-def test_pulse_rotation_forms(gpu, orc, prec, tol, sigma):
+def test_pulse_rotation_forms(gpu, orc, prec, sigma):
     n = (33, 17, 40)
     p = gpu.Params(*n, J=0.0, D=0.0, H=(0.0, 0.0, 0.0), lam=0.5, T=sigma ** 2, dt=1.0, R=1, seed=5, precision=prec)
     s0 = spin_inputs.random_spins(*n, seed=3)
     got, _ = run_gpu(gpu, p, s0, 3)
     ref, _ = run_oracle(orc, p, s0, 3)
+    tol = 1e-13 if prec == 64 else 3 * (4 * 6 * sigma + 10) * 2.0 ** -24
     assert np.max(np.abs(got - ref)) < tol
 
 
 def test_noise_uniforms_small_words(gpu):
     """2^22 draws, so that words below 2^44 (the conversion's other branch, one
-    in 2^20) occur: Gaussians against numpy's from the same words."""
+    in 2^20) occur: Gaussians against numpy's from the same words, whose
+    uniforms the FP32 path rounds once to float."""
     words, g32 = gpu.spin_noise_draw(9, 3, 1, 1 << 22, precision=32)
     torch.cuda.synchronize()
     w = words.cpu().numpy().view(np.uint64)
     assert int((w < np.uint64(1 << 44)).sum()) > 0
-    u = ((w >> np.uint64(11)).astype(np.float64) + 0.5) * 2.0 ** -53
+    u = (((w >> np.uint64(11)).astype(np.float64) + 0.5) * 2.0 ** -53).astype(np.float32).astype(np.float64)
     r0, r2 = np.sqrt(-2 * np.log(u[:, 0])), np.sqrt(-2 * np.log(u[:, 2]))
     a, b = 2 * np.pi * u[:, 1], 2 * np.pi * u[:, 3]
     ref = np.stack([r0 * np.cos(a), r0 * np.sin(a), r2 * np.cos(b)], 1)
     assert np.max(np.abs(g32.cpu().numpy() - ref)) < 1e-5
+
+
+# rows fewer than, equal to and beyond one block's warps and the grid; row ends
+# inside and at a lane's stride; M and E against a plain FP64 reduction (FP32
+# terms: bounds of the parity tests)
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+@pytest.mark.parametrize("bc", [0, 1])
+@pytest.mark.parametrize("shape", [(1, 1, 1), (33, 1, 1), (1, 1, 17), (32, 4, 4), (31, 5, 3), (70, 16, 305)])
+def test_observables_reduction(gpu, dtype, bc, shape):
+    nx, ny, nz = shape
+    s = torch.from_numpy(spin_inputs.random_spins(nx, ny, nz, seed=6)).to("cuda", dtype)
+    h = torch.from_numpy(spin_inputs.site_fields(nx, ny, nz, 0.3, seed=7)).to("cuda", dtype)
+    J, D, H = 0.8, 0.3, (0.1, -0.2, 0.4)
+    out = torch.zeros(5, dtype=torch.float64, device="cuda")
+    gpu.spin_observables_noalloc(s, J, D, H, out, h_site=h, bc=bc)
+    x, f = s.double(), h.double() + torch.tensor(H, dtype=torch.float64, device="cuda").reshape(3, 1, 1, 1)
+    bonds = x.new_zeros(())
+    for d in (1, 2, 3):
+        p = x * torch.roll(x, -1, d)
+        bonds = bonds + (p.narrow(d, 0, x.shape[d] - 1).sum() if bc else p.sum())
+    n = nx * ny * nz
+    E = float((-J * bonds - D * x[2].square().sum() - (f * x).sum()) / n)
+    M = (x.reshape(3, -1).sum(1) / n).tolist()
+    got = out.tolist()
+    tm, te = (1e-6, 5e-6) if dtype == torch.float32 else (1e-13, 1e-13)
+    assert max(abs(a - b) for a, b in zip(got[:3], M)) < tm and abs(got[3] - E) < te and got[4] == 0
+    s[1, nz // 2, ny // 2, nx - 1] = float("inf")
+    s[0, 0, 0, 0] = float("nan")
+    gpu.spin_observables_noalloc(s, J, D, H, out, h_site=h, bc=bc)
+    assert out[4].item() == (1 if n == 1 else 2 if (nz // 2, ny // 2, nx - 1) != (0, 0, 0) else 1)
