@@ -73,69 +73,92 @@ struct MetroMath<float> {
     __device__ __forceinline__ static float sqrt_(float x) { return sqrtf(x); }
 };
 
+// What bounds it: instruction issue, a third of it the 64-bit products of
+// Philox4x64-10 (which run in half of the FMA pipe).  The random numbers do
+// not depend on the state, so each launch is a programmatic dependent of the
+// one before: it draws the numbers of its trials while that one drains, and
+// waits before it reads a spin.  Neighbour indices are selected, not branched
+// to, in 32 bits (N < 2^31); accepted trials are counted per block.
+__device__ __forceinline__ void colour_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+__device__ __forceinline__ void colour_go() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+
 template <typename real, bool HSITE>
-__global__ void __launch_bounds__(256) k_metropolis(MetroArgs<real> A) {
+__global__ void __launch_bounds__(256) k_metropolis(const __grid_constant__ MetroArgs<real> A) {
     using M = MetroMath<real>;
-    const int hx = (A.nx + 1) >> 1;
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long total = (long long)A.ny * A.nz * hx;
-    int acc = 0;
-    if (t < total) {
-        const int q = (int)(t % hx);
-        const long long row = t / hx;
-        const int y = (int)(row % A.ny);
-        const int z = (int)(row / A.ny);
-        const int x = 2 * q + ((y + z + A.color) & 1);
-        if (x < A.nx) {
-            const long long i = x + (long long)A.nx * (y + (long long)A.ny * z);
-            const Words4 w = philox4x64_10((uint64_t)i, (uint64_t)A.sweep, A.replica, 0ULL, A.seed, kStreamMC);
-            real cz, st, sp, cp;
-            M::polar(w.w[0], cz, st);
-            M::sincos2pi(M::u(w.w[1]), &sp, &cp);
-            const real o0 = A.s0[i], o1 = A.s1[i], o2 = A.s2[i];
-            real n0 = o0 + A.Rtrial * (st * cp), n1 = o1 + A.Rtrial * (st * sp), n2 = o2 + A.Rtrial * cz;
-            const real nn = M::sqrt_(n0 * n0 + n1 * n1 + n2 * n2);
-            n0 /= nn;
-            n1 /= nn;
-            n2 /= nn;
-            // exchange field of the six neighbours (free boundaries: missing
-            // neighbours contribute nothing)
-            real l0 = 0, l1 = 0, l2 = 0;
-            const long long sx = 1, sy = A.nx, sz = (long long)A.nx * A.ny;
-            auto add = [&](long long j) {
-                l0 += A.s0[j];
-                l1 += A.s1[j];
-                l2 += A.s2[j];
-            };
-            if (x > 0) add(i - sx); else if (!A.bc) add(i + (A.nx - 1) * sx);
-            if (x < A.nx - 1) add(i + sx); else if (!A.bc) add(i - (A.nx - 1) * sx);
-            if (y > 0) add(i - sy); else if (!A.bc) add(i + (A.ny - 1) * sy);
-            if (y < A.ny - 1) add(i + sy); else if (!A.bc) add(i - (A.ny - 1) * sy);
-            if (z > 0) add(i - sz); else if (!A.bc) add(i + (A.nz - 1) * sz);
-            if (z < A.nz - 1) add(i + sz); else if (!A.bc) add(i - (A.nz - 1) * sz);
-            l0 = A.J * l0 + A.Hx;
-            l1 = A.J * l1 + A.Hy;
-            l2 = A.J * l2 + A.Hz;
-            if (HSITE) {
-                l0 += A.h0[i];
-                l1 += A.h1[i];
-                l2 += A.h2[i];
-            }
-            const real e_old = -(o0 * l0 + o1 * l1 + o2 * l2) - A.D * o2 * o2;
-            const real e_new = -(n0 * l0 + n1 * l1 + n2 * l2) - A.D * n2 * n2;
-            const real dE = e_new - e_old;
-            if (dE <= real(0) || M::u(w.w[2]) < M::exp_(-dE / A.T)) {
-                A.s0[i] = n0;
-                A.s1[i] = n1;
-                A.s2[i] = n2;
-                acc = 1;
-            }
+    colour_go();
+    const unsigned hx = (unsigned)(A.nx + 1) >> 1;
+    const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;   // below 2^31 + one block
+    const unsigned total = (unsigned)A.ny * A.nz * hx;          // at most (N + rows)/2, below 2^31
+    bool acc = false;
+    const unsigned row = t / hx;
+    const int z = (int)(row / (unsigned)A.ny);
+    const int y = (int)row - z * A.ny;
+    const int x = 2 * (int)(t - row * hx) + ((y + z + A.color) & 1);
+    const bool valid = t < total && x < A.nx;
+    const int i = (int)((unsigned)x + (unsigned)A.nx * row);
+    const Words4 w = philox4x64_10((uint64_t)(unsigned)i, (uint64_t)A.sweep, A.replica, 0ULL, A.seed, kStreamMC);
+    real cz, st, sp, cp;
+    M::polar(w.w[0], cz, st);
+    M::sincos2pi(M::u(w.w[1]), &sp, &cp);
+    const real ua = M::u(w.w[2]);
+    colour_wait();
+    if (valid) {
+        const int P = A.nx * A.ny;
+        const bool xl = x > 0, xh = x < A.nx - 1, yl = y > 0, yh = y < A.ny - 1, zl = z > 0, zh = z < A.nz - 1;
+        const int nb[6] = {xl ? i - 1 : i + (A.nx - 1), xh ? i + 1 : i - (A.nx - 1),
+                           yl ? i - A.nx : i + (P - A.nx), yh ? i + A.nx : i - (P - A.nx),
+                           zl ? i - P : i + (A.nz - 1) * P, zh ? i + P : i - (A.nz - 1) * P};
+        // free boundaries: a missing neighbour contributes nothing
+        const bool in[6] = {xl || !A.bc, xh || !A.bc, yl || !A.bc, yh || !A.bc, zl || !A.bc, zh || !A.bc};
+        const real o0 = A.s0[i], o1 = A.s1[i], o2 = A.s2[i];
+        real l0 = 0, l1 = 0, l2 = 0;
+#pragma unroll
+        for (int q = 0; q < 6; ++q) {
+            l0 += in[q] ? A.s0[nb[q]] : real(0);
+            l1 += in[q] ? A.s1[nb[q]] : real(0);
+            l2 += in[q] ? A.s2[nb[q]] : real(0);
+        }
+        l0 = A.J * l0 + A.Hx;
+        l1 = A.J * l1 + A.Hy;
+        l2 = A.J * l2 + A.Hz;
+        if (HSITE) {
+            l0 += A.h0[i];
+            l1 += A.h1[i];
+            l2 += A.h2[i];
+        }
+        real n0 = o0 + A.Rtrial * (st * cp), n1 = o1 + A.Rtrial * (st * sp), n2 = o2 + A.Rtrial * cz;
+        const real nn = M::sqrt_(n0 * n0 + n1 * n1 + n2 * n2);
+        n0 /= nn;
+        n1 /= nn;
+        n2 /= nn;
+        const real e_old = -(o0 * l0 + o1 * l1 + o2 * l2) - A.D * o2 * o2;
+        const real e_new = -(n0 * l0 + n1 * l1 + n2 * l2) - A.D * n2 * n2;
+        const real dE = e_new - e_old;
+        if (dE <= real(0) || ua < M::exp_(-dE / A.T)) {
+            A.s0[i] = n0;
+            A.s1[i] = n1;
+            A.s2[i] = n2;
+            acc = true;
         }
     }
     if (A.accepted) {
-        const unsigned cnt = __reduce_add_sync(0xffffffffu, (unsigned)acc);
-        if ((threadIdx.x & 31) == 0 && cnt) atomicAdd(A.accepted, (unsigned long long)cnt);
+        const int cnt = __syncthreads_count(acc);
+        if (threadIdx.x == 0 && cnt) atomicAdd(A.accepted, (unsigned long long)cnt);
     }
+}
+
+template <typename real, bool HSITE>
+cudaError_t launch_colour(const MetroArgs<real>& A, unsigned blocks, cudaStream_t st) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_metropolis<real, HSITE>, A);
 }
 
 // Colour c of sweeps sweep0 .. sweep0+nsweeps-1 (c < 0: both colours, 0 then 1).
@@ -174,10 +197,8 @@ cudaError_t sweeps_t(const spin_params* p, void* s, const void* h_site, uint64_t
         for (int c = 0; c < 2; ++c) {
             if (only_color >= 0 && c != only_color) continue;
             A.color = c;
-            if (h_site)
-                k_metropolis<real, true><<<blocks, 256, 0, st>>>(A);
-            else
-                k_metropolis<real, false><<<blocks, 256, 0, st>>>(A);
+            const cudaError_t e = h_site ? launch_colour<real, true>(A, blocks, st) : launch_colour<real, false>(A, blocks, st);
+            if (e != cudaSuccess) return e;
         }
     }
     return cudaGetLastError();
