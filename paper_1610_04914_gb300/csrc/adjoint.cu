@@ -35,6 +35,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "pdl.cuh"
 #include "spin_device.cuh"
 #include "spin_internal.h"
 
@@ -45,11 +46,6 @@ namespace {
 constexpr int kAT = 256;                 // threads per block (8 warps)
 constexpr int kAW = kAT / 32;
 
-// Programmatic dependent launch of the transposed-step kernels: each is
-// launched while the kernel before it drains, and waits (griddepcontrol.wait,
-// a no-op without a programmatic dependency) for that kernel's completion and
-// memory before touching global memory; each lets its successor launch once
-// all of its blocks have stored their results.
 // Resident blocks per SM asked of the chain-tableau transposes: 6 blocks of
 // 256 threads cap them at 40 registers (from 44-48), so a 64^3 lattice's 1024
 // blocks take 1.12 rounds of 152 SMs instead of 1.35; measured 4.5% faster
@@ -58,37 +54,12 @@ constexpr int kAW = kAT / 32;
 #ifndef SPIN_ADJ_MINB
 #define SPIN_ADJ_MINB 6
 #endif
-#ifndef SPIN_ADJ_PDL
-#define SPIN_ADJ_PDL 1
-#endif
-__device__ __forceinline__ void pdl_wait() {
-#if SPIN_ADJ_PDL
-    asm volatile("griddepcontrol.wait;\n" ::: "memory");
-#endif
-}
-__device__ __forceinline__ void pdl_trigger() {
-#if SPIN_ADJ_PDL
-    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
-#endif
-}
+
+// The transposed-step kernels are programmatic dependents (pdl.cuh) that let
+// their successor launch once all of their blocks have stored their results.
 template <typename Kern, typename... Args>
-cudaError_t pdl_launch(Kern kernel, dim3 grid, cudaStream_t st, Args... args) {
-#if SPIN_ADJ_PDL
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(kAT);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, args...);
-#else
-    kernel<<<grid, kAT, 0, st>>>(args...);
-    return cudaGetLastError();
-#endif
+cudaError_t adj_launch(Kern kernel, dim3 grid, cudaStream_t st, const Args&... args) {
+    return launch_pdl(kernel, grid, dim3(kAT), 0, st, args...);
 }
 
 // A site of the lattice with its six neighbours (x-1, x+1, y-1, y+1, z-1, z+1;
@@ -376,7 +347,7 @@ __global__ void __launch_bounds__(kAT) k_adj_top_w(TopArgs<real> a, AdjGeom<real
     const Site<real> st = site_here<real>(G.nx, G.ny, G.nz, G.bc);
     const int i = st.i;
     top_body<real, PREC, HSITE, S, CHAIN>(a, G, st, a.lam.c[0][i], a.lam.c[1][i], a.lam.c[2][i]);
-    pdl_trigger();
+    pdl_go();
 }
 
 // Stage j of the transposed step: the neighbour part ("x-part") of stage j,
@@ -449,7 +420,7 @@ __global__ void __launch_bounds__(kAT, CHAIN ? SPIN_ADJ_MINB : 1) k_adj_xw(XWArg
         const real v[3] = {G.dt * lk[0], G.dt * lk[1], G.dt * lk[2]};
         w_part<real, PREC, HSITE>(a.prev, a.hs, st, G, v, a.wn, a.un, a.gh, a.gjd);
     }
-    pdl_trigger();
+    pdl_go();
 }
 
 // The first stage's x-part of step m (lam_s += lx, final: the adjoint of step
@@ -478,7 +449,7 @@ __global__ void __launch_bounds__(kAT, CHAIN ? SPIN_ADJ_MINB : 1) k_adj_x0_top(X
         l[c] = lm[c] + lx;
     }
     top_body<real, PREC, HSITE, S, CHAIN>(ta, G, st, l[0], l[1], l[2]);
-    pdl_trigger();
+    pdl_go();
 }
 
 // FP64 sums of kSumParts consecutive parts of each of the arrays at v + c N
@@ -632,21 +603,21 @@ cudaError_t launch_xw_t(int j, int S, bool chain, const XWArgs<real>& a, const A
     if (!adj_tableau_supported(S, chain)) return cudaErrorInvalidValue;
     if (chain) {
         switch (j) {
-            case 0: return pdl_launch(k_adj_xw<real, PREC, HSITE, 0, false, true>, gb, st, a, G);
-            case 1: return pdl_launch(k_adj_xw<real, PREC, HSITE, 1, true, true>, gb, st, a, G);
-            case 2: return pdl_launch(k_adj_xw<real, PREC, HSITE, 2, true, true>, gb, st, a, G);
-            case 3: return pdl_launch(k_adj_xw<real, PREC, HSITE, 3, true, true>, gb, st, a, G);
+            case 0: return adj_launch(k_adj_xw<real, PREC, HSITE, 0, false, true>, gb, st, a, G);
+            case 1: return adj_launch(k_adj_xw<real, PREC, HSITE, 1, true, true>, gb, st, a, G);
+            case 2: return adj_launch(k_adj_xw<real, PREC, HSITE, 2, true, true>, gb, st, a, G);
+            case 3: return adj_launch(k_adj_xw<real, PREC, HSITE, 3, true, true>, gb, st, a, G);
             default: return cudaErrorInvalidValue;
         }
         return cudaSuccess;
     }
     switch (j) {
-        case 0: return pdl_launch(k_adj_xw<real, PREC, HSITE, 0, false, false>, gb, st, a, G);
-        case 1: return pdl_launch(k_adj_xw<real, PREC, HSITE, 1, true, false>, gb, st, a, G);
-        case 2: return pdl_launch(k_adj_xw<real, PREC, HSITE, 2, true, false>, gb, st, a, G);
-        case 3: return pdl_launch(k_adj_xw<real, PREC, HSITE, 3, true, false>, gb, st, a, G);
-        case 4: return pdl_launch(k_adj_xw<real, PREC, HSITE, 4, true, false>, gb, st, a, G);
-        case 5: return pdl_launch(k_adj_xw<real, PREC, HSITE, 5, true, false>, gb, st, a, G);
+        case 0: return adj_launch(k_adj_xw<real, PREC, HSITE, 0, false, false>, gb, st, a, G);
+        case 1: return adj_launch(k_adj_xw<real, PREC, HSITE, 1, true, false>, gb, st, a, G);
+        case 2: return adj_launch(k_adj_xw<real, PREC, HSITE, 2, true, false>, gb, st, a, G);
+        case 3: return adj_launch(k_adj_xw<real, PREC, HSITE, 3, true, false>, gb, st, a, G);
+        case 4: return adj_launch(k_adj_xw<real, PREC, HSITE, 4, true, false>, gb, st, a, G);
+        case 5: return adj_launch(k_adj_xw<real, PREC, HSITE, 5, true, false>, gb, st, a, G);
         default: return cudaErrorInvalidValue;
     }
     return cudaSuccess;
@@ -667,8 +638,8 @@ cudaError_t launch_xw(bool prec, bool hsite, int j, int S, bool chain, const XWA
 template <typename real, bool PREC, bool HSITE>
 cudaError_t launch_x0_top_t(int S, bool chain, const XWArgs<real>& xa, const TopArgs<real>& ta, const AdjGeom<real>& G,
                             dim3 gb, cudaStream_t st) {
-    if (chain && S == 2) return pdl_launch(k_adj_x0_top<real, PREC, HSITE, 2, true>, gb, st, xa, ta, G);
-    else if (chain && S == 4) return pdl_launch(k_adj_x0_top<real, PREC, HSITE, 4, true>, gb, st, xa, ta, G);
+    if (chain && S == 2) return adj_launch(k_adj_x0_top<real, PREC, HSITE, 2, true>, gb, st, xa, ta, G);
+    else if (chain && S == 4) return adj_launch(k_adj_x0_top<real, PREC, HSITE, 4, true>, gb, st, xa, ta, G);
     else return cudaErrorInvalidValue;
     return cudaSuccess;
 }
@@ -687,9 +658,9 @@ cudaError_t launch_x0_top(bool prec, bool hsite, int S, bool chain, const XWArgs
 template <typename real, bool PREC, bool HSITE>
 cudaError_t launch_top_w_t(int S, bool chain, const TopArgs<real>& a, const AdjGeom<real>& G, dim3 gb,
                            cudaStream_t st) {
-    if (chain && S == 2) return pdl_launch(k_adj_top_w<real, PREC, HSITE, 2, true>, gb, st, a, G);
-    else if (chain && S == 4) return pdl_launch(k_adj_top_w<real, PREC, HSITE, 4, true>, gb, st, a, G);
-    else if (!chain && S == 6) return pdl_launch(k_adj_top_w<real, PREC, HSITE, 6, false>, gb, st, a, G);
+    if (chain && S == 2) return adj_launch(k_adj_top_w<real, PREC, HSITE, 2, true>, gb, st, a, G);
+    else if (chain && S == 4) return adj_launch(k_adj_top_w<real, PREC, HSITE, 4, true>, gb, st, a, G);
+    else if (!chain && S == 6) return adj_launch(k_adj_top_w<real, PREC, HSITE, 6, false>, gb, st, a, G);
     else return cudaErrorInvalidValue;
     return cudaSuccess;
 }

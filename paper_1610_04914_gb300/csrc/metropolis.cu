@@ -15,6 +15,7 @@
 #include <cmath>
 
 #include "../../include/spinpulse.h"
+#include "pdl.cuh"
 #include "spin_device.cuh"
 #include "spin_internal.h"
 
@@ -79,13 +80,10 @@ struct MetroMath<float> {
 // one before: it draws the numbers of its trials while that one drains, and
 // waits before it reads a spin.  Neighbour indices are selected, not branched
 // to, in 32 bits (N < 2^31); accepted trials are counted per block.
-__device__ __forceinline__ void colour_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
-__device__ __forceinline__ void colour_go() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
-
 template <typename real, bool HSITE>
 __global__ void __launch_bounds__(256) k_metropolis(const __grid_constant__ MetroArgs<real> A) {
     using M = MetroMath<real>;
-    colour_go();
+    pdl_go();
     const unsigned hx = (unsigned)(A.nx + 1) >> 1;
     const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;   // below 2^31 + one block
     const unsigned total = (unsigned)A.ny * A.nz * hx;          // at most (N + rows)/2, below 2^31
@@ -101,7 +99,7 @@ __global__ void __launch_bounds__(256) k_metropolis(const __grid_constant__ Metr
     M::polar(w.w[0], cz, st);
     M::sincos2pi(M::u(w.w[1]), &sp, &cp);
     const real ua = M::u(w.w[2]);
-    colour_wait();
+    pdl_wait();
     if (valid) {
         const int P = A.nx * A.ny;
         const bool xl = x > 0, xh = x < A.nx - 1, yl = y > 0, yh = y < A.ny - 1, zl = z > 0, zh = z < A.nz - 1;
@@ -147,20 +145,6 @@ __global__ void __launch_bounds__(256) k_metropolis(const __grid_constant__ Metr
     }
 }
 
-template <typename real, bool HSITE>
-cudaError_t launch_colour(const MetroArgs<real>& A, unsigned blocks, cudaStream_t st) {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(blocks);
-    cfg.blockDim = dim3(256);
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_metropolis<real, HSITE>, A);
-}
-
 // Colour c of sweeps sweep0 .. sweep0+nsweeps-1 (c < 0: both colours, 0 then 1).
 template <typename real>
 cudaError_t sweeps_t(const spin_params* p, void* s, const void* h_site, uint64_t seed, double Rtrial,
@@ -197,7 +181,9 @@ cudaError_t sweeps_t(const spin_params* p, void* s, const void* h_site, uint64_t
         for (int c = 0; c < 2; ++c) {
             if (only_color >= 0 && c != only_color) continue;
             A.color = c;
-            const cudaError_t e = h_site ? launch_colour<real, true>(A, blocks, st) : launch_colour<real, false>(A, blocks, st);
+            const cudaError_t e =
+                h_site ? launch_pdl(k_metropolis<real, true>, dim3(blocks), dim3(256), 0, st, A)
+                       : launch_pdl(k_metropolis<real, false>, dim3(blocks), dim3(256), 0, st, A);
             if (e != cudaSuccess) return e;
         }
     }

@@ -12,12 +12,13 @@
 // double by integer operations (to_f64), the block's sums are formed from
 // shared memory with every lane busy (4 x 512 values by four warps: 80
 // instructions; shuffle trees in every warp took 25 per warp, 400 per block),
-// and 1/N comes from the host.  The two passes at 128^3, cold: FP32 25.5 + 9.7
+// 1/N comes from the host, and both passes are programmatic dependents.  The two passes at 128^3, cold: FP32 25.5 + 9.7
 // -> 16.0 + 7.3 us, FP64 121 -> 77 us for the first.
 #include <cuda_runtime.h>
 
 #include <algorithm>
 
+#include "pdl.cuh"
 #include "spin_device.cuh"
 #include "spin_internal.h"
 
@@ -123,10 +124,6 @@ __device__ __forceinline__ void obs_block(const ObsLane& o, double* __restrict__
     if (t == 0) rec[4] = (double)bad;
 }
 
-// Pass 2 is launched while pass 1 drains and waits for it here.
-__device__ __forceinline__ void obs_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
-__device__ __forceinline__ void obs_go() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
-
 template <typename real, bool HSITE>
 __global__ void __launch_bounds__(kObsThreads, 2)
     k_obs_partial(const real* __restrict__ sx, const real* __restrict__ sy, const real* __restrict__ sz,
@@ -135,7 +132,8 @@ __global__ void __launch_bounds__(kObsThreads, 2)
                   int bc) {
     // one warp per lattice row (y, z); lanes stride along x, so no per-site
     // index division and the row's loads are coalesced
-    obs_go();
+    pdl_wait();
+    pdl_go();
     const long long P = (long long)nx * ny;
     const int rows = ny * nz;
     const int lane = threadIdx.x & 31;
@@ -155,7 +153,7 @@ __global__ void __launch_bounds__(kObsThreads) k_obs_final(const double* __restr
                                                            long long* __restrict__ interval,
                                                            long long* __restrict__ sample_count, int R) {
     __shared__ double tot[5];
-    obs_wait();
+    pdl_wait();
     long long m = 0, count = 0;
     if (ring && threadIdx.x == 0) {
         m = *interval;
@@ -192,28 +190,14 @@ __global__ void __launch_bounds__(kObsThreads) k_obs_final(const double* __restr
     }
 }
 
-// Launch pass 2 as a programmatic dependent of pass 1.
-template <typename Kern, typename... Args>
-cudaError_t launch_final(Kern kernel, int threads, cudaStream_t st, Args... args) {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(1);
-    cfg.blockDim = dim3(threads);
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, args...);
-}
-
 // Batched replicas: the same row-wise reduction, each block on a row range
 // of one replica; the final pass gives one record per replica.
 __global__ void __launch_bounds__(kObsThreads, 2)
     k_obs_batch_partial(const float* __restrict__ sx, const float* __restrict__ sy, const float* __restrict__ sz,
                         const BatchRep* __restrict__ reps, const ObsBlock* __restrict__ blocks, double J, double D,
                         double H0, double H1, double H2, double* __restrict__ partials) {
-    obs_go();
+    pdl_wait();
+    pdl_go();
     const ObsBlock ob = blocks[blockIdx.x];
     const BatchRep rp = reps[ob.rep];
     const int L = rp.L;
@@ -238,7 +222,7 @@ __global__ void __launch_bounds__(kObsFinalThreads) k_obs_batch_final(const doub
                                                                       double* __restrict__ out, double* __restrict__ ring,
                                                                       int ring_len, long long* __restrict__ interval,
                                                                       long long* __restrict__ sample_count, int R) {
-    obs_wait();
+    pdl_wait();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const long long m = ring ? *interval : 0;
     const long long count = ring ? *sample_count : 0;
@@ -280,17 +264,15 @@ cudaError_t launch_observables(const real* s[3], const real* hs[3], Geom g, Phys
                                int nblocks, double* out5, double* sample_ring, int ring, long long* d_interval,
                                long long* d_sample_count, int R, cudaStream_t stream, int bc) {
     const double D = 0.5 * ph.twoD;
-    if (hs[0])
-        k_obs_partial<real, true><<<nblocks, kObsThreads, 0, stream>>>(s[0], s[1], s[2], hs[0], hs[1], hs[2], g.nx, g.ny, g.nz,
-                                                                       (double)ph.J, D, (double)ph.H[0], (double)ph.H[1],
-                                                                       (double)ph.H[2], partials, bc);
-    else
-        k_obs_partial<real, false><<<nblocks, kObsThreads, 0, stream>>>(s[0], s[1], s[2], nullptr, nullptr, nullptr, g.nx, g.ny,
-                                                                        g.nz, (double)ph.J, D, (double)ph.H[0],
-                                                                        (double)ph.H[1], (double)ph.H[2], partials, bc);
-    const cudaError_t e = cudaGetLastError();
+    const dim3 grid(nblocks), block(kObsThreads);
+    const bool in = sizeof(real) == 4 && g.N() <= kPdlGraphSites;
+    const cudaError_t e =
+        hs[0] ? launch_pdl_in(in, k_obs_partial<real, true>, grid, block, 0, stream, s[0], s[1], s[2], hs[0], hs[1], hs[2], g.nx,
+                           g.ny, g.nz, ph.J, D, ph.H[0], ph.H[1], ph.H[2], partials, bc)
+              : launch_pdl_in(in, k_obs_partial<real, false>, grid, block, 0, stream, s[0], s[1], s[2], hs[0], hs[1], hs[2], g.nx,
+                           g.ny, g.nz, ph.J, D, ph.H[0], ph.H[1], ph.H[2], partials, bc);
     if (e != cudaSuccess) return e;
-    return launch_final(k_obs_final, 160, stream, (const double*)partials, nblocks, 1.0 / (double)g.N(), out5,
+    return launch_pdl_in(in, k_obs_final, dim3(1), dim3(160), 0, stream, (const double*)partials, nblocks, 1.0 / (double)g.N(), out5,
                         sample_ring, ring, d_interval, d_sample_count, R);
 }
 
@@ -298,11 +280,10 @@ cudaError_t launch_observables_batch(const float* s[3], const BatchRep* reps, co
                                      const int* first_block, int nrep, Phys<double> ph, double* partials,
                                      double* out, double* ring, int ring_len, long long* d_interval,
                                      long long* d_sample_count, int R, cudaStream_t stream) {
-    k_obs_batch_partial<<<nblocks, kObsThreads, 0, stream>>>(s[0], s[1], s[2], reps, blocks, ph.J, 0.5 * ph.twoD,
-                                                             ph.H[0], ph.H[1], ph.H[2], partials);
-    const cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_pdl(k_obs_batch_partial, dim3(nblocks), dim3(kObsThreads), 0, stream, s[0], s[1], s[2], reps,
+                                     blocks, ph.J, 0.5 * ph.twoD, ph.H[0], ph.H[1], ph.H[2], partials);
     if (e != cudaSuccess) return e;
-    return launch_final(k_obs_batch_final, kObsFinalThreads, stream, (const double*)partials, first_block, reps, nrep, out,
+    return launch_pdl(k_obs_batch_final, dim3(1), dim3(kObsFinalThreads), 0, stream, (const double*)partials, first_block, reps, nrep, out,
                         ring, ring_len, d_interval, d_sample_count, R);
 }
 

@@ -30,6 +30,7 @@
 #include <algorithm>
 
 #include "patch_common.cuh"
+#include "pdl.cuh"
 #include "spin_device.cuh"
 #include "spin_internal.h"
 
@@ -556,6 +557,10 @@ __device__ __forceinline__ void patch_tile(const PatchArgs& a, int bx, int by, i
     }
     const int z0 = bz * a.tz;
     const int t0 = z0 - 2 * S + 2;
+    // the kernel before this one has finished; the next may take the SMs this
+    // one's CTAs leave
+    pdl_wait();
+    pdl_go();
     const long long k = PULSE ? *a.interval : 0;
 
     PRings<S, HSITE> r;

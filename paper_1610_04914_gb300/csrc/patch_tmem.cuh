@@ -265,6 +265,8 @@ __device__ __forceinline__ void tm_tile(const PatchArgs& a, int bx, int by, int 
 
     const int z0 = bz * a.tz;
     const int t0 = z0 - 2 * S + 2;
+    pdl_wait();
+    pdl_go();
     f2 xr[3][4][3], sc[3];
 #pragma unroll
     for (int q = 0; q < 4; ++q)

@@ -37,6 +37,7 @@ struct spin_lattice {
     double* ring;
     long long samples_read;
     cudaGraphExec_t graph[2];  // one noise interval starting from buffer 0 / 1
+    int graph_end[2];          // the buffer it ends in
     cudaStream_t capture_stream;
     // trajectory recording for the adjoint
     bool rec_active;
@@ -187,13 +188,24 @@ cudaError_t observe(spin_lattice* h, int b, bool sample, cudaStream_t st) {
                                       h->p.bc);
 }
 
-// One step n -> n+1 from buffer `from` on stream st (no host bookkeeping).
-cudaError_t launch_one_step(spin_lattice* h, int from, long long n_next, cudaStream_t st) {
-    const bool pulse = h->p.noise && is_pulse_step(n_next, h->p.steps_per_pulse);
+// One step n -> n+1 from buffer *buf on stream st, which becomes the buffer of
+// the new state (no other host bookkeeping).  A step goes from one buffer to
+// the other; with an odd number of steps per interval the pulse of the FP32
+// fused paths, a kernel of its own, goes back, so that an interval ends where
+// it began and the state needs no copy to the caller's arrays (256^3: 60 us).
+cudaError_t launch_one_step(spin_lattice* h, int* buf, long long n_next, cudaStream_t st) {
+    const int R = h->p.steps_per_pulse;
+    const bool pulse = h->p.noise && is_pulse_step(n_next, R);
+    const int from = *buf;
+    int to = from ^ 1;
     cudaError_t e;
     if (h->elt == 4) {
         StepLaunch<float> L = make_launch<float>(h, from, pulse);
         L.stream = st;
+        if (pulse && (R & 1) && !L.force_generic && (h->tab.chain || rk5_fused_supports(L))) {
+            to = from;
+            for (int c = 0; c < 3; ++c) L.pulse_out[c] = static_cast<float*>(h->buf[to][c]);
+        }
         e = launch_step<float>(L);
     } else {
         StepLaunch<double> L = make_launch<double>(h, from, pulse);
@@ -201,7 +213,8 @@ cudaError_t launch_one_step(spin_lattice* h, int from, long long n_next, cudaStr
         e = launch_step<double>(L);
     }
     if (e != cudaSuccess) return e;
-    if (n_next % h->p.steps_per_pulse == 0) e = observe(h, from ^ 1, true, st);
+    *buf = to;
+    if (n_next % R == 0) e = observe(h, to, true, st);
     return e;
 }
 
@@ -216,9 +229,9 @@ int capture_interval(spin_lattice* h, int from) {
     // the graph covers steps mR+1 .. mR+R; pulse and sample positions depend
     // only on n mod R, so step numbers 1..R describe every interval
     for (int q = 1; q <= R && e == cudaSuccess; ++q) {
-        e = launch_one_step(h, b, q, cs);
-        b ^= 1;
+        e = launch_one_step(h, &b, q, cs);
     }
+    h->graph_end[from] = b;
     cudaGraph_t graph = nullptr;
     cudaError_t e2 = cudaStreamEndCapture(cs, &graph);
     if (e != cudaSuccess) {
@@ -401,15 +414,14 @@ int spin_step_pulse(spin_lattice* h, int64_t nsteps) {
                 }
                 SPIN_CUDA(h, cudaGraphLaunch(h->graph[h->cur], h->st));
                 h->n += R;
-                if (R & 1) h->cur ^= 1;
+                h->cur = h->graph_end[h->cur];
                 nsteps -= R;
                 int rc = record_if_due(h);
                 if (rc != SPIN_OK) return rc;
                 continue;
             }
             if (h->n % R == 0 && nsteps >= R) h->eager_intervals++;
-            SPIN_CUDA(h, launch_one_step(h, h->cur, h->n + 1, h->st));
-            h->cur ^= 1;
+            SPIN_CUDA(h, launch_one_step(h, &h->cur, h->n + 1, h->st));
             h->n += 1;
             nsteps -= 1;
             int rc = record_if_due(h);
@@ -423,15 +435,14 @@ int spin_step_pulse(spin_lattice* h, int64_t nsteps) {
             }
             SPIN_CUDA(h, cudaGraphLaunch(h->graph[h->cur], h->st));
             h->n += R;
-            if (R & 1) h->cur ^= 1;
+            h->cur = h->graph_end[h->cur];
             nsteps -= R;
             continue;
         }
         const bool interval_start = h->n % R == 0 && nsteps >= R;
         const int steps = interval_start ? R : 1;
         for (int q = 0; q < steps; ++q) {
-            SPIN_CUDA(h, launch_one_step(h, h->cur, h->n + 1, h->st));
-            h->cur ^= 1;
+            SPIN_CUDA(h, launch_one_step(h, &h->cur, h->n + 1, h->st));
             h->n += 1;
         }
         nsteps -= steps;

@@ -188,38 +188,37 @@ __device__ __forceinline__ void rotation_series(double p, double& sinc, double& 
 // kSmallPhi2 with probability below 1e-6 (chi-squared, three degrees), so the
 // warp does not diverge; for larger sigma every site takes the general form.
 constexpr float kSeriesSigma = 0.35f;
+// Contractions are written out, so that every kernel that rotates rounds alike.
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+template <typename real>
+__device__ __forceinline__ real dot_rn(real ax, real ay, real az, real bx, real by, real bz) {
+    return fma(az, bz, fma(ay, by, mul_rn(ax, bx)));
+}
 template <typename real>
 __device__ __forceinline__ void pulse_rotate(real& sx, real& sy, real& sz, real px, real py, real pz, real sigma) {
-    const real phi2 = px * px + py * py + pz * pz;
+    const real phi2 = dot_rn(px, py, pz, px, py, pz);
+    real nx = px, ny = py, nz = pz, A, C, B;   // s' = s C + (n x s) A + n (n.s) B
     if (sigma <= real(kSeriesSigma) && phi2 <= real(kSmallPhi2)) {
-        real A, B;
         rotation_series(phi2, A, B);
-        const real C = real(1) - phi2 * B;
-        const real ps = (px * sx + py * sy + pz * sz) * B;
-        const real cx = py * sz - pz * sy;
-        const real cy = pz * sx - px * sz;
-        const real cz = px * sy - py * sx;
-        sx = sx * C + cx * A + px * ps;
-        sy = sy * C + cy * A + py * ps;
-        sz = sz * C + cz * A + pz * ps;
-    } else if (phi2 > real(0)) {
+        C = fma(-phi2, B, real(1));
+    } else {
+        if (!(phi2 > real(0))) return;
         const real phi = Math<real>::sqrt_(phi2);
         const real inv = real(1) / phi;
-        const real nx = px * inv, ny = py * inv, nz = pz * inv;
-        real sn, cs;
-        Math<real>::sincos_(phi, &sn, &cs);
-        const real ns = nx * sx + ny * sy + nz * sz;
-        const real om = (real(1) - cs) * ns;
-        const real cx = ny * sz - nz * sy;
-        const real cy = nz * sx - nx * sz;
-        const real cz = nx * sy - ny * sx;
-        const real ox = sx * cs + cx * sn + nx * om;
-        const real oy = sy * cs + cy * sn + ny * om;
-        const real oz = sz * cs + cz * sn + nz * om;
-        sx = ox;
-        sy = oy;
-        sz = oz;
+        nx = mul_rn(px, inv);
+        ny = mul_rn(py, inv);
+        nz = mul_rn(pz, inv);
+        Math<real>::sincos_(phi, &A, &C);
+        B = real(1) - C;
     }
+    const real om = mul_rn(dot_rn(nx, ny, nz, sx, sy, sz), B);
+    const real cx = fma(ny, sz, -mul_rn(nz, sy));
+    const real cy = fma(nz, sx, -mul_rn(nx, sz));
+    const real cz = fma(nx, sy, -mul_rn(ny, sx));
+    sx = fma(nx, om, fma(cx, A, mul_rn(sx, C)));
+    sy = fma(ny, om, fma(cy, A, mul_rn(sy, C)));
+    sz = fma(nz, om, fma(cz, A, mul_rn(sz, C)));
 }
 
 // One pulse on one site: draw G_i for pulse k, rotate by sigma G_i.
@@ -229,7 +228,7 @@ __device__ __forceinline__ void pulse_site(real& sx, real& sy, real& sz, uint64_
     const Words4 w = noise_words(seed, site, k, replica);
     real g0, g1, g2;
     Gauss<real>::draw(w, g0, g1, g2);
-    pulse_rotate<real>(sx, sy, sz, sigma * g0, sigma * g1, sigma * g2, sigma);
+    pulse_rotate<real>(sx, sy, sz, mul_rn(sigma, g0), mul_rn(sigma, g1), mul_rn(sigma, g2), sigma);
 }
 
 // Exact float -> double for FP64 accumulation of FP32 terms, with 32-bit integer

@@ -46,6 +46,7 @@ struct StepLaunch {
     uint64_t replica;
     real sigma;            // pulse angle scale sqrt(2 lambda T Delta t)
     const long long* d_interval;  // device: pulse number of the current interval
+    real* pulse_out[3];    // FP32 fused paths: where the pulse writes the state (null: in place, L.out)
     int* d_status;         // device status word (bit 0: a bounded wait in a kernel gave up) or null
     real* tmp;             // generic path: (stages + 1) * 3N scratch
     cudaStream_t stream;
@@ -69,7 +70,8 @@ cudaError_t prepare_step_kernels();
 // FP32 fused step with register patches (chain tableaus, 2 or 4 stages).
 cudaError_t launch_step_patch(const StepLaunch<float>& L);
 cudaError_t prepare_patch_kernels();
-// The noise rotation of Eq. (s_rotation) over every site of L.out, in place.
+// The noise rotation of Eq. (s_rotation) over every site of L.out, in place or
+// to L.pulse_out.
 cudaError_t launch_pulse_lattice(const StepLaunch<float>& L);
 // FP64 chain tableaus, one kernel per stage; L.tmp holds stage64_scratch(S) N
 // doubles.

@@ -27,30 +27,6 @@ namespace spin {
 
 namespace {
 
-// The adjoint's recomputation runs its steps back to back as programmatic
-// dependents: a store step waits for the kernel before it
-// (griddepcontrol.wait; a no-op without a programmatic dependency) before it
-// touches global memory, and lets the next launch once all of its CTAs are
-// done, so a launch overlaps the drain of its predecessor.  (The plain steps,
-// replayed in whole-interval graphs, measured no gain from it: 0.530 against
-// 0.527 ms per 128^3 interval.)
-__device__ __forceinline__ void dependent_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
-__device__ __forceinline__ void dependents_go() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
-template <typename Kern, typename... Args>
-cudaError_t launch_dependent(Kern kernel, dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, args...);
-}
-
 template <int S, bool PREC, bool HSITE, bool PULSE>
 __global__ void __launch_bounds__(kPT* PatchShape<S>::TY, 1) k_step_patch(PatchArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -63,10 +39,8 @@ __global__ void __launch_bounds__(kPT* PatchShape<S>::TY, 1) k_step_patch(PatchA
 template <int S, bool PREC, bool HSITE>
 __global__ void __launch_bounds__(kPT* PatchShape<S>::TY, 1) k_step_patch_store(PatchArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    dependent_wait();
     patch_tile<S, PREC, HSITE, false, true, 0>(a, (int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z,
                                             reinterpret_cast<float*>(smem_raw));
-    dependents_go();
 }
 
 // RK4 step with the spin planes staged by TMA; the tensor maps live in the
@@ -95,8 +69,7 @@ cudaError_t patch_tmem_launch(const PatchArgs& a, dim3 grid, cudaStream_t st, bo
     const size_t smem = patch_smem<4, PREC, false, false, kTmemVariant>();
     if (prepare)
         return cudaFuncSetAttribute(k_step_patch_tmem<PREC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_step_patch_tmem<PREC><<<grid, dim3(kPT, PatchShape<4, kTmemVariant>::TY), smem, st>>>(a);
-    return cudaGetLastError();
+    return launch_pdl(k_step_patch_tmem<PREC>, grid, dim3(kPT, PatchShape<4, kTmemVariant>::TY), smem, st, a);
 }
 
 // z chunks of a tiling: one resident CTA per SM, so the chunk length that
@@ -132,8 +105,7 @@ cudaError_t patch_launch(const PatchArgs& a, dim3 grid, cudaStream_t st, bool pr
     if (prepare)
         return cudaFuncSetAttribute(k_step_patch<S, PREC, HSITE, PULSE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)smem);
-    k_step_patch<S, PREC, HSITE, PULSE><<<grid, dim3(kPT, PatchShape<S>::TY), smem, st>>>(a);
-    return cudaGetLastError();
+    return launch_pdl(k_step_patch<S, PREC, HSITE, PULSE>, grid, dim3(kPT, PatchShape<S>::TY), smem, st, a);
 }
 
 template <int S, bool PREC, bool HSITE>
@@ -142,7 +114,7 @@ cudaError_t patch_store_launch(const PatchArgs& a, dim3 grid, cudaStream_t st, b
     if (prepare)
         return cudaFuncSetAttribute(k_step_patch_store<S, PREC, HSITE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)smem);
-    return launch_dependent(k_step_patch_store<S, PREC, HSITE>, grid, dim3(kPT, PatchShape<S>::TY), smem, st, a);
+    return launch_pdl(k_step_patch_store<S, PREC, HSITE>, grid, dim3(kPT, PatchShape<S>::TY), smem, st, a);
 }
 
 template <int S, bool PREC, bool HSITE, bool STORE>
@@ -151,8 +123,7 @@ cudaError_t patch_tma_launch(const PatchArgs& a, const TmaMaps* maps, dim3 grid,
     if (prepare)
         return cudaFuncSetAttribute(k_step_patch_tma<S, PREC, HSITE, STORE>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_step_patch_tma<S, PREC, HSITE, STORE><<<grid, dim3(kPT, PatchShape<S>::TY), smem, st>>>(a, *maps);
-    return cudaGetLastError();
+    return launch_pdl(k_step_patch_tma<S, PREC, HSITE, STORE>, grid, dim3(kPT, PatchShape<S>::TY), smem, st, a, *maps);
 }
 
 template <int S>
@@ -213,17 +184,26 @@ cudaError_t patch_dispatch(const PatchArgs& a, dim3 grid, cudaStream_t st, bool 
 // pulse steps of a single lattice the step kernel runs without its epilogue
 // rotation and this kernel rotates the finished state in place.  The
 // arithmetic per site is the fused epilogue's, so the results are identical.
-__global__ void __launch_bounds__(256) k_pulse_f32(float* __restrict__ sx, float* __restrict__ sy, float* __restrict__ sz,
-                                                   unsigned N, uint64_t seed, const long long* __restrict__ interval,
-                                                   uint64_t replica, float sigma) {
-    const uint64_t k = (uint64_t)*interval;
+//
+// The draw does not depend on the state: the kernel is launched while the step
+// before it drains and each thread draws for its first site before it waits.
+// The state may go to other arrays (odd intervals, spin_api.cu).
+__global__ void __launch_bounds__(256) k_pulse_f32(const float* sx, const float* sy, const float* sz, float* ox, float* oy,
+                                                   float* oz, unsigned N, uint64_t seed,
+                                                   const long long* __restrict__ interval, uint64_t replica,
+                                                   float sigma) {
+    const uint64_t k = (uint64_t)*interval;   // written at the last interval's end, before the step before this
     // N < 2^31 and the stride is far below 2^31, so the index cannot wrap
     for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
+        float g0, g1, g2;
+        Gauss<float>::draw(noise_words(seed, (uint64_t)i, k, replica), g0, g1, g2);
+        pdl_wait();   // returns at once after the first time
+        pdl_go();
         float x = sx[i], y = sy[i], z = sz[i];
-        pulse_site<float>(x, y, z, seed, (uint64_t)i, k, replica, sigma);
-        sx[i] = x;
-        sy[i] = y;
-        sz[i] = z;
+        pulse_rotate<float>(x, y, z, mul_rn(sigma, g0), mul_rn(sigma, g1), mul_rn(sigma, g2), sigma);
+        ox[i] = x;
+        oy[i] = y;
+        oz[i] = z;
     }
 }
 
@@ -365,9 +345,9 @@ cudaError_t launch_step_patch(const StepLaunch<float>& L) {
 cudaError_t launch_pulse_lattice(const StepLaunch<float>& L) {
     const long long N = L.g.N();
     const int blocks = (int)std::max<long long>(1, std::min<long long>((N + 255) / 256, 152LL * 32));
-    k_pulse_f32<<<blocks, 256, 0, L.stream>>>(L.out[0], L.out[1], L.out[2], (unsigned)N, L.seed, L.d_interval,
-                                              L.replica, L.sigma);
-    return cudaGetLastError();
+    float* const* o = L.pulse_out[0] ? L.pulse_out : L.out;
+    return launch_pdl_in(N <= kPdlGraphSites, k_pulse_f32, dim3(blocks), dim3(256), 0, L.stream, (const float*)L.out[0], (const float*)L.out[1],
+                      (const float*)L.out[2], o[0], o[1], o[2], (unsigned)N, L.seed, L.d_interval, L.replica, L.sigma);
 }
 
 }  // namespace spin

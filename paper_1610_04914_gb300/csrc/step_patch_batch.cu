@@ -45,8 +45,8 @@ cudaError_t batch_launch(const PatchArgs& a, const BatchItem* items, int nitems,
         return cudaFuncSetAttribute(k_step_patch_batch<S, PREC, PULSE, V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)smem);
     if (nitems <= 0) return cudaSuccess;
-    k_step_patch_batch<S, PREC, PULSE, V><<<nitems, dim3(kPT, PatchShape<S, V>::TY), smem, st>>>(a, items, reps);
-    return cudaGetLastError();
+    return launch_pdl(k_step_patch_batch<S, PREC, PULSE, V>, dim3(nitems), dim3(kPT, PatchShape<S, V>::TY), smem, st, a,
+                      items, reps);
 }
 
 template <int S, int V>
@@ -91,6 +91,8 @@ __global__ void __launch_bounds__(256) k_pulse_batch(float* __restrict__ sx, flo
     const ObsBlock ob = blocks[blockIdx.x];
     const BatchRep rp = reps[ob.rep];
     const uint64_t k = (uint64_t)*interval;
+    pdl_wait();
+    pdl_go();
     const unsigned first = (unsigned)ob.row0 * rp.L;
     const unsigned count = (unsigned)ob.nrows * rp.L;
     for (unsigned q = threadIdx.x; q < count; q += blockDim.x) {
@@ -109,8 +111,7 @@ __global__ void __launch_bounds__(256) k_pulse_batch(float* __restrict__ sx, flo
 
 cudaError_t launch_pulse_batch(float* s[3], const BatchRep* reps, const ObsBlock* blocks, int nblocks, uint64_t seed,
                                const long long* d_interval, cudaStream_t st) {
-    k_pulse_batch<<<nblocks, 256, 0, st>>>(s[0], s[1], s[2], reps, blocks, seed, d_interval);
-    return cudaGetLastError();
+    return launch_pdl(k_pulse_batch, dim3(nblocks), dim3(256), 0, st, s[0], s[1], s[2], reps, blocks, seed, d_interval);
 }
 int patch_out_x(int stages) { return kPC - 2 * stages; }
 int patch_rows(int stages, int variant) {

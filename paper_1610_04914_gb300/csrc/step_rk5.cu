@@ -36,6 +36,7 @@
 #include <algorithm>
 
 #include "patch_common.cuh"
+#include "pdl.cuh"
 #include "spin_device.cuh"
 #include "spin_internal.h"
 
@@ -403,6 +404,8 @@ __global__ void __launch_bounds__(kNT, 1) k_step_rk5(Rk5Args a) {
     }
     const int z0 = (int)blockIdx.z * a.tz;
     const int t0 = z0 - 2 * kH + 2;
+    pdl_wait();
+    pdl_go();
 
     R5Rings r;
 #pragma unroll
@@ -490,8 +493,7 @@ cudaError_t rk5_launch(const Rk5Args& a, dim3 grid, cudaStream_t st, bool prepar
     if (prepare)
         return cudaFuncSetAttribute(k_step_rk5<SEG, PREC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)rk5_smem<SEG>());
-    k_step_rk5<SEG, PREC><<<grid, dim3(kPT, kTY), rk5_smem<SEG>(), st>>>(a);
-    return cudaGetLastError();
+    return launch_pdl(k_step_rk5<SEG, PREC>, grid, dim3(kPT, kTY), rk5_smem<SEG>(), st, a);
 }
 
 // The kernel hard-codes which Butcher coefficients are zero.

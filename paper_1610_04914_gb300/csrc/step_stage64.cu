@@ -23,6 +23,7 @@
 // scratch (6N doubles); for S = 2, X_2 in scratch (3N).
 #include <cuda_runtime.h>
 
+#include "pdl.cuh"
 #include "spin_device.cuh"
 #include "spin_internal.h"
 
@@ -48,14 +49,9 @@ struct Stage64Args {
 
 enum StageRole { kFirst, kMiddle, kLast2, kLast4 };
 
-// Each kernel of the chain is launched while the one before it drains and
-// waits for it here, before its first global access.
-__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
-__device__ __forceinline__ void chain_go() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
-
 template <int ROLE, bool PREC, bool HSITE, bool PULSE>
 __global__ void __launch_bounds__(128) k_stage64(const __grid_constant__ Stage64Args a) {
-    chain_go();
+    pdl_go();
     const unsigned iu = blockIdx.x * blockDim.x + threadIdx.x;   // N < 2^31, the last block may pass it
     if (iu >= (unsigned)a.N) return;
     const int i = (int)iu;
@@ -69,7 +65,7 @@ __global__ void __launch_bounds__(128) k_stage64(const __grid_constant__ Stage64
     const bool fx0 = a.bc && x == 0, fx1 = a.bc && x == a.nx - 1;
     const bool fy0 = a.bc && y == 0, fy1 = a.bc && y == a.ny - 1;
     const bool fz0 = a.bc && z == 0, fz1 = a.bc && z == a.nz - 1;
-    chain_wait();
+    pdl_wait();
     double h[3], v[3], s[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -116,16 +112,8 @@ template <int ROLE, bool PREC, bool HSITE, bool PULSE>
 cudaError_t stage_launch(const Stage64Args& a, cudaStream_t st) {
     // small lattices are spread over the SMs one warp per block
     const int threads = a.N <= 152 * 4 * 32 ? 32 : 128;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)((a.N + threads - 1) / threads));
-    cfg.blockDim = dim3(threads);
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_stage64<ROLE, PREC, HSITE, PULSE>, a);
+    return launch_pdl(k_stage64<ROLE, PREC, HSITE, PULSE>, dim3((unsigned)((a.N + threads - 1) / threads)), dim3(threads),
+                      0, st, a);
 }
 
 template <int ROLE, bool PULSE>

@@ -96,3 +96,28 @@ def test_observables_reduction(gpu, dtype, bc, shape):
     s[0, 0, 0, 0] = float("nan")
     gpu.spin_observables_noalloc(s, J, D, H, out, h_site=h, bc=bc)
     assert out[4].item() == (1 if n == 1 else 2 if (nz // 2, ny // 2, nx - 1) != (0, 0, 0) else 1)
+
+
+# odd intervals: the pulse goes back to the buffer the interval began in; whole
+# intervals (eager, then graphs), single steps and recorded runs end in the same
+# states, samples and checkpoints, bit for bit
+@pytest.mark.parametrize("integ", ["RK4", "RK2_MIDPOINT", "RK5_BUTCHER"])
+@pytest.mark.parametrize("R", [1, 3, 5])
+def test_odd_intervals_bitwise(gpu, integ, R):
+    p = gpu.Params(30, 17, 12, J=0.9, D=0.15, H=(0.05, -0.1, 0.2), lam=0.1, T=0.7, dt=0.07, R=R, seed=7,
+                   integrator=getattr(gpu, integ))
+    s0 = torch.from_numpy(spin_inputs.random_spins(30, 17, 12, seed=3))
+    one, whole, rec = (gpu.Lattice(p, s0) for _ in range(3))
+    n = 4 * R + 2
+    states = [one.state.clone()]
+    for _ in range(n):
+        one.step(1)
+        states.append(one.state.clone())
+    whole.step(n)
+    rec.record(R, n)
+    rec.step(n)
+    assert torch.equal(one.state, whole.state) and torch.equal(one.state, rec.state)
+    assert one.samples() == whole.samples() == rec.samples()
+    slots = rec.store.view(torch.float32)[: (n // R + 1) * one.state.numel()].reshape(n // R + 1, -1)
+    for c in range(n // R + 1):
+        assert torch.equal(slots[c], states[c * R].reshape(-1)), c
