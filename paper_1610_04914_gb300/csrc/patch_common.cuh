@@ -125,17 +125,12 @@ __device__ __forceinline__ int wrapi(int v, int n) {
     return r < 0 ? r + n : r;
 }
 
-// Right-hand side of Eq. (LLL) for a column pair: H = J sum_nn + H_ext
-// (+ 2D s_z z), a = s x H, b = s x a, f = a - lambda b (precessional) or
-// f = -lambda b (the slow equation, precession dropped).
+// Right-hand side of Eq. (LLL) for a pair of spins in the field H = (hx, hy,
+// hz): a = s x H, b = s x a, f = a - lambda b (precessional) or f = -lambda b
+// (the slow equation, precession dropped); nlam = -lambda of each.
 template <bool PREC>
-__device__ __forceinline__ void rhs_pair(const f2 (&sum)[3], const f2 (&cen)[3], float J, float twoD, float Hx,
-                                         float Hy, float Hz, float lambda, f2 (&f)[3]) {
-    const f2 hx = fma2(sp2(J), sum[0], sp2(Hx));
-    const f2 hy = fma2(sp2(J), sum[1], sp2(Hy));
-    f2 hz = fma2(sp2(J), sum[2], sp2(Hz));
+__device__ __forceinline__ void rhs_field_pair(const f2 (&cen)[3], f2 hx, f2 hy, f2 hz, f2 nlam, f2 (&f)[3]) {
     const f2 sx = cen[0], sy = cen[1], sz = cen[2];
-    hz = fma2(sp2(twoD), sz, hz);
     const f2 nx_ = make_float2(-sx.x, -sx.y), ny_ = make_float2(-sy.x, -sy.y), nz_ = make_float2(-sz.x, -sz.y);
     const f2 ax = fma2(nz_, hy, mul2(sy, hz));
     const f2 ay = fma2(nx_, hz, mul2(sz, hx));
@@ -144,14 +139,24 @@ __device__ __forceinline__ void rhs_pair(const f2 (&sum)[3], const f2 (&cen)[3],
     const f2 by = fma2(nx_, az, mul2(sz, ax));
     const f2 bz = fma2(ny_, ax, mul2(sx, ay));
     if (PREC) {
-        f[0] = fma2(sp2(-lambda), bx, ax);
-        f[1] = fma2(sp2(-lambda), by, ay);
-        f[2] = fma2(sp2(-lambda), bz, az);
+        f[0] = fma2(nlam, bx, ax);
+        f[1] = fma2(nlam, by, ay);
+        f[2] = fma2(nlam, bz, az);
     } else {
-        f[0] = mul2(sp2(-lambda), bx);
-        f[1] = mul2(sp2(-lambda), by);
-        f[2] = mul2(sp2(-lambda), bz);
+        f[0] = mul2(nlam, bx);
+        f[1] = mul2(nlam, by);
+        f[2] = mul2(nlam, bz);
     }
+}
+
+// The same for a column pair with H = J sum_nn + H_ext + 2D s_z z.
+template <bool PREC>
+__device__ __forceinline__ void rhs_pair(const f2 (&sum)[3], const f2 (&cen)[3], float J, float twoD, float Hx,
+                                         float Hy, float Hz, float lambda, f2 (&f)[3]) {
+    const f2 hx = fma2(sp2(J), sum[0], sp2(Hx));
+    const f2 hy = fma2(sp2(J), sum[1], sp2(Hy));
+    const f2 hz = fma2(sp2(J), sum[2], sp2(Hz));
+    rhs_field_pair<PREC>(cen, hx, hy, fma2(sp2(twoD), cen[2], hz), sp2(-lambda), f);
 }
 
 }  // namespace

@@ -27,6 +27,7 @@
 #include <vector>
 
 #include "../../include/spinpulse.h"
+#include "patch_common.cuh"
 #include "spin_device.cuh"
 #include "spin_internal.h"
 
@@ -74,7 +75,19 @@ bool tableau_mask_matches(int integ, const Tableau& tb) {
 // One step of integrator INTEG on one spin, then |s| = 1.  RECT:
 // the rectangular-noise field z is added to H_eff in the precession term of
 // every stage (Eqs. (LLL), (zeta_n)); otherwise the noiseless equation.
-template <typename real, bool PREC, int INTEG, bool RECT>
+// The right-hand side in a field along z (AXIAL: H_x = H_y = 0, as in the
+// paper's spin in a field): the terms with a zero factor of Eq. (LLL)'s cross
+// products left out, 10 operations instead of 16.
+template <typename real, bool PREC>
+__device__ __forceinline__ void axial_rhs(real x, real y, real z, real hz, real lam, real& f0, real& f1, real& f2) {
+    const real ax = y * hz, ay = -x * hz;          // a = s x H, a_z = 0
+    const real bx = -z * ay, by = z * ax, bz = x * ay - y * ax;   // b = s x a
+    f0 = (PREC ? ax : real(0)) - lam * bx;
+    f1 = (PREC ? ay : real(0)) - lam * by;
+    f2 = -lam * bz;
+}
+
+template <typename real, bool PREC, int INTEG, bool RECT, bool AXIAL = false>
 __device__ __forceinline__ void single_step(real& s0, real& s1, real& s2, real lam, const SingleCommon<real>& C,
                                             real z0, real z1, real z2) {
     constexpr int ST = integ_stages(INTEG);
@@ -93,6 +106,8 @@ __device__ __forceinline__ void single_step(real& s0, real& s1, real& s2, real l
         real f0, f1, f2;
         if (RECT)
             llg_rhs_noise<real>(x0, x1, x2, C.Hx, C.Hy, C.Hz + C.D2 * x2, z0, z1, z2, lam, f0, f1, f2);
+        else if (AXIAL)
+            axial_rhs<real, PREC>(x0, x1, x2, C.Hz + C.D2 * x2, lam, f0, f1, f2);
         else
             llg_rhs<real, PREC>(x0, x1, x2, C.Hx, C.Hy, C.Hz + C.D2 * x2, lam, f0, f1, f2);
         K[j][0] = C.dt * f0;
@@ -134,7 +149,13 @@ struct RunArgs {
     int stop;
 };
 
-template <typename real, bool PREC, int INTEG, bool RECT>
+// Steps from phase ph = n mod R to the next event of the schedule: the pulse at
+// phase half, or the interval's end.
+__device__ __forceinline__ int steps_to_event(int ph, int half, int R, bool pulses) {
+    return pulses && ph < half ? half - ph : R - ph;
+}
+
+template <typename real, bool PREC, int INTEG, bool RECT, bool AXIAL>
 __global__ void __launch_bounds__(128) k_single_run(RunArgs<real> A) {
     const SingleCommon<real>& C = A.c;
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
@@ -150,27 +171,56 @@ __global__ void __launch_bounds__(128) k_single_run(RunArgs<real> A) {
     int ph = (int)(A.n0 % C.R);
     long long kq = A.n0 / C.R;
     const int half = C.R / 2;
-    real z0 = 0, z1 = 0, z2 = 0;
-    if (RECT && ph != 0) draw_zeta<real>(C, (uint64_t)kq, (uint64_t)r, sig, z0, z1, z2);  // mid-interval start
-    for (long long n = A.n0 + 1; n <= A.n0 + A.nsteps; ++n) {
-        if (RECT && ph == 0) draw_zeta<real>(C, (uint64_t)kq, (uint64_t)r, sig, z0, z1, z2);  // interval (n-1) div R
-        single_step<real, PREC, INTEG, RECT>(s0, s1, s2, lam, C, z0, z1, z2);
-        if (++ph == C.R) {
-            ph = 0;
-            ++kq;
+    const bool pulses = !RECT && C.noise;
+    long long n = A.n0;
+    const long long end = A.n0 + A.nsteps;
+    bool crossed = false;
+    if (RECT) {
+        real z0 = 0, z1 = 0, z2 = 0;
+        if (ph != 0) draw_zeta<real>(C, (uint64_t)kq, (uint64_t)r, sig, z0, z1, z2);  // mid-interval start
+        while (n < end && !crossed) {
+            if (ph == 0) draw_zeta<real>(C, (uint64_t)kq, (uint64_t)r, sig, z0, z1, z2);  // interval n div R
+            single_step<real, PREC, INTEG, RECT>(s0, s1, s2, lam, C, z0, z1, z2);
+            ++n;
+            if (++ph == C.R) {
+                ph = 0;
+                ++kq;
+                if (A.sz_sum) {
+                    acc += to_f64(s2);
+                    ++cnt;
+                }
+            }
+            crossed = A.stop && s2 < real(0);
         }
-        // pulse number (n - 1) div R: kq, or kq - 1 when n is a multiple of R
-        if (!RECT && C.noise && ph == half)
-            pulse_site<real>(s0, s1, s2, C.seed, 0ULL, (uint64_t)(ph == 0 ? kq - 1 : kq), (uint64_t)r, sig);
-        if (A.sz_sum && ph == 0) {
-            acc += (double)s2;
-            ++cnt;
-        }
-        if (A.stop && s2 < real(0)) {
-            fp = n;
-            break;
+    } else {
+        while (n < end && !crossed) {
+            const int m = (int)min((long long)steps_to_event(ph, half, C.R, pulses), end - n);
+            int q = 0;
+            do {
+                single_step<real, PREC, INTEG, RECT, AXIAL>(s0, s1, s2, lam, C, real(0), real(0), real(0));
+                ++q;
+                crossed = A.stop && s2 < real(0);
+            } while (q < m && !crossed);
+            n += q;
+            ph += q;
+            if (q == m) {
+                if (ph == C.R) {
+                    ph = 0;
+                    ++kq;
+                }
+                // pulse number (n - 1) div R: kq, or kq - 1 when n is a multiple of R
+                if (pulses && ph == half) {
+                    pulse_site<real>(s0, s1, s2, C.seed, 0ULL, (uint64_t)(ph == 0 ? kq - 1 : kq), (uint64_t)r, sig);
+                    crossed = A.stop && s2 < real(0);   // the step ends with its pulse
+                }
+                if (A.sz_sum && ph == 0) {
+                    acc += to_f64(s2);
+                    ++cnt;
+                }
+            }
         }
     }
+    if (crossed) fp = n;
     C.sx[r] = s0;
     C.sy[r] = s1;
     C.sz[r] = s2;
@@ -178,6 +228,116 @@ __global__ void __launch_bounds__(128) k_single_run(RunArgs<real> A) {
     if (A.sz_sum) {
         A.sz_sum[r] += acc;
         A.sz_count[r] += cnt;
+    }
+}
+
+// Two replicas per thread, their components paired in packed f32x2 operands:
+// FP32 runs without a first-passage stop.  The run kernel is bound by
+// instruction issue; a packed instruction does both replicas' arithmetic in one
+// issue slot.  The step's dt is folded into the tableau (ca = dt a, cb = dt b).
+// Worth it once the halved thread count still gives every scheduler a few
+// warps (pair_min).
+constexpr int kPairThreads = 64;
+struct PairArgs {
+    SingleCommon<float> c;
+    float ca[6][6], cb[6];
+    double* sz_sum;
+    long long* sz_count;
+    long long n0, nsteps;
+};
+
+template <bool PREC, int INTEG, bool AXIAL>
+__device__ __forceinline__ void pair_step(f2 (&s)[3], f2 nlam, const PairArgs& A) {
+    constexpr int ST = integ_stages(INTEG);
+    f2 f[ST][3];
+#pragma unroll
+    for (int j = 0; j < ST; ++j) {
+        f2 x[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            x[c] = s[c];
+#pragma unroll
+            for (int l = 0; l < j; ++l)
+                if (a_nonzero(INTEG, j, l)) x[c] = fma2(sp2(A.ca[j][l]), f[l][c], x[c]);
+        }
+        const f2 hz = fma2(sp2(A.c.D2), x[2], sp2(A.c.Hz));
+        if (AXIAL) {
+            const f2 ax = mul2(x[1], hz), nay = mul2(x[0], hz);   // a = s x H: a_x, -a_y
+            const f2 nx = make_float2(-x[0].x, -x[0].y), ny = make_float2(-x[1].x, -x[1].y);
+            const f2 bx = mul2(x[2], nay), by = mul2(x[2], ax), bz = fma2(nx, nay, mul2(ny, ax));   // b = s x a
+            const f2 ay = make_float2(-nay.x, -nay.y);
+            f[j][0] = PREC ? fma2(nlam, bx, ax) : mul2(nlam, bx);
+            f[j][1] = PREC ? fma2(nlam, by, ay) : mul2(nlam, by);
+            f[j][2] = mul2(nlam, bz);
+        } else {
+            rhs_field_pair<PREC>(x, sp2(A.c.Hx), sp2(A.c.Hy), hz, nlam, f[j]);
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+        for (int j = 0; j < ST; ++j)
+            if (b_nonzero(INTEG, j)) s[c] = fma2(sp2(A.cb[j]), f[j][c], s[c]);
+    if (A.c.renorm) {
+        const f2 n2 = fma2(s[0], s[0], fma2(s[1], s[1], mul2(s[2], s[2])));
+        const f2 inv = make_float2(rsqrtf(n2.x), rsqrtf(n2.y));
+#pragma unroll
+        for (int c = 0; c < 3; ++c) s[c] = mul2(s[c], inv);
+    }
+}
+
+template <bool PREC, int INTEG, bool AXIAL>
+__global__ void __launch_bounds__(kPairThreads) k_single_run_pair(const __grid_constant__ PairArgs A) {
+    const SingleCommon<float>& C = A.c;
+    const int pairs = (C.nrep + 1) >> 1;
+    const int r0 = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r0 >= pairs) return;
+    const bool two = r0 + pairs < C.nrep;            // the last thread of an odd count has one replica
+    const int r1 = two ? r0 + pairs : r0;
+    f2 s[3] = {make_float2(C.sx[r0], C.sx[r1]), make_float2(C.sy[r0], C.sy[r1]), make_float2(C.sz[r0], C.sz[r1])};
+    const float sg0 = C.sigma[r0], sg1 = C.sigma[r1];
+    const f2 nlam = make_float2(-C.lambda[r0], -C.lambda[r1]);
+    double acc0 = 0.0, acc1 = 0.0;
+    long long cnt = 0;
+    int ph = (int)(A.n0 % C.R);   // n mod R and n div R of the step n just completed
+    long long kq = A.n0 / C.R;
+    const int half = C.R / 2;
+    long long left = A.nsteps;
+    while (left > 0) {
+        const int m = (int)min((long long)steps_to_event(ph, half, C.R, C.noise != 0), left);
+        for (int q = 0; q < m; ++q) pair_step<PREC, INTEG, AXIAL>(s, nlam, A);
+        left -= m;
+        ph += m;
+        if (ph == C.R) {
+            ph = 0;
+            ++kq;
+        }
+        if (C.noise && ph == half) {
+            const uint64_t k = (uint64_t)(ph == 0 ? kq - 1 : kq);
+            pulse_site<float>(s[0].x, s[1].x, s[2].x, C.seed, 0ULL, k, (uint64_t)r0, sg0);
+            pulse_site<float>(s[0].y, s[1].y, s[2].y, C.seed, 0ULL, k, (uint64_t)r1, sg1);
+        }
+        if (A.sz_sum && ph == 0) {
+            acc0 += to_f64(s[2].x);
+            acc1 += to_f64(s[2].y);
+            ++cnt;
+        }
+    }
+    C.sx[r0] = s[0].x;
+    C.sy[r0] = s[1].x;
+    C.sz[r0] = s[2].x;
+    if (two) {
+        C.sx[r1] = s[0].y;
+        C.sy[r1] = s[1].y;
+        C.sz[r1] = s[2].y;
+    }
+    if (A.sz_sum) {
+        A.sz_sum[r0] += acc0;
+        A.sz_count[r0] += cnt;
+        if (two) {
+            A.sz_sum[r1] += acc1;
+            A.sz_count[r1] += cnt;
+        }
     }
 }
 
@@ -286,7 +446,10 @@ SingleCommon<real> make_common(const spin_params* p, int nrep, void* s, void* sc
 template <typename real, bool PREC, int INTEG, bool RECT>
 struct RunK {
     static void launch(int blocks, cudaStream_t st, const RunArgs<real>& A) {
-        k_single_run<real, PREC, INTEG, RECT><<<blocks, 128, 0, st>>>(A);
+        if (!RECT && A.c.Hx == real(0) && A.c.Hy == real(0))
+            k_single_run<real, PREC, INTEG, RECT, !RECT><<<blocks, 128, 0, st>>>(A);
+        else
+            k_single_run<real, PREC, INTEG, RECT, false><<<blocks, 128, 0, st>>>(A);
     }
 };
 template <typename real, bool PREC, int INTEG, bool RECT>
@@ -370,6 +533,49 @@ cudaError_t run_t(const spin_params* p, int nrep, void* s, void* scratch, long l
     return dispatch<real, RunK>(p, nrep, A, st);
 }
 
+// Replicas from which two share a thread: 3 to 4 packed warps per scheduler.
+// RK5, R = 40, 400 steps, pair / scalar kernel: 49152 replicas 187 / 164 us,
+// 65536 186 / 208, 131072 336 / 342, 389120 780 / 919; Heun with a pulse every
+// other step: 65536 231 / 211, 98304 286 / 296, 389120 784 / 876 (the draws
+// are not packed, so two-stage steps gain later).  Field with an x component.
+int pair_min(int integrator) { return integ_stages(integrator) >= 4 ? 65536 : 98304; }
+
+template <int INTEG>
+cudaError_t pair_launch(const PairArgs& A, bool prec, cudaStream_t st) {
+    const int blocks = ((A.c.nrep + 1) / 2 + kPairThreads - 1) / kPairThreads;
+    const bool axial = A.c.Hx == 0.f && A.c.Hy == 0.f;
+    if (prec)
+        axial ? k_single_run_pair<true, INTEG, true><<<blocks, kPairThreads, 0, st>>>(A)
+              : k_single_run_pair<true, INTEG, false><<<blocks, kPairThreads, 0, st>>>(A);
+    else
+        axial ? k_single_run_pair<false, INTEG, true><<<blocks, kPairThreads, 0, st>>>(A)
+              : k_single_run_pair<false, INTEG, false><<<blocks, kPairThreads, 0, st>>>(A);
+    return cudaGetLastError();
+}
+
+cudaError_t run_pairs(const spin_params* p, int nrep, void* s, void* scratch, long long n0, long long nsteps,
+                      double* sz_sum, long long* sz_count, cudaStream_t st) {
+    const Tableau tb = tableau_for(p->integrator);
+    if (!tableau_mask_matches(p->integrator, tb)) return cudaErrorInvalidValue;
+    PairArgs A{};
+    A.c = make_common<float>(p, nrep, s, scratch);
+    for (int j = 0; j < 6; ++j) {
+        A.cb[j] = (float)(tb.b[j] * p->dt);
+        for (int l = 0; l < 6; ++l) A.ca[j][l] = (float)(tb.a[j][l] * p->dt);
+    }
+    A.sz_sum = sz_sum;
+    A.sz_count = sz_count;
+    A.n0 = n0;
+    A.nsteps = nsteps;
+    switch (p->integrator) {
+        case 0: return pair_launch<0>(A, p->precession != 0, st);
+        case 1: return pair_launch<1>(A, p->precession != 0, st);
+        case 2: return pair_launch<2>(A, p->precession != 0, st);
+        case 3: return pair_launch<3>(A, p->precession != 0, st);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
 template <typename real>
 cudaError_t escape_t(const spin_params* p, int nrep, const double* s_init, void* s, void* scratch, long long n0,
                      long long nsteps, long long* trial, long long* local_step, long long* fpt_sum, double* fpt_sq,
@@ -423,6 +629,8 @@ extern "C" int spin_single_run(const spin_params* p, int32_t nrep, void* s, void
         p->precision == 64
             ? run_t<double>(p, nrep, s, scratch, n0, nsteps, stop_on_crossing, (long long*)first_passage, sz_sum,
                             (long long*)sz_count, st)
+        : !stop_on_crossing && p->noise != 2 && nrep >= pair_min(p->integrator)
+            ? run_pairs(p, nrep, s, scratch, n0, nsteps, sz_sum, (long long*)sz_count, st)
             : run_t<float>(p, nrep, s, scratch, n0, nsteps, stop_on_crossing, (long long*)first_passage, sz_sum,
                            (long long*)sz_count, st);
     return e == cudaSuccess ? SPIN_OK : SPIN_ECUDA;

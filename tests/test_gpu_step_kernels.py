@@ -121,3 +121,29 @@ def test_odd_intervals_bitwise(gpu, integ, R):
     slots = rec.store.view(torch.float32)[: (n // R + 1) * one.state.numel()].reshape(n // R + 1, -1)
     for c in range(n // R + 1):
         assert torch.equal(slots[c], states[c * R].reshape(-1)), c
+
+
+# the pair kernel (from 65536 replicas; an odd count leaves one replica alone),
+# the axial right-hand side (H along z, with anisotropy) and calls that end
+# mid-interval, against the oracle on sampled replicas (tolerances of
+# test_gpu_single.py)
+@pytest.mark.parametrize("integ,precession", [(0, 1), (1, 1), (1, 0), (3, 1)])
+@pytest.mark.parametrize("H", [(0.0, 0.0, 0.9), (0.3, -0.2, 0.4)])
+@pytest.mark.parametrize("nrep", [131, 98305])
+def test_single_pairs(gpu, orc, integ, precession, H, nrep):
+    p = gpu.Params(1, 1, 1, J=0.0, D=0.4, H=H, lam=0.2, T=0.0, dt=0.1, R=6, integrator=integ, precession=precession,
+                   seed=21, precision=32)
+    T = np.linspace(0.05, 1.0, nrep)
+    v = np.random.default_rng(4).normal(size=(3, nrep))
+    s0 = (v / np.linalg.norm(v, axis=0)).astype(np.float32)
+    ss = gpu.SingleSpins(p, T, torch.from_numpy(s0))
+    ss.run(16, average=True).run(20, average=True)
+    torch.cuda.synchronize()
+    got, sums = ss.state.double().cpu().numpy(), ss.sz_sum.cpu().numpy()
+    assert (ss.sz_count.cpu().numpy() == 6).all()
+    for r in (0, 1, 64, nrep // 2 - 1, nrep // 2, nrep // 2 + 1, nrep - 1):
+        q = orc.Params(1, 1, 1, J=0.0, D=0.4, H=H, lam=0.2, T=float(T[r]), dt=0.1, R=6, integrator=integ,
+                       precession=precession, seed=21, replica=r)
+        ref, smp = orc.run(q, s0[:, r].astype(np.float64).reshape(3, 1, 1, 1), 36)
+        assert np.max(np.abs(got[:, r] - ref.reshape(3))) < 2e-5
+        assert abs(sums[r] - smp[:, 3].sum()) < 6 * 2e-5
