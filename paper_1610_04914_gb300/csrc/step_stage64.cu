@@ -15,9 +15,8 @@
 // The accumulator of the tableau is not kept: with K_j = dt f(X_j) and
 // X_{j+1} = s + a_{j+1,j} K_j, every K_j but the last is (X_{j+1} - s)/a_{j+1,j},
 // so the last stage forms
-//   y = g_0 s + sum_{j=2..S} g_j X_j + b_S K_S,  g_j = b_{j-1}/a_{j,j-1},
-//   g_0 = 1 - sum_j g_j
-// from the stage inputs (own site only), then renormalises and, on pulse
+//   y = s + sum_{j=2..S} g_j (X_j - s) + b_S K_S,  g_j = b_{j-1}/a_{j,j-1},
+// from the stage inputs (own site only; RK4: (X_2 + 2 X_3 + X_4 - s)/3 + K_4/6), then renormalises and, on pulse
 // steps, rotates.  For S = 4, X_2 lives in the step's output array (the last
 // stage reads it at its own site before it writes there), X_3 and X_4 in
 // scratch (6N doubles); for S = 2, X_2 in scratch (3N).
@@ -40,16 +39,78 @@ struct Stage64Args {
     int nx, ny, nz, N;
     double J, twoD, H[3], lambda;
     double c;              // dt a_{j+1,j}; last stage: dt b_S
-    double g0, gx, gq[2];  // last stage: weights of s, X_S, X_2, X_3
+    double g0, gx;         // last stage of S = 2: weights of s and X_2
     int bc, renorm;
     uint64_t seed, replica;
     double sigma;
     const long long* interval;
 };
 
+// Fixed-point sums of doubles without the FP64 pipe: the mantissas, shifted to
+// the largest exponent of the terms, add exactly as 64-bit integers and the sum
+// is rounded once to nearest.  A term loses only what lies 2^-60 below the
+// largest, so a sum is at least as exact as the additions in a row would be;
+// those are 5 of a component's 12 FP64 instructions per stage, and the integer
+// pipes are idle.  Magnitudes below 2^-923 count as zero; where a term is above
+// 2^977, infinite or NaN (emax > kMaxExp) the caller takes the plain sum.
+constexpr unsigned kMinExp = 100u, kMaxExp = 2000u;
+__device__ __forceinline__ unsigned exponent(double v) { return ((unsigned)__double2hiint(v) >> 20) & 0x7FFu; }
+// v in units of 2^(emax - 1082): 53 bits at bits 7 .. 59, shifted right
+__device__ __forceinline__ long long fixed(double v, unsigned emax) {
+    const unsigned h = (unsigned)__double2hiint(v);
+    const unsigned long long m = (((unsigned long long)((h & 0xFFFFFu) | 0x100000u) << 32) |
+                                  (unsigned)__double2loint(v)) << 7;
+    const long long x = (long long)(m >> min(emax - ((h >> 20) & 0x7FFu), 63u));
+    const long long sg = (long long)((int)h >> 31);
+    return (x ^ sg) - sg;
+}
+__device__ __forceinline__ double from_fixed(long long S, unsigned emax) {
+    const long long sg = S >> 63;
+    const unsigned long long a = (unsigned long long)((S ^ sg) - sg);
+    const int lz = __clzll((long long)a);
+    const unsigned long long n = a << lz;      // leading bit at 63
+    unsigned long long r = n >> 11;
+    const unsigned rem = (unsigned)n & 0x7FFu;
+    r += (rem > 0x400u || (rem == 0x400u && (r & 1ULL))) ? 1ULL : 0ULL;
+    // leading bit of a at bit 63 - lz: biased exponent emax + 4 - lz, of which
+    // the mantissa's leading bit adds one
+    r += (unsigned long long)(emax + 3u - (unsigned)lz) << 52;
+    r |= (unsigned long long)sg & 0x8000000000000000ULL;
+    return a == 0ULL ? 0.0 : __longlong_as_double((long long)r);
+}
+// Kept out of line: inlined, the compiler would execute it for every site.
+__device__ __noinline__ double plain_sum6(double a, double b, double c, double d, double e, double f) {
+    return ((a + b) + (c + d)) + (e + f);
+}
+__device__ __forceinline__ double sum6(const double (&q)[6]) {
+    unsigned emax = kMinExp;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) emax = max(emax, exponent(q[k]));
+    if (emax > kMaxExp) return plain_sum6(q[0], q[1], q[2], q[3], q[4], q[5]);
+    long long S = 0;   // six terms below 2^60 each
+#pragma unroll
+    for (int k = 0; k < 6; ++k) S += fixed(q[k], emax);
+    return from_fixed(S, emax);
+}
+// x2 + 2 x3 + x4 - s: the part of the RK4 result that its stage inputs hold,
+// times three
+__device__ __noinline__ double plain_rk4_sum(double x2, double x3, double x4, double s) {
+    return (x2 + 2.0 * x3) + (x4 - s);
+}
+__device__ __forceinline__ double rk4_sum(double x2, double x3, double x4, double s) {
+    const unsigned emax = max(max(exponent(x2), exponent(x3)), max(max(exponent(x4), exponent(s)), kMinExp));
+    if (emax > kMaxExp) return plain_rk4_sum(x2, x3, x4, s);
+    return from_fixed(fixed(x2, emax) + 2 * fixed(x3, emax) + fixed(x4, emax) - fixed(s, emax), emax);
+}
+
 enum StageRole { kFirst, kMiddle, kLast2, kLast4 };
 
-template <int ROLE, bool PREC, bool HSITE, bool PULSE>
+// WIDE: sums through the integer pipes, for lattices that fill the FP64 pipe
+// (the smallest ones wait on latencies instead, of which the integer form has
+// more: 16^3 242 against 250 us for 10 steps).  UNITX: J = 1 and the uniform
+// field along z without site fields, so that H_x and H_y are the bare neighbour
+// sums (the products and sums with 1 and 0 would be two more instructions).
+template <int ROLE, bool PREC, bool HSITE, bool PULSE, bool WIDE, bool UNITX>
 __global__ void __launch_bounds__(128) k_stage64(const __grid_constant__ Stage64Args a) {
     pdl_go();
     const unsigned iu = blockIdx.x * blockDim.x + threadIdx.x;   // N < 2^31, the last block may pass it
@@ -71,11 +132,11 @@ __global__ void __launch_bounds__(128) k_stage64(const __grid_constant__ Stage64
     for (int c = 0; c < 3; ++c) {
         const double* q = a.x[c];
         v[c] = q[i];
-        const double l = fx0 ? 0.0 : q[xm], r = fx1 ? 0.0 : q[xp];
-        const double u = fy0 ? 0.0 : q[ym], d = fy1 ? 0.0 : q[yp];
-        const double b = fz0 ? 0.0 : q[zm], t = fz1 ? 0.0 : q[zp];
+        const double nb[6] = {fx0 ? 0.0 : q[xm], fx1 ? 0.0 : q[xp], fy0 ? 0.0 : q[ym],
+                              fy1 ? 0.0 : q[yp], fz0 ? 0.0 : q[zm], fz1 ? 0.0 : q[zp]};
         s[c] = ROLE == kFirst ? v[c] : a.s[c][i];
-        h[c] = a.J * (((l + r) + (u + d)) + (b + t)) + a.H[c];
+        const double sum = WIDE ? sum6(nb) : ((nb[0] + nb[1]) + (nb[2] + nb[3])) + (nb[4] + nb[5]);
+        h[c] = UNITX && c < 2 ? sum : a.J * sum + a.H[c];
         if (HSITE) h[c] += a.hs[c][i];
     }
     h[2] += a.twoD * v[2];
@@ -88,12 +149,13 @@ __global__ void __launch_bounds__(128) k_stage64(const __grid_constant__ Stage64
     } else {
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            double acc = a.g0 * s[c];
+            double acc;
             if (ROLE == kLast4) {
-                acc += a.gq[0] * a.q[0][c][i];
-                acc += a.gq[1] * a.q[1][c][i];
+                const double x2 = a.q[0][c][i], x3 = a.q[1][c][i];
+                acc = (1.0 / 3.0) * (WIDE ? rk4_sum(x2, x3, v[c], s[c]) : (x2 + 2.0 * x3) + (v[c] - s[c]));
+            } else {
+                acc = a.g0 * s[c] + a.gx * v[c];
             }
-            acc += a.gx * v[c];
             o[c] = acc + a.c * f[c];
         }
         if (a.renorm) {
@@ -110,16 +172,29 @@ __global__ void __launch_bounds__(128) k_stage64(const __grid_constant__ Stage64
 
 template <int ROLE, bool PREC, bool HSITE, bool PULSE>
 cudaError_t stage_launch(const Stage64Args& a, cudaStream_t st) {
-    // small lattices are spread over the SMs one warp per block
-    const int threads = a.N <= 152 * 4 * 32 ? 32 : 128;
-    return launch_pdl(k_stage64<ROLE, PREC, HSITE, PULSE>, dim3((unsigned)((a.N + threads - 1) / threads)), dim3(threads),
-                      0, st, a);
+    // up to one warp per scheduler: one warp per block, spread over the SMs
+    const bool wide = a.N > 152 * 4 * 32;
+    const dim3 block(wide ? 128 : 32), grid((unsigned)(((unsigned)a.N + block.x - 1) / block.x));
+    const bool unitx = !HSITE && a.J == 1.0 && a.H[0] == 0.0 && a.H[1] == 0.0;
+    if (wide)
+        return unitx ? launch_pdl(k_stage64<ROLE, PREC, HSITE, PULSE, true, !HSITE>, grid, block, 0, st, a)
+                     : launch_pdl(k_stage64<ROLE, PREC, HSITE, PULSE, true, false>, grid, block, 0, st, a);
+    return unitx ? launch_pdl(k_stage64<ROLE, PREC, HSITE, PULSE, false, !HSITE>, grid, block, 0, st, a)
+                 : launch_pdl(k_stage64<ROLE, PREC, HSITE, PULSE, false, false>, grid, block, 0, st, a);
 }
 
 template <int ROLE, bool PULSE>
 cudaError_t stage_dispatch(const Stage64Args& a, cudaStream_t st, bool prec, bool hs) {
     if (prec) return hs ? stage_launch<ROLE, true, true, PULSE>(a, st) : stage_launch<ROLE, true, false, PULSE>(a, st);
     return hs ? stage_launch<ROLE, false, true, PULSE>(a, st) : stage_launch<ROLE, false, false, PULSE>(a, st);
+}
+
+// The four-stage tableau whose result the last stage forms with fixed weights.
+bool rk4_weights(const Tableau& tb) {
+    const double third[3] = {tb.b[0] / tb.a[1][0], tb.b[1] / tb.a[2][1] / 2.0, tb.b[2] / tb.a[3][2]};
+    for (double g : third)
+        if (!(g > 1.0 / 3.0 - 1e-15 && g < 1.0 / 3.0 + 1e-15)) return false;
+    return true;
 }
 
 }  // namespace
@@ -151,12 +226,7 @@ cudaError_t launch_step_stage64(const StepLaunch<double>& L) {
         a.s[c] = L.in[c];
     }
     const bool prec = L.precession != 0, hs = L.hs[0] != nullptr;
-    // weights of the stage inputs X_2 .. X_S in the result
-    double g[5] = {}, g0 = 1.0;
-    for (int j = 2; j <= S; ++j) {
-        g[j] = tb.b[j - 2] / tb.a[j - 1][j - 2];
-        g0 -= g[j];
-    }
+    if (S == 4 && !rk4_weights(tb)) return cudaErrorInvalidValue;
     // stage 1 .. S-1 write X_2 .. X_S, of S = 4 the first into the output array
     auto scratch = [&](int q, int c) { return L.tmp + ((size_t)q * 3 + c) * N; };
     const double* prev[3] = {L.in[0], L.in[1], L.in[2]};
@@ -172,11 +242,9 @@ cudaError_t launch_step_stage64(const StepLaunch<double>& L) {
                        : stage_dispatch<kMiddle, false>(a, L.stream, prec, hs);
         } else {
             a.c = tb.b[S - 1] * L.dt;
-            a.g0 = g0;
-            a.gx = g[S];
+            a.gx = tb.b[0] / tb.a[1][0];
+            a.g0 = 1.0 - a.gx;
             if (S == 4) {
-                a.gq[0] = g[2];
-                a.gq[1] = g[3];
                 for (int c = 0; c < 3; ++c) {
                     a.q[0][c] = L.out[c];
                     a.q[1][c] = scratch(0, c);
