@@ -5,6 +5,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "noise_tables.cuh"
+
 namespace spin {
 
 // Key word 1 of the noise stream ("noise" in ASCII).
@@ -52,6 +54,23 @@ __device__ __forceinline__ Words4 noise_words(uint64_t seed, uint64_t site, uint
     return philox4x64_10(site, k, replica, 0ULL, seed, kStreamNoise);
 }
 
+// Exact float -> double for FP64 accumulation of FP32 terms, with 32-bit integer
+// operations only: the hardware conversion uses this GPU's FP64 pipe, which
+// runs at ~1/64 of the FP32 rate and is needed for the FP64 additions
+// themselves.  The exponent is rebased from 127 to 1023; subnormals are first
+// scaled by 2^24; zeros, infinities and NaNs keep their sign and payload.
+// (Every case is selected, none branched to: a conversion instruction in a
+// rare branch would be executed always, with its result discarded.)
+__device__ __forceinline__ double to_f64(float f) {
+    const unsigned b = __float_as_uint(f);
+    const bool sub = (b & 0x7F800000u) == 0u;
+    const unsigned m = sub ? __float_as_uint(f * 16777216.0f) : b;
+    const unsigned e = (m >> 23) & 0xFFu;
+    const unsigned x = e == 0u ? 0u : e == 0xFFu ? 2047u : e + (sub ? 872u : 896u);
+    return __hiloint2double((int)((b & 0x80000000u) | (x << 20) | ((m & 0x7FFFFFu) >> 3)), (int)(m << 29));
+}
+__device__ __forceinline__ double to_f64(double d) { return d; }
+
 // Box-Muller.  Uniforms are u = ((w >> 11) + 1/2) 2^-53 in (0, 1); G0, G1 from
 // (u0, u1) and G2 from (u2, u3).
 template <typename real>
@@ -71,14 +90,68 @@ struct Gauss<double> {
         // value m 2^-54: exponent 63 - lz - 54, mantissa below the leading bit
         return __longlong_as_double((long long)(((uint64_t)(1023 + 9 - lz) << 52) + ((m << lz) << 1 >> 12)));
     }
+    // -2 ln u for u in (0, 1), table-driven (P. T. P. Tang, ACM TOMS 16, 1990):
+    // u = 2^e m, m in [sqrt(1/2), sqrt(2)), ln m = -ln c + ln(1 + r) with c from
+    // the table, r = m c - 1, |r| <= 2^-8, and the series of ln(1 + r) to r^7.
+    // Ten FP64 instructions (log: about 35; the pulse of an FP64 128^3 lattice
+    // 657 -> 414 us with root and angle below).  Near u = 1, c = 1 and e = 0: no
+    // cancellation.
+    __device__ __forceinline__ static double neg2log(double u) {
+        const int h = __double2hiint(u);
+        const int e = (h - 0x3FE6A09E) >> 20;
+        const int mh = h - (e << 20);
+        const double m = __hiloint2double(mh, __double2loint(u));
+        const double2 t = __ldg(&kLogTable[((mh - 0x3FE00000 + (1 << 12)) >> 13) - kLogFirst]);
+        const double r = fma(m, t.x, -1.0);
+        double q = fma(1.0 / 7.0, r, -1.0 / 6.0);
+        q = fma(q, r, 1.0 / 5.0);
+        q = fma(q, r, -1.0 / 4.0);
+        q = fma(q, r, 1.0 / 3.0);
+        q = fma(q, r, -1.0 / 2.0);
+        const double l = fma(r * r, q, r);
+        return fma(-2.0, l, fma(to_f64((float)e), -1.3862943611198906188, t.y));   // -2 ln 2
+    }
+    // sqrt of a normal x: the FP32 reciprocal root of x with its mantissa cut to
+    // 24 bits, then one third-order step; five FP64 instructions, error below one
+    // unit in the last place.
+    __device__ __forceinline__ static double root(double x) {
+        const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x);
+        const float xf = __uint_as_float(((h - 0x38000000u) << 3) | (l >> 29));
+        const double g = to_f64(rsqrtf(xf));
+        const double t = x * g;
+        const double d = fma(-t, g, 1.0);
+        return fma(t * d, fma(0.375, d, 0.5), t);
+    }
+    // cos and sin of 2 pi u, u = (2k+1) 2^-54 the uniform of word w: the nearest
+    // multiple of 2 pi/64 from the table, the rest (|phi| <= pi/64) by series.
+    __device__ __forceinline__ static void angle(uint64_t w, double& c, double& s) {
+        const uint64_t m = (w >> 10) | 1ULL;
+        const unsigned k = (unsigned)((m + (1ULL << 47)) >> 48);
+        const long long d = (long long)(m - ((uint64_t)k << 48));   // |d| <= 2^47
+        const double2 t = __ldg(&kTrigTable[k & 63u]);
+        // d as a double: added to the bits of 1.5 2^52, which is then subtracted
+        const double x = __longlong_as_double(0x4338000000000000LL + d) - 6755399441055744.0;
+        const double phi = x * 3.4878684980086318e-16;               // 2 pi 2^-54
+        const double z = phi * phi;
+        double p = fma(-1.0 / 5040.0, z, 1.0 / 120.0);
+        p = fma(p, z, -1.0 / 6.0);
+        const double sn = fma(phi * z, p, phi);
+        double q = fma(1.0 / 40320.0, z, -1.0 / 720.0);
+        q = fma(q, z, 1.0 / 24.0);
+        q = fma(q, z, -0.5);
+        const double cm = z * q;                                     // cos(phi) - 1
+        c = fma(t.x, cm, fma(-t.y, sn, t.x));
+        s = fma(t.y, cm, fma(t.x, sn, t.y));
+    }
     __device__ __forceinline__ static void draw(const Words4& w, double& g0, double& g1, double& g2) {
-        const double r0 = sqrt(-2.0 * log(u01(w.w[0])));
-        const double r2 = sqrt(-2.0 * log(u01(w.w[2])));
-        double s1, c1;
-        sincospi(2.0 * u01(w.w[1]), &s1, &c1);
+        const double r0 = root(neg2log(u01(w.w[0])));
+        const double r2 = root(neg2log(u01(w.w[2])));
+        double s1, c1, s3, c3;
+        angle(w.w[1], c1, s1);
+        angle(w.w[3], c3, s3);
         g0 = r0 * c1;
         g1 = r0 * s1;
-        g2 = r2 * cospi(2.0 * u01(w.w[3]));
+        g2 = r2 * c3;
     }
 };
 
@@ -230,23 +303,6 @@ __device__ __forceinline__ void pulse_site(real& sx, real& sy, real& sz, uint64_
     Gauss<real>::draw(w, g0, g1, g2);
     pulse_rotate<real>(sx, sy, sz, mul_rn(sigma, g0), mul_rn(sigma, g1), mul_rn(sigma, g2), sigma);
 }
-
-// Exact float -> double for FP64 accumulation of FP32 terms, with 32-bit integer
-// operations only: the hardware conversion uses this GPU's FP64 pipe, which
-// runs at ~1/64 of the FP32 rate and is needed for the FP64 additions
-// themselves.  The exponent is rebased from 127 to 1023; subnormals are first
-// scaled by 2^24; zeros, infinities and NaNs keep their sign and payload.
-// (Every case is selected, none branched to: a conversion instruction in a
-// rare branch would be executed always, with its result discarded.)
-__device__ __forceinline__ double to_f64(float f) {
-    const unsigned b = __float_as_uint(f);
-    const bool sub = (b & 0x7F800000u) == 0u;
-    const unsigned m = sub ? __float_as_uint(f * 16777216.0f) : b;
-    const unsigned e = (m >> 23) & 0xFFu;
-    const unsigned x = e == 0u ? 0u : e == 0xFFu ? 2047u : e + (sub ? 872u : 896u);
-    return __hiloint2double((int)((b & 0x80000000u) | (x << 20) | ((m & 0x7FFFFFu) >> 3)), (int)(m << 29));
-}
-__device__ __forceinline__ double to_f64(double d) { return d; }
 
 // isfinite without the FP64 pipe (its comparison would run there)
 __device__ __forceinline__ bool finite_bits(float f) { return (__float_as_uint(f) & 0x7F800000u) != 0x7F800000u; }

@@ -10,7 +10,9 @@
 // 8 x 8 outputs, four times the FP64 work.  Here every stage of every site is
 // computed exactly once, and the stage inputs X_j go through memory.  RK4,
 // one interval: 128^3 (4 steps, one pulse) 16.08 -> 3.60 ms, 16^3 (10 steps,
-// one pulse, observables) 2.09 -> 0.25 ms.
+// one pulse, observables) 2.09 -> 0.25 ms; with the sums below off the FP64
+// pipe and the cheaper noise draw 1.97 and 0.23 ms.  The pipe is then 85%
+// active.
 //
 // The accumulator of the tableau is not kept: with K_j = dt f(X_j) and
 // X_{j+1} = s + a_{j+1,j} K_j, every K_j but the last is (X_{j+1} - s)/a_{j+1,j},

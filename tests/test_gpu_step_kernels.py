@@ -147,3 +147,42 @@ def test_single_pairs(gpu, orc, integ, precession, H, nrep):
         ref, smp = orc.run(q, s0[:, r].astype(np.float64).reshape(3, 1, 1, 1), 36)
         assert np.max(np.abs(got[:, r] - ref.reshape(3))) < 2e-5
         assert abs(sums[r] - smp[:, 3].sum()) < 6 * 2e-5
+
+
+def test_noise_fp64_draw(gpu):
+    """2^20 FP64 draws (every interval of the logarithm's and the angles'
+    tables, uniforms down to 2^-20 and up to 1 - 2^-20) against numpy from the
+    same words; 2e-14 as in the parity test: a few roundings of r <= 8.7 here and
+    in numpy's argument 2 pi u."""
+    words, g = gpu.spin_noise_draw(11, 5, 2, 1 << 20, precision=64)
+    torch.cuda.synchronize()
+    w = words.cpu().numpy().view(np.uint64)
+    u = ((w >> np.uint64(11)).astype(np.float64) + 0.5) * 2.0 ** -53
+    r0, r2 = np.sqrt(-2 * np.log(u[:, 0])), np.sqrt(-2 * np.log(u[:, 2]))
+    a, b = 2 * np.pi * u[:, 1], 2 * np.pi * u[:, 3]
+    ref = np.stack([r0 * np.cos(a), r0 * np.sin(a), r2 * np.cos(b)], 1)
+    assert np.max(np.abs(g.cpu().numpy() - ref)) < 2e-14
+
+
+# the fixed-point sums of the FP64 stages (beyond 19456 sites): mixed magnitudes
+# (components from 1 down to 2^-70), exact zeros, and a non-finite spin, which
+# has to reach its neighbours and nobody else
+def test_fp64_stage_sums(gpu, orc):
+    n = (28, 27, 26)
+    g = np.random.default_rng(8)
+    s0 = spin_inputs.random_spins(*n, seed=3)
+    s0[0] *= 2.0 ** -g.integers(0, 70, s0[0].shape)
+    s0[1, :9] = 0.0
+    s0[:, 20:] = np.array([0.0, 0.0, 1.0]).reshape(3, 1, 1, 1)
+    for J, H in ((1.0, (0.0, 0.0, 0.2)), (0.9, (0.05, -0.1, 0.2))):
+        p = gpu.Params(*n, J=J, D=0.15, H=H, lam=0.1, T=0.7, dt=0.07, R=3, seed=77, precision=64)
+        got, lat = run_gpu(gpu, p, s0, 3)
+        ref, _ = run_oracle(orc, p, s0, 3)
+        assert np.max(np.abs(got - ref)) < 1e-13
+    bad = torch.from_numpy(s0.copy())
+    bad[0, 13, 13, 13] = float("inf")
+    p.noise, p.integrator = 0, gpu.RK2_MIDPOINT
+    lat = gpu.Lattice(p, bad).step(1)
+    z, y, x = torch.where(~torch.isfinite(lat.state).all(0))
+    d = (z - 13).abs() + (y - 13).abs() + (x - 13).abs()
+    assert int(d.max()) == 2 and len(d) == 25   # two stages: the octahedron of radius 2
