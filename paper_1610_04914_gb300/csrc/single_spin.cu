@@ -231,6 +231,55 @@ __global__ void __launch_bounds__(128) k_single_run(RunArgs<real> A) {
     }
 }
 
+// Rectangular noise with LANES lanes per replica, for runs without a
+// first-passage stop of so few replicas that latency bounds them: a draw is a
+// longer chain of dependent operations than a step.  Each lane of a group draws
+// the field of another one of the next LANES intervals, then all of them take
+// the steps of those intervals alike, the field coming from its lane.
+template <typename real, int INTEG, int LANES>
+__global__ void __launch_bounds__(128) k_single_rect(RunArgs<real> A) {
+    const SingleCommon<real>& C = A.c;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const int sub = t & (LANES - 1);
+    const bool mine = t / LANES < C.nrep;
+    const int r = min(t / LANES, C.nrep - 1);   // idle lanes of the last warp follow the last replica
+    real s0 = C.sx[r], s1 = C.sy[r], s2 = C.sz[r];
+    const real sig = C.sigma[r], lam = C.lambda[r];
+    double acc = 0.0;
+    long long cnt = 0;
+    int ph = (int)(A.n0 % C.R);   // n mod R and n div R of the step n just completed
+    long long kq = A.n0 / C.R;
+    long long left = A.nsteps;
+    while (left > 0) {
+        real z0, z1, z2;
+        draw_zeta<real>(C, (uint64_t)(kq + sub), (uint64_t)r, sig, z0, z1, z2);
+#pragma unroll 1
+        for (int q = 0; q < LANES && left > 0; ++q) {
+            const real y0 = __shfl_sync(0xffffffffu, z0, q, LANES);
+            const real y1 = __shfl_sync(0xffffffffu, z1, q, LANES);
+            const real y2 = __shfl_sync(0xffffffffu, z2, q, LANES);
+            const int m = (int)min((long long)(C.R - ph), left);
+            for (int p = 0; p < m; ++p) single_step<real, true, INTEG, true>(s0, s1, s2, lam, C, y0, y1, y2);
+            left -= m;
+            ph += m;
+            if (ph == C.R) {
+                ph = 0;
+                ++kq;
+                acc += to_f64(s2);
+                ++cnt;
+            }
+        }
+    }
+    if (!mine || sub != 0) return;
+    C.sx[r] = s0;
+    C.sy[r] = s1;
+    C.sz[r] = s2;
+    if (A.sz_sum) {
+        A.sz_sum[r] += acc;
+        A.sz_count[r] += cnt;
+    }
+}
+
 // Two replicas per thread, their components paired in packed f32x2 operands:
 // FP32 runs without a first-passage stop.  The run kernel is bound by
 // instruction issue; a packed instruction does both replicas' arithmetic in one
@@ -519,6 +568,33 @@ cudaError_t upload_scales(const spin_params* p, int nrep, const double* T, const
     return e;
 }
 
+// Lanes per replica of a rectangular-noise run: while the launch leaves most
+// schedulers with a warp or less.  Heun, R = 1, 200 steps with 1 / 2 / 4 / 8
+// lanes: 1000 replicas 154 / 117 / 82 / 69 us, 8192 157 / 119 / 99 / 116, 16384
+// 156 / 142 / 145 / 184; RK5, R = 4: 1000 80 / 71 / 64 / 62, 8192 82 / 72 / 87 /
+// 142, 16384 82 / 94 / 149 / 228.
+int rect_lanes(int nrep) { return nrep <= 2048 ? 8 : nrep <= 6144 ? 4 : nrep <= 12288 ? 2 : 1; }
+
+template <typename real, int INTEG>
+cudaError_t rect_launch(int nrep, int lanes, const RunArgs<real>& A, cudaStream_t st) {
+    const unsigned blocks = (unsigned)(((long long)nrep * lanes + 127) / 128);
+    if (lanes == 2) k_single_rect<real, INTEG, 2><<<blocks, 128, 0, st>>>(A);
+    else if (lanes == 4) k_single_rect<real, INTEG, 4><<<blocks, 128, 0, st>>>(A);
+    else k_single_rect<real, INTEG, 8><<<blocks, 128, 0, st>>>(A);
+    return cudaGetLastError();
+}
+template <typename real>
+cudaError_t rect_dispatch(const spin_params* p, int nrep, int lanes, const RunArgs<real>& A, cudaStream_t st) {
+    if (!tableau_mask_matches(p->integrator, tableau_for(p->integrator))) return cudaErrorInvalidValue;
+    switch (p->integrator) {
+        case 0: return rect_launch<real, 0>(nrep, lanes, A, st);
+        case 1: return rect_launch<real, 1>(nrep, lanes, A, st);
+        case 2: return rect_launch<real, 2>(nrep, lanes, A, st);
+        case 3: return rect_launch<real, 3>(nrep, lanes, A, st);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
 template <typename real>
 cudaError_t run_t(const spin_params* p, int nrep, void* s, void* scratch, long long n0, long long nsteps, int stop,
                   long long* fp, double* sz_sum, long long* sz_count, cudaStream_t st) {
@@ -530,6 +606,10 @@ cudaError_t run_t(const spin_params* p, int nrep, void* s, void* scratch, long l
     A.n0 = n0;
     A.nsteps = nsteps;
     A.stop = stop;
+    if (p->noise == 2 && !stop) {
+        const int lanes = rect_lanes(nrep);
+        if (lanes > 1) return rect_dispatch<real>(p, nrep, lanes, A, st);
+    }
     return dispatch<real, RunK>(p, nrep, A, st);
 }
 

@@ -186,3 +186,29 @@ def test_fp64_stage_sums(gpu, orc):
     z, y, x = torch.where(~torch.isfinite(lat.state).all(0))
     d = (z - 13).abs() + (y - 13).abs() + (x - 13).abs()
     assert int(d.max()) == 2 and len(d) == 25   # two stages: the octahedron of radius 2
+
+
+# rectangular noise with 8, 4, 2 and 1 lanes per replica (the last warp partly
+# idle), calls that end mid-interval, against the oracle on sampled replicas
+@pytest.mark.parametrize("prec,tol", [(64, 1e-12), (32, 2e-5)])
+@pytest.mark.parametrize("nrep", [3, 2049, 6145, 12289])
+@pytest.mark.parametrize("integ,R", [(3, 1), (1, 4)])
+def test_single_rect_lanes(gpu, orc, prec, tol, nrep, integ, R):
+    p = gpu.Params(1, 1, 1, J=0.0, D=0.4, H=(0.3, -0.2, 0.4), lam=0.2, T=0.0, dt=0.1, R=R, integrator=integ, noise=2,
+                   seed=21, precision=prec)
+    T = np.linspace(0.05, 1.0, nrep)
+    v = np.random.default_rng(4).normal(size=(3, nrep))
+    s0 = v / np.linalg.norm(v, axis=0)
+    if prec == 32:
+        s0 = s0.astype(np.float32).astype(np.float64)
+    ss = gpu.SingleSpins(p, T, torch.from_numpy(s0))
+    ss.run(10, average=True).run(11, average=True)
+    torch.cuda.synchronize()
+    got, sums = ss.state.double().cpu().numpy(), ss.sz_sum.cpu().numpy()
+    assert (ss.sz_count.cpu().numpy() == 21 // R).all()
+    for r in (0, 1, nrep // 2, nrep - 1):
+        q = orc.Params(1, 1, 1, J=0.0, D=0.4, H=(0.3, -0.2, 0.4), lam=0.2, T=float(T[r]), dt=0.1, R=R, integrator=integ,
+                       seed=21, replica=r)
+        ref, smp = orc.run(q, s0[:, r].reshape(3, 1, 1, 1), 21, noise=2)
+        assert np.max(np.abs(got[:, r] - ref.reshape(3))) < tol
+        assert abs(sums[r] - smp[:, 3].sum()) < 21 * tol
