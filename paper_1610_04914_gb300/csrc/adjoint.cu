@@ -59,7 +59,7 @@ constexpr int kAW = kAT / 32;
 // their successor launch once all of their blocks have stored their results.
 template <typename Kern, typename... Args>
 cudaError_t adj_launch(Kern kernel, dim3 grid, cudaStream_t st, const Args&... args) {
-    return launch_pdl(kernel, grid, dim3(kAT), 0, st, args...);
+    return launch_pdl(true, kernel, grid, dim3(kAT), 0, st, args...);
 }
 
 // A site of the lattice with its six neighbours (x-1, x+1, y-1, y+1, z-1, z+1;

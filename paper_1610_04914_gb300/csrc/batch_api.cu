@@ -243,7 +243,8 @@ cudaError_t batch_observe(spin_batch* b, int buf, bool sample, cudaStream_t st) 
     const float* s[3] = {(const float*)b->buf[buf][0], (const float*)b->buf[buf][1], (const float*)b->buf[buf][2]};
     return launch_observables_batch(s, b->reps, b->oblocks, b->nblocks_obs, b->first_block, b->nrep, bphys(b),
                                     b->partials, b->out, sample ? b->ring : nullptr, SPIN_BATCH_SAMPLE_RING,
-                                    b->d_interval, b->d_sample_count, b->p.steps_per_pulse, st);
+                                    b->d_interval, b->d_sample_count, b->p.steps_per_pulse, st,
+                                    b->capture_stream && st == b->capture_stream);
 }
 
 // One launch per tile variant in use, each over its slice of the item table.
@@ -266,7 +267,8 @@ cudaError_t batch_one_step(spin_batch* b, int from, long long n_next, cudaStream
     if (e != cudaSuccess) return e;
     if (pulse) {
         float* s[3] = {(float*)b->buf[from ^ 1][0], (float*)b->buf[from ^ 1][1], (float*)b->buf[from ^ 1][2]};
-        e = launch_pulse_batch(s, b->reps, b->oblocks, b->nblocks_obs, b->p.seed, b->d_interval, st);
+        e = launch_pulse_batch(s, b->reps, b->oblocks, b->nblocks_obs, b->p.seed, b->d_interval, st,
+                               b->capture_stream && st == b->capture_stream);
         if (e != cudaSuccess) return e;
     }
     if (n_next % R == 0) e = batch_observe(b, from ^ 1, true, st);

@@ -182,8 +182,8 @@ cudaError_t sweeps_t(const spin_params* p, void* s, const void* h_site, uint64_t
             if (only_color >= 0 && c != only_color) continue;
             A.color = c;
             const cudaError_t e =
-                h_site ? launch_pdl(k_metropolis<real, true>, dim3(blocks), dim3(256), 0, st, A)
-                       : launch_pdl(k_metropolis<real, false>, dim3(blocks), dim3(256), 0, st, A);
+                h_site ? launch_pdl(true, k_metropolis<real, true>, dim3(blocks), dim3(256), 0, st, A)
+                       : launch_pdl(true, k_metropolis<real, false>, dim3(blocks), dim3(256), 0, st, A);
             if (e != cudaSuccess) return e;
         }
     }

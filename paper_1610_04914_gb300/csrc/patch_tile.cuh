@@ -93,6 +93,7 @@ struct PatchArgs {
     uint64_t seed, replica;
     float sigma;
     const long long* interval;
+    int pdl;           // host: launch as a programmatic dependent
     int bc;            // 1: free boundaries (outside columns and planes read as zero spins)
     int pair8;         // 1: each thread's column pair is one aligned 8-byte word of every input plane
     int pair8out;      // 1: the same for the output planes
@@ -676,6 +677,7 @@ inline PatchArgs patch_args_common(const StepLaunch<float>& L) {
     a.sigma = L.sigma;
     a.interval = L.d_interval;
     a.bc = L.bc;
+    a.pdl = L.graph ? 0 : 1;
     a.err = L.d_status;
     return a;
 }

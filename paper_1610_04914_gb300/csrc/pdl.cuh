@@ -6,14 +6,14 @@
 // that calls pdl_go after its own pdl_wait also promises its successor that
 // everything before it has finished.
 //
-// In a captured graph the kernels get ordinary edges unless the caller asks
-// otherwise.  Programmatic edges between graph nodes gained nothing or cost
-// time (an interval of 96 replicas 2048 -> 2133 us, RK5 at 128^3 1108 -> 1148,
+// In interval graphs the kernels get ordinary edges, with one exception.
+// Programmatic edges between graph nodes gained nothing or cost time (an interval of 96 replicas 2048 -> 2133 us, RK5 at 128^3 1108 -> 1148,
 // 10 FP64 steps at 16^3 243 -> 244, 2 FP64 Heun steps at 41x11x101 59 -> 66)
 // but for the pulse and the observables of FP32 lattices up to about 2^20
 // sites (64^3 particle, 20 RK2 steps 500 -> 477; 45x37x27 RK4 260 -> 250;
 // 128^3 513 -> 514).  On a stream every kernel gains: the first, uncaptured
-// interval at 128^3 575 -> 535 us.
+// interval at 128^3 575 -> 535 us; batched steps keep ordinary launches, whose
+// tiling is tuned on them.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -24,14 +24,9 @@ __device__ __forceinline__ void pdl_go() { asm volatile("griddepcontrol.launch_d
 
 constexpr long long kPdlGraphSites = 1LL << 20;
 
+// pdl = false: an ordinary launch.
 template <typename Kern, typename... Args>
-cudaError_t launch_pdl_in(bool in_graph, Kern kernel, dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                          const Args&... args) {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (!in_graph) {
-        const cudaError_t e = cudaStreamIsCapturing(st, &cap);
-        if (e != cudaSuccess) return e;
-    }
+cudaError_t launch_pdl(bool pdl, Kern kernel, dim3 grid, dim3 block, size_t smem, cudaStream_t st, const Args&... args) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
     cfg.blockDim = block;
@@ -41,12 +36,8 @@ cudaError_t launch_pdl_in(bool in_graph, Kern kernel, dim3 grid, dim3 block, siz
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = cap == cudaStreamCaptureStatusNone ? 1 : 0;
+    cfg.numAttrs = pdl ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
-}
-template <typename Kern, typename... Args>
-cudaError_t launch_pdl(Kern kernel, dim3 grid, dim3 block, size_t smem, cudaStream_t st, const Args&... args) {
-    return launch_pdl_in(false, kernel, grid, block, smem, st, args...);
 }
 
 }  // namespace spin

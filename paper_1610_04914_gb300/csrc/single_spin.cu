@@ -573,7 +573,7 @@ cudaError_t upload_scales(const spin_params* p, int nrep, const double* T, const
 // lanes: 1000 replicas 154 / 117 / 82 / 69 us, 8192 157 / 119 / 99 / 116, 16384
 // 156 / 142 / 145 / 184; RK5, R = 4: 1000 80 / 71 / 64 / 62, 8192 82 / 72 / 87 /
 // 142, 16384 82 / 94 / 149 / 228.
-int rect_lanes(int nrep) { return nrep <= 2048 ? 8 : nrep <= 6144 ? 4 : nrep <= 12288 ? 2 : 1; }
+int rect_lanes(int nrep) { return nrep <= 2048 ? 8 : nrep <= 6144 ? 4 : nrep <= 10240 ? 2 : 1; }
 
 template <typename real, int INTEG>
 cudaError_t rect_launch(int nrep, int lanes, const RunArgs<real>& A, cudaStream_t st) {

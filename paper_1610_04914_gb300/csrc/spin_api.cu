@@ -95,6 +95,12 @@ Layout layout_for(const spin_params* p) {
     L.tmp = off;
     if (generic) off += align_up(elt * (size_t)(tb.stages + 1) * 3 * (size_t)g.N());
     else if (elt == 8) off += align_up(elt * (size_t)stage64_scratch(tb.stages) * (size_t)g.N());
+    // stage inputs of the small-lattice FP32 stage kernels, with site fields or
+    // without
+    if (elt == 4 && stage32_small(g, tb.stages == 4 ? 4 : 2, true, false)) {
+        if (!generic) L.tmp = off;
+        off += align_up(elt * (size_t)stage32_scratch(tb.stages) * (size_t)g.N());
+    }
     L.partials = off;
     off += align_up(sizeof(double) * 5 * (size_t)observables_blocks(g));
     L.out_sample = off;
@@ -170,6 +176,9 @@ Phys<double> phys64(const spin_lattice* h) {
     return ph;
 }
 
+// Work on the handle's capture stream goes into an interval graph.
+bool captured(const spin_lattice* h, cudaStream_t st) { return h->capture_stream && st == h->capture_stream; }
+
 // Launch observables of buffer b; sample=true records into the ring.
 cudaError_t observe(spin_lattice* h, int b, bool sample, cudaStream_t st) {
     if (h->elt == 4) {
@@ -178,14 +187,14 @@ cudaError_t observe(spin_lattice* h, int b, bool sample, cudaStream_t st) {
         return launch_observables<float>(s, hs, h->g, phys64(h), h->partials, h->nblocks_obs,
                                          sample ? h->out_sample : h->out_obs, sample ? h->ring : nullptr,
                                          SPIN_SAMPLE_RING, h->d_interval, h->d_sample_count, h->p.steps_per_pulse, st,
-                                         h->p.bc);
+                                         h->p.bc, captured(h, st));
     }
     const double* s[3] = {(const double*)h->buf[b][0], (const double*)h->buf[b][1], (const double*)h->buf[b][2]};
     const double* hs[3] = {(const double*)h->hs[0], (const double*)h->hs[1], (const double*)h->hs[2]};
     return launch_observables<double>(s, hs, h->g, phys64(h), h->partials, h->nblocks_obs,
                                       sample ? h->out_sample : h->out_obs, sample ? h->ring : nullptr,
                                       SPIN_SAMPLE_RING, h->d_interval, h->d_sample_count, h->p.steps_per_pulse, st,
-                                      h->p.bc);
+                                      h->p.bc, captured(h, st));
 }
 
 // One step n -> n+1 from buffer *buf on stream st, which becomes the buffer of
@@ -202,6 +211,7 @@ cudaError_t launch_one_step(spin_lattice* h, int* buf, long long n_next, cudaStr
     if (h->elt == 4) {
         StepLaunch<float> L = make_launch<float>(h, from, pulse);
         L.stream = st;
+        L.graph = captured(h, st);
         if (pulse && (R & 1) && !L.force_generic && (h->tab.chain || rk5_fused_supports(L))) {
             to = from;
             for (int c = 0; c < 3; ++c) L.pulse_out[c] = static_cast<float*>(h->buf[to][c]);
@@ -210,6 +220,7 @@ cudaError_t launch_one_step(spin_lattice* h, int* buf, long long n_next, cudaStr
     } else {
         StepLaunch<double> L = make_launch<double>(h, from, pulse);
         L.stream = st;
+        L.graph = captured(h, st);
         e = launch_step<double>(L);
     }
     if (e != cudaSuccess) return e;

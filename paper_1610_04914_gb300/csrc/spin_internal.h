@@ -52,6 +52,7 @@ struct StepLaunch {
     cudaStream_t stream;
     int force_generic;
     int bc;                // 0 periodic, 1 free boundaries
+    int graph;             // 1: captured into an interval graph (kernels get ordinary edges)
     // FP32 fused path only: if st_n[0][0] is set, the step also writes, at
     // every site, the stage inputs X_j (j = 2..S, st_x[j-2]), the neighbour
     // sums sum_nn X_j of every stage (j = 1..S, st_n[j-1]) and the
@@ -73,6 +74,11 @@ cudaError_t prepare_patch_kernels();
 // The noise rotation of Eq. (s_rotation) over every site of L.out, in place or
 // to L.pulse_out.
 cudaError_t launch_pulse_lattice(const StepLaunch<float>& L);
+// FP32 chain tableaus on small lattices, one kernel per stage (bitwise the fused
+// step); L.tmp holds stage32_scratch(S) N floats unless the stages are stored.
+bool stage32_small(const Geom& g, int stages, bool field, bool store);
+int stage32_scratch(int stages);
+cudaError_t launch_step_stage32(const StepLaunch<float>& L);
 // FP64 chain tableaus, one kernel per stage; L.tmp holds stage64_scratch(S) N
 // doubles.
 cudaError_t launch_step_stage64(const StepLaunch<double>& L);
@@ -112,11 +118,11 @@ struct ObsBlock {
 };
 // Pulse rotation of every site of every replica (block table as above).
 cudaError_t launch_pulse_batch(float* s[3], const BatchRep* reps, const ObsBlock* blocks, int nblocks, uint64_t seed,
-                               const long long* d_interval, cudaStream_t st);
+                               const long long* d_interval, cudaStream_t st, bool graph);
 cudaError_t launch_observables_batch(const float* s[3], const BatchRep* reps, const ObsBlock* blocks, int nblocks,
                                      const int* first_block, int nrep, Phys<double> ph, double* partials,
                                      double* out, double* ring, int ring_len, long long* d_interval,
-                                     long long* d_sample_count, int R, cudaStream_t stream);
+                                     long long* d_sample_count, int R, cudaStream_t stream, bool graph);
 
 // FP64 observables: per-block partials, then a one-block deterministic sum.
 // out5 = (M_x, M_y, M_z, E, nonfinite count); if sample_ring != null the
@@ -126,7 +132,7 @@ template <typename real>
 cudaError_t launch_observables(const real* s[3], const real* hs[3], Geom g, Phys<double> ph,
                                double* partials, int nblocks, double* out5, double* sample_ring,
                                int ring, long long* d_interval, long long* d_sample_count, int R,
-                               cudaStream_t stream, int bc = 0);
+                               cudaStream_t stream, int bc, bool graph);
 int observables_blocks(Geom g);
 
 cudaError_t launch_noise_draw(uint64_t seed, long long k, long long replica, long long n, int precision,

@@ -2,7 +2,8 @@
 // Eq. (LLL), on the simple-cubic lattice, followed by renormalisation and, on
 // pulse steps, the noise rotation of Eq. (s_rotation).  The paths:
 //  * chain tableaus (RK4, RK2 midpoint, Heun: stage j needs only K_{j-1}) in
-//    FP32: one fused kernel per step, all stages on chip (patch_tile.cuh);
+//    FP32: one fused kernel per step, all stages on chip (patch_tile.cuh); on
+//    small lattices one kernel per stage (step_stage32.cu);
 //  * chain tableaus in FP64: one kernel per stage (step_stage64.cu);
 //  * Butcher RK5 in FP32 without a per-site field: two fused three-stage
 //    segments (step_rk5.cu);
@@ -257,7 +258,12 @@ static cudaError_t launch_generic(const StepLaunch<real>& L) {
 template <typename real>
 cudaError_t launch_step(const StepLaunch<real>& L) {
     if (L.tab->chain && !L.force_generic && (L.tab->stages == 4 || L.tab->stages == 2)) {
-        if (sizeof(real) == 4) return launch_step_patch(reinterpret_cast<const StepLaunch<float>&>(L));
+        if (sizeof(real) == 4) {
+            const StepLaunch<float>& F = reinterpret_cast<const StepLaunch<float>&>(L);
+            if (!stage32_small(L.g, L.tab->stages, F.hs[0] != nullptr, F.st_n[0][0] != nullptr)) return launch_step_patch(F);
+            const cudaError_t e = launch_step_stage32(F);
+            return e != cudaSuccess || !L.pulse ? e : launch_pulse_lattice(F);
+        }
         return launch_step_stage64(reinterpret_cast<const StepLaunch<double>&>(L));
     }
     if (sizeof(real) == 4 && !L.force_generic && rk5_fused_supports(reinterpret_cast<const StepLaunch<float>&>(L)))

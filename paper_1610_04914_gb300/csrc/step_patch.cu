@@ -69,7 +69,7 @@ cudaError_t patch_tmem_launch(const PatchArgs& a, dim3 grid, cudaStream_t st, bo
     const size_t smem = patch_smem<4, PREC, false, false, kTmemVariant>();
     if (prepare)
         return cudaFuncSetAttribute(k_step_patch_tmem<PREC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    return launch_pdl(k_step_patch_tmem<PREC>, grid, dim3(kPT, PatchShape<4, kTmemVariant>::TY), smem, st, a);
+    return launch_pdl(a.pdl != 0, k_step_patch_tmem<PREC>, grid, dim3(kPT, PatchShape<4, kTmemVariant>::TY), smem, st, a);
 }
 
 // z chunks of a tiling: one resident CTA per SM, so the chunk length that
@@ -105,7 +105,7 @@ cudaError_t patch_launch(const PatchArgs& a, dim3 grid, cudaStream_t st, bool pr
     if (prepare)
         return cudaFuncSetAttribute(k_step_patch<S, PREC, HSITE, PULSE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)smem);
-    return launch_pdl(k_step_patch<S, PREC, HSITE, PULSE>, grid, dim3(kPT, PatchShape<S>::TY), smem, st, a);
+    return launch_pdl(a.pdl != 0, k_step_patch<S, PREC, HSITE, PULSE>, grid, dim3(kPT, PatchShape<S>::TY), smem, st, a);
 }
 
 template <int S, bool PREC, bool HSITE>
@@ -114,7 +114,7 @@ cudaError_t patch_store_launch(const PatchArgs& a, dim3 grid, cudaStream_t st, b
     if (prepare)
         return cudaFuncSetAttribute(k_step_patch_store<S, PREC, HSITE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)smem);
-    return launch_pdl(k_step_patch_store<S, PREC, HSITE>, grid, dim3(kPT, PatchShape<S>::TY), smem, st, a);
+    return launch_pdl(a.pdl != 0, k_step_patch_store<S, PREC, HSITE>, grid, dim3(kPT, PatchShape<S>::TY), smem, st, a);
 }
 
 template <int S, bool PREC, bool HSITE, bool STORE>
@@ -123,7 +123,7 @@ cudaError_t patch_tma_launch(const PatchArgs& a, const TmaMaps* maps, dim3 grid,
     if (prepare)
         return cudaFuncSetAttribute(k_step_patch_tma<S, PREC, HSITE, STORE>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    return launch_pdl(k_step_patch_tma<S, PREC, HSITE, STORE>, grid, dim3(kPT, PatchShape<S>::TY), smem, st, a, *maps);
+    return launch_pdl(a.pdl != 0, k_step_patch_tma<S, PREC, HSITE, STORE>, grid, dim3(kPT, PatchShape<S>::TY), smem, st, a, *maps);
 }
 
 template <int S>
@@ -346,7 +346,7 @@ cudaError_t launch_pulse_lattice(const StepLaunch<float>& L) {
     const long long N = L.g.N();
     const int blocks = (int)std::max<long long>(1, std::min<long long>((N + 255) / 256, 152LL * 32));
     float* const* o = L.pulse_out[0] ? L.pulse_out : L.out;
-    return launch_pdl_in(N <= kPdlGraphSites, k_pulse_f32, dim3(blocks), dim3(256), 0, L.stream, (const float*)L.out[0], (const float*)L.out[1],
+    return launch_pdl(!L.graph || N <= kPdlGraphSites, k_pulse_f32, dim3(blocks), dim3(256), 0, L.stream, (const float*)L.out[0], (const float*)L.out[1],
                       (const float*)L.out[2], o[0], o[1], o[2], (unsigned)N, L.seed, L.d_interval, L.replica, L.sigma);
 }
 

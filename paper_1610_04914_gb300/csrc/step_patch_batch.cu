@@ -45,8 +45,8 @@ cudaError_t batch_launch(const PatchArgs& a, const BatchItem* items, int nitems,
         return cudaFuncSetAttribute(k_step_patch_batch<S, PREC, PULSE, V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)smem);
     if (nitems <= 0) return cudaSuccess;
-    return launch_pdl(k_step_patch_batch<S, PREC, PULSE, V>, dim3(nitems), dim3(kPT, PatchShape<S, V>::TY), smem, st, a,
-                      items, reps);
+    k_step_patch_batch<S, PREC, PULSE, V><<<nitems, dim3(kPT, PatchShape<S, V>::TY), smem, st>>>(a, items, reps);
+    return cudaGetLastError();
 }
 
 template <int S, int V>
@@ -110,8 +110,8 @@ __global__ void __launch_bounds__(256) k_pulse_batch(float* __restrict__ sx, flo
 }  // namespace
 
 cudaError_t launch_pulse_batch(float* s[3], const BatchRep* reps, const ObsBlock* blocks, int nblocks, uint64_t seed,
-                               const long long* d_interval, cudaStream_t st) {
-    return launch_pdl(k_pulse_batch, dim3(nblocks), dim3(256), 0, st, s[0], s[1], s[2], reps, blocks, seed, d_interval);
+                               const long long* d_interval, cudaStream_t st, bool graph) {
+    return launch_pdl(!graph, k_pulse_batch, dim3(nblocks), dim3(256), 0, st, s[0], s[1], s[2], reps, blocks, seed, d_interval);
 }
 int patch_out_x(int stages) { return kPC - 2 * stages; }
 int patch_rows(int stages, int variant) {

@@ -71,7 +71,8 @@ struct Rk5Args {
     float a21, a31, a32, a42, a43, a51, a54, a61, a62, a63, a64, a65;
     float b1, b3, b4, b5, b6;
     int renorm;
-    int bc;                          // 1: free boundaries
+    int bc;
+    int pdl;                         // host: launch as a programmatic dependent
     int pair8;                       // 1: column pairs are aligned 8-byte words of the state arrays
     int* err;                        // device status word: bit 0 set when a bounded wait gave up
 };
@@ -493,7 +494,7 @@ cudaError_t rk5_launch(const Rk5Args& a, dim3 grid, cudaStream_t st, bool prepar
     if (prepare)
         return cudaFuncSetAttribute(k_step_rk5<SEG, PREC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)rk5_smem<SEG>());
-    return launch_pdl(k_step_rk5<SEG, PREC>, grid, dim3(kPT, kTY), rk5_smem<SEG>(), st, a);
+    return launch_pdl(a.pdl != 0, k_step_rk5<SEG, PREC>, grid, dim3(kPT, kTY), rk5_smem<SEG>(), st, a);
 }
 
 // The kernel hard-codes which Butcher coefficients are zero.
@@ -551,6 +552,7 @@ cudaError_t launch_step_rk5(const StepLaunch<float>& L) {
     a.b6 = c(tb.b[5]);
     a.renorm = L.renorm;
     a.bc = L.bc;
+    a.pdl = L.graph ? 0 : 1;
     a.car = L.tmp;   // 12 floats per site in the step scratch
     a.err = L.d_status;
     a.pair8 = pairs_aligned(a.nx, L.in[0], L.in[1], L.in[2]) && pairs_aligned(a.nx, L.out[0], L.out[1], L.out[2]);

@@ -43,6 +43,7 @@ struct Stage64Args {
     double c;              // dt a_{j+1,j}; last stage: dt b_S
     double g0, gx;         // last stage of S = 2: weights of s and X_2
     int bc, renorm;
+    int pdl;   // host: launch as a programmatic dependent
     uint64_t seed, replica;
     double sigma;
     const long long* interval;
@@ -179,10 +180,10 @@ cudaError_t stage_launch(const Stage64Args& a, cudaStream_t st) {
     const dim3 block(wide ? 128 : 32), grid((unsigned)(((unsigned)a.N + block.x - 1) / block.x));
     const bool unitx = !HSITE && a.J == 1.0 && a.H[0] == 0.0 && a.H[1] == 0.0;
     if (wide)
-        return unitx ? launch_pdl(k_stage64<ROLE, PREC, HSITE, PULSE, true, !HSITE>, grid, block, 0, st, a)
-                     : launch_pdl(k_stage64<ROLE, PREC, HSITE, PULSE, true, false>, grid, block, 0, st, a);
-    return unitx ? launch_pdl(k_stage64<ROLE, PREC, HSITE, PULSE, false, !HSITE>, grid, block, 0, st, a)
-                 : launch_pdl(k_stage64<ROLE, PREC, HSITE, PULSE, false, false>, grid, block, 0, st, a);
+        return unitx ? launch_pdl(a.pdl != 0, k_stage64<ROLE, PREC, HSITE, PULSE, true, !HSITE>, grid, block, 0, st, a)
+                     : launch_pdl(a.pdl != 0, k_stage64<ROLE, PREC, HSITE, PULSE, true, false>, grid, block, 0, st, a);
+    return unitx ? launch_pdl(a.pdl != 0, k_stage64<ROLE, PREC, HSITE, PULSE, false, !HSITE>, grid, block, 0, st, a)
+                 : launch_pdl(a.pdl != 0, k_stage64<ROLE, PREC, HSITE, PULSE, false, false>, grid, block, 0, st, a);
 }
 
 template <int ROLE, bool PULSE>
@@ -218,6 +219,7 @@ cudaError_t launch_step_stage64(const StepLaunch<double>& L) {
     a.lambda = L.ph.lambda;
     a.bc = L.bc;
     a.renorm = L.renorm;
+    a.pdl = L.graph ? 0 : 1;
     a.seed = L.seed;
     a.replica = L.replica;
     a.sigma = L.sigma;

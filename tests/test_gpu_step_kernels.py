@@ -191,7 +191,7 @@ def test_fp64_stage_sums(gpu, orc):
 # rectangular noise with 8, 4, 2 and 1 lanes per replica (the last warp partly
 # idle), calls that end mid-interval, against the oracle on sampled replicas
 @pytest.mark.parametrize("prec,tol", [(64, 1e-12), (32, 2e-5)])
-@pytest.mark.parametrize("nrep", [3, 2049, 6145, 12289])
+@pytest.mark.parametrize("nrep", [3, 2049, 6145, 10241])
 @pytest.mark.parametrize("integ,R", [(3, 1), (1, 4)])
 def test_single_rect_lanes(gpu, orc, prec, tol, nrep, integ, R):
     p = gpu.Params(1, 1, 1, J=0.0, D=0.4, H=(0.3, -0.2, 0.4), lam=0.2, T=0.0, dt=0.1, R=R, integrator=integ, noise=2,
@@ -212,3 +212,30 @@ def test_single_rect_lanes(gpu, orc, prec, tol, nrep, integ, R):
         ref, smp = orc.run(q, s0[:, r].reshape(3, 1, 1, 1), 21, noise=2)
         assert np.max(np.abs(got[:, r] - ref.reshape(3))) < tol
         assert abs(sums[r] - smp[:, 3].sum()) < 21 * tol
+
+
+# lattices just within and beyond the sizes that take the per-stage FP32
+# kernels: bitwise one trajectory per lattice however its sites are computed --
+# a batch replica (always the tile) against the single lattice at the same size,
+# and the oracle at a ragged, a flat, a free-boundary and a field lattice
+@pytest.mark.parametrize("integ", ["RK4", "RK2_MIDPOINT", "HEUN"])
+@pytest.mark.parametrize("L", [8, 47, 48, 49, 64, 65])
+def test_fp32_stage_kernels_bitwise(gpu, integ, L):
+    if integ == "RK4" and L > 49 or integ == "HEUN" and L not in (8, 64):
+        pytest.skip("far from this tableau's size limit")
+    kw = dict(J=0.9, D=0.15, H=(0.05, -0.1, 0.2), lam=0.1, dt=0.07, R=3, seed=77, integrator=getattr(gpu, integ))
+    s0 = spin_inputs.random_spins(L, L, L, seed=3).astype(np.float32)
+    b = gpu.Batch(gpu.Params(1, 1, 1, **kw), [L], [0.7], [s0], chunk_planes=gpu.batch.DEFAULT_TILING)
+    lat = gpu.Lattice(gpu.Params(L, L, L, T=0.7, **kw), torch.from_numpy(s0))
+    b.step(7)
+    lat.step(7)
+    torch.cuda.synchronize()
+    assert torch.equal(lat.state, b.replica_state(0))
+
+
+@pytest.mark.parametrize("integ", ["RK4", "RK2_MIDPOINT", "HEUN"])
+@pytest.mark.parametrize("shape,precession,hsite,bc", [
+    ((129, 151, 1), 1, False, 0), ((1, 1, 700), 0, True, 1), ((45, 37, 27), 1, True, 1), ((57, 56, 55), 0, True, 0)])
+def test_fp32_stage_kernels_oracle(gpu, orc, integ, shape, precession, hsite, bc):
+    _compare(gpu, orc, shape, 3 * 2e-6, hsite=hsite, precision=32, integrator=getattr(gpu, integ),
+             precession=precession, bc=bc)
