@@ -452,45 +452,53 @@ __global__ void __launch_bounds__(kAT, CHAIN ? SPIN_ADJ_MINB : 1) k_adj_x0_top(X
     pdl_go();
 }
 
-// FP64 sums of kSumParts consecutive parts of each of the arrays at v + c N
-// (c < gridDim.y, N doubles each): block (p, c) writes parts[c kSumParts + p];
-// fixed order (deterministic).
+// FP64 sums of kSumParts consecutive parts of each of five arrays of N doubles
+// (the per-site dL/dJ and dL/dD terms and the three components of the field
+// gradient, whose sum is dL/dH): block (p, c) writes parts[c kSumParts + p];
+// fixed order (deterministic), four chains of additions per thread.
 constexpr int kSumParts = 152;
-__global__ void k_adj_sum_parts(const double* __restrict__ v, long long N, double* __restrict__ parts) {
+__global__ void __launch_bounds__(kAT) k_adj_sum_parts(const double* __restrict__ gjd, const double* __restrict__ gh,
+                                                       long long N, double* __restrict__ parts) {
     __shared__ double red[kAW];
+    pdl_wait();
     const long long c = blockIdx.y, p = blockIdx.x;
     const long long lo = p * N / kSumParts, hi = (p + 1) * N / kSumParts;
-    const double* g = v + c * N;
-    double t = 0;
-    for (long long q = lo + threadIdx.x; q < hi; q += blockDim.x) t += g[q];
-    t = block_sum<double>(t, red);
-    if (threadIdx.x == 0) parts[c * kSumParts + p] = t;
+    const double* g = c < 2 ? gjd + c * N : gh + (c - 2) * N;
+    double t[4] = {0, 0, 0, 0};
+    long long q = lo + threadIdx.x;
+    for (; q + 3 * kAT < hi; q += 4 * kAT)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) t[k] += g[q + k * kAT];
+    for (; q < hi; q += kAT) t[0] += g[q];
+    const double v = block_sum<double>((t[0] + t[1]) + (t[2] + t[3]), red);
+    if (threadIdx.x == 0) parts[c * kSumParts + p] = v;
+    pdl_go();
 }
 
-// acc[first + c] (+)= the FP64 sum of parts[c kSumParts ...] (one block per
-// array, fixed order): dL/dJ, dL/dD (added to the seed's explicit terms) from
-// the per-site terms, dL/dH = sum_i dL/dh_i from the field gradient.
-__global__ void k_adj_sum_final(const double* __restrict__ parts, double* __restrict__ acc, int first, int add) {
+// acc[c] = the FP64 sum of parts[c kSumParts ...] (one block per array, fixed
+// order).
+__global__ void __launch_bounds__(kAT) k_adj_sum_final(const double* __restrict__ parts, double* __restrict__ acc) {
     __shared__ double red[kAW];
+    pdl_wait();
     const double* g = parts + (long long)blockIdx.x * kSumParts;
     double v = 0;
-    for (int q = threadIdx.x; q < kSumParts; q += blockDim.x) v += g[q];
+    for (int q = threadIdx.x; q < kSumParts; q += kAT) v += g[q];
     const double t = block_sum<double>(v, red);
-    if (threadIdx.x == 0) acc[first + blockIdx.x] = add ? acc[first + blockIdx.x] + t : t;
+    if (threadIdx.x == 0) acc[blockIdx.x] = t;
 }
 
-// Loss seed: lam_i = (-dLdE H_eff,i + dLdM)/N from the final state, with the
-// explicit final-time terms: partials of bonds (J) and sum s_z^2 (D);
-// gh += -dLdE s_i/N (the explicit dE/dh_i, which also gives dE/dH through the
-// final sum of gh).
+// Loss seed: lam_i = (-dLdE H_eff,i + dLdM)/N from the final state, and the
+// first terms of the FP64 gradient arrays, the explicit dependence of E(s_n) on
+// the parameters: gh = -dLdE s_i/N and, in gjd, -dLdE/N times the site's
+// forward bonds (J) and s_z^2 (D).  cE = -dLdE/N, cM = dLdM/N.  (About 20 FP64
+// instructions a site; with divisions, hardware conversions and block sums of
+// the bonds it took 55 us of a 64^3 gradient.)
 template <typename real, bool HSITE>
 __global__ void __launch_bounds__(kAT) k_adj_seed(CV3<real> s, CV3<real> hs, V3<real> lam, V3<double> gh,
-                                                  double* __restrict__ partials, AdjGeom<real> G, double dLdE,
-                                                  double dM0, double dM1, double dM2) {
-    __shared__ double red[kAW];
-    const long long N = G.N;
-    const double dM[3] = {dM0, dM1, dM2};
-    double bonds = 0, sz2 = 0;
+                                                  double* __restrict__ gjd, AdjGeom<real> G, double cE, double cM0,
+                                                  double cM1, double cM2) {
+    pdl_wait();
+    const double cM[3] = {cM0, cM1, cM2};
     const Site<real> st = site_here<real>(G.nx, G.ny, G.nz, G.bc);
     const int i = st.i;
     real h[3];
@@ -501,40 +509,22 @@ __global__ void __launch_bounds__(kAT) k_adj_seed(CV3<real> s, CV3<real> hs, V3<
     }
     h[2] += G.twoD * s.c[2][i];
     if (st.valid) {
+        double bonds = 0;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            lam.c[c][i] = (real)((-dLdE * (double)h[c] + dM[c]) / (double)N);
-            gh.c[c][i] += -dLdE * (double)s.c[c][i] / (double)N;
+            const double v = to_f64(s.c[c][i]);
+            lam.c[c][i] = (real)fma(cE, to_f64(h[c]), cM[c]);
+            gh.c[c][i] = cE * v;
+            double f = 0;   // forward neighbours inside the lattice
+            if (st.wn[1] != real(0)) f += to_f64(s.c[c][st.nb[1]]);
+            if (st.wn[3] != real(0)) f += to_f64(s.c[c][st.nb[3]]);
+            if (st.wn[5] != real(0)) f += to_f64(s.c[c][st.nb[5]]);
+            bonds = fma(v, f, bonds);
+            if (c == 2) gjd[G.N + i] = cE * (v * v);
         }
-        const double a = s.c[0][i], b = s.c[1][i], c = s.c[2][i];
-        const double w1 = st.wn[1], w3 = st.wn[3], w5 = st.wn[5];   // forward bonds inside the lattice
-        const int* nb = st.nb;
-        bonds = a * (w1 * s.c[0][nb[1]] + w3 * s.c[0][nb[3]] + w5 * s.c[0][nb[5]]) +
-                b * (w1 * s.c[1][nb[1]] + w3 * s.c[1][nb[3]] + w5 * s.c[1][nb[5]]) +
-                c * (w1 * s.c[2][nb[1]] + w3 * s.c[2][nb[3]] + w5 * s.c[2][nb[5]]);
-        sz2 = c * c;
+        gjd[i] = cE * bonds;
     }
-    const double vals[2] = {bonds, sz2};
-    for (int q = 0; q < 2; ++q) {
-        const double t = block_sum<double>(vals[q], red);
-        if (threadIdx.x == 0) partials[(long long)block_record() * 2 + q] = t;
-    }
-}
-
-// explicit terms -> gradient accumulators acc = (gJ, gD)
-__global__ void k_adj_seed_finish(const double* __restrict__ partials, int nblocks, double* __restrict__ acc,
-                                  double dLdE, double N) {
-    __shared__ double red[kAW];
-    double t[2];
-    for (int q = 0; q < 2; ++q) {
-        double v = 0;
-        for (int b = threadIdx.x; b < nblocks; b += blockDim.x) v += partials[(long long)b * 2 + q];
-        t[q] = block_sum<double>(v, red);
-    }
-    if (threadIdx.x == 0) {
-        acc[0] += -dLdE * t[0] / N;
-        acc[1] += -dLdE * t[1] / N;
-    }
+    pdl_go();
 }
 
 int grid_for(long long n) { return (int)std::max<long long>(1, std::min<long long>((n + kAT - 1) / kAT, 152LL * 8)); }
@@ -544,11 +534,6 @@ int grid_for(long long n) { return (int)std::max<long long>(1, std::min<long lon
 dim3 grid3(const Geom& g) { return dim3((g.nx + 31) / 32, (g.ny + kAW - 1) / kAW, g.nz); }
 
 }  // namespace
-
-int adjoint_blocks(Geom g) {
-    const dim3 d = grid3(g);
-    return (int)(d.x * d.y * d.z);
-}
 
 constexpr size_t kStageStoreMax = (size_t)8 << 30;   // bytes of stage storage at most
 
@@ -573,7 +558,6 @@ size_t adjoint_workspace_bytes(const Geom& g, int elt, const Tableau& tb, int pa
     b += al(sizeof(double) * 3 * (size_t)g.N());   // FP64 field gradient when the caller does not want it
     b += al(sizeof(double) * 2 * (size_t)g.N());   // FP64 per-site dL/dJ and dL/dD terms
     b += al(sizeof(double) * 5 * (size_t)kSumParts);           // per-part sums of those and of the field gradient
-    b += al(sizeof(double) * 2 * (size_t)adjoint_blocks(g));   // the seed's per-block partials
     b += al(sizeof(double) * 8);         // accumulators
     b += al(sizeof(long long));          // pulse-number slot
     return b;
@@ -732,14 +716,11 @@ cudaError_t adjoint_run(const AdjointRun<real>& A) {
     // is its sum either way)
     double* gh = A.g_h ? A.g_h : reinterpret_cast<double*>(ws + off);
     off += al(sizeof(double) * 3 * (size_t)N);
-    const int nb = adjoint_blocks(g);
     const dim3 gb = grid3(g);
     double* gjd = reinterpret_cast<double*>(ws + off);
     off += al(sizeof(double) * 2 * (size_t)N);
     double* parts = reinterpret_cast<double*>(ws + off);
     off += al(sizeof(double) * 5 * (size_t)kSumParts);
-    double* partials = reinterpret_cast<double*>(ws + off);
-    off += al(sizeof(double) * 2 * (size_t)nb);
     double* acc = reinterpret_cast<double*>(ws + off);
     off += al(sizeof(double) * 8);
     long long* kslot = reinterpret_cast<long long*>(ws + off);
@@ -772,23 +753,16 @@ cudaError_t adjoint_run(const AdjointRun<real>& A) {
     G.H[2] = (real)A.H[2];
     G.lambda = (real)A.lambda;
     G.dt = (real)A.dt;
-    cudaError_t e = cudaMemsetAsync(acc, 0, sizeof(double) * 8, st);
-    if (e != cudaSuccess) return e;
-    if (!A.g_h && (e = cudaMemsetAsync(gh, 0, sizeof(double) * 3 * (size_t)N, st)) != cudaSuccess) return e;
+    cudaError_t e;
 
     // seed from the final state (component arrays of the caller)
     CV3<real> fin;
     for (int c = 0; c < 3; ++c) fin.c[c] = A.final_state[c];
-    if (HS)
-        k_adj_seed<real, true><<<gb, kAT, 0, st>>>(fin, hs3, v3<real>(lam, N), gh3, partials, G, A.dLdE, A.dLdM[0],
-                                                   A.dLdM[1], A.dLdM[2]);
-    else
-        k_adj_seed<real, false><<<gb, kAT, 0, st>>>(fin, hs3, v3<real>(lam, N), gh3, partials, G, A.dLdE, A.dLdM[0],
-                                                    A.dLdM[1], A.dLdM[2]);
-    k_adj_seed_finish<<<1, kAT, 0, st>>>(partials, nb, acc, A.dLdE, (double)N);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    // the per-site FP64 J and D terms start at zero
-    e = cudaMemsetAsync(gjd, 0, sizeof(double) * 2 * (size_t)N, st);
+    const double invN = 1.0 / (double)N, cE = -A.dLdE * invN;
+    e = HS ? adj_launch(k_adj_seed<real, true>, gb, st, fin, hs3, v3<real>(lam, N), gh3, gjd, G, cE, A.dLdM[0] * invN,
+                        A.dLdM[1] * invN, A.dLdM[2] * invN)
+           : adj_launch(k_adj_seed<real, false>, gb, st, fin, hs3, v3<real>(lam, N), gh3, gjd, G, cE, A.dLdM[0] * invN,
+                        A.dLdM[1] * invN, A.dLdM[2] * invN);
     if (e != cudaSuccess) return e;
 
     const long long total = A.n_end - A.n0;
@@ -936,13 +910,10 @@ cudaError_t adjoint_run(const AdjointRun<real>& A) {
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
         }
     }
-    // dL/dJ, dL/dD (added to the seed's explicit terms) and dL/dH: FP64 sums in
-    // two deterministic passes
-    k_adj_sum_parts<<<dim3(kSumParts, 2), kAT, 0, st>>>(gjd, N, parts);
-    k_adj_sum_parts<<<dim3(kSumParts, 3), kAT, 0, st>>>(gh, N, parts + 2 * kSumParts);
-    k_adj_sum_final<<<2, kAT, 0, st>>>(parts, acc, 0, 1);
-    k_adj_sum_final<<<3, kAT, 0, st>>>(parts + 2 * kSumParts, acc, 2, 0);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    // dL/dJ, dL/dD and dL/dH: FP64 sums in two deterministic passes
+    if ((e = adj_launch(k_adj_sum_parts, dim3(kSumParts, 5), st, (const double*)gjd, (const double*)gh, N, parts)) != cudaSuccess)
+        return e;
+    if ((e = adj_launch(k_adj_sum_final, dim3(5), st, (const double*)parts, acc)) != cudaSuccess) return e;
     // results: gradient accumulators to the host, dL/ds_0 to the caller
     if (A.g_s0) {
         e = cudaMemcpyAsync(A.g_s0, lam, compb, cudaMemcpyDeviceToDevice, st);

@@ -310,7 +310,6 @@ int backward_t(spin_lattice* h, const double dLdM[3], double dLdE, void* ws, dou
     A.gH = gH;
     A.g_h = static_cast<double*>(g_h_site);
     A.g_s0 = static_cast<real*>(g_s0);
-    if (g_h_site) SPIN_CUDA(h, cudaMemsetAsync(g_h_site, 0, sizeof(double) * 3 * (size_t)h->g.N(), h->st));
     SPIN_CUDA(h, adjoint_run<real>(A));
     int status = 0;   // the recomputing steps' bounded waits (adjoint_run has synchronised)
     SPIN_CUDA(h, cudaMemcpy(&status, h->d_status, sizeof(int), cudaMemcpyDeviceToHost));
