@@ -3,6 +3,7 @@
 // CUDA-graph cache for whole noise intervals.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -13,6 +14,16 @@
 #include "spin_internal.h"
 
 using namespace spin;
+
+// Small lattices replay several intervals as one graph: the GPU idles for a few
+// microseconds between two graph launches, and an interval of a few small kernels
+// takes only tens (64^3, RK2, R = 2, ten intervals of a call 477 -> 452 us).
+// A longer graph is captured once enough intervals have been replayed to pay for
+// it, and holds at most kGraphSteps steps.
+constexpr int kGraphLevels = 4;
+constexpr int kGraphSteps = 32;
+constexpr long long kLongGraphSites = 1LL << 20;
+constexpr long long kLongGraphAfter = 8;
 
 struct spin_lattice {
     spin_params p;
@@ -36,8 +47,9 @@ struct spin_lattice {
     int* d_status;           // bit 0: a bounded device wait gave up
     double* ring;
     long long samples_read;
-    cudaGraphExec_t graph[2];  // one noise interval starting from buffer 0 / 1
-    int graph_end[2];          // the buffer it ends in
+    cudaGraphExec_t graph[kGraphLevels][2];  // 2^level noise intervals starting from buffer 0 / 1
+    int graph_end[kGraphLevels][2];          // the buffer they end in
+    long long replayed;        // intervals replayed from graphs
     cudaStream_t capture_stream;
     // trajectory recording for the adjoint
     bool rec_active;
@@ -229,20 +241,20 @@ cudaError_t launch_one_step(spin_lattice* h, int* buf, long long n_next, cudaStr
     return e;
 }
 
-// Capture one full interval (R steps + sample) starting from buffer `from`.
-int capture_interval(spin_lattice* h, int from) {
+// Capture 2^level full intervals (R steps + sample) starting from buffer `from`.
+int capture_interval(spin_lattice* h, int level, int from) {
     if (!h->capture_stream) SPIN_CUDA(h, cudaStreamCreateWithFlags(&h->capture_stream, cudaStreamNonBlocking));
     cudaStream_t cs = h->capture_stream;
     SPIN_CUDA(h, cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
     const int R = h->p.steps_per_pulse;
     int b = from;
     cudaError_t e = cudaSuccess;
-    // the graph covers steps mR+1 .. mR+R; pulse and sample positions depend
-    // only on n mod R, so step numbers 1..R describe every interval
-    for (int q = 1; q <= R && e == cudaSuccess; ++q) {
+    // the graph covers steps mR+1 .. (m+2^level)R; pulse and sample positions
+    // depend only on n mod R, so step numbers from 1 on describe every interval
+    for (int q = 1; q <= (R << level) && e == cudaSuccess; ++q) {
         e = launch_one_step(h, &b, q, cs);
     }
-    h->graph_end[from] = b;
+    h->graph_end[level][from] = b;
     cudaGraph_t graph = nullptr;
     cudaError_t e2 = cudaStreamEndCapture(cs, &graph);
     if (e != cudaSuccess) {
@@ -250,13 +262,35 @@ int capture_interval(spin_lattice* h, int from) {
         return set_err(h, SPIN_ECUDA, "interval capture: %s", cudaGetErrorString(e));
     }
     if (e2 != cudaSuccess) return set_err(h, SPIN_ECUDA, "cudaStreamEndCapture: %s", cudaGetErrorString(e2));
-    cudaError_t e3 = cudaGraphInstantiate(&h->graph[from], graph, 0);
+    cudaError_t e3 = cudaGraphInstantiate(&h->graph[level][from], graph, 0);
     cudaGraphDestroy(graph);
     if (e3 != cudaSuccess) {
-        h->graph[from] = nullptr;
+        h->graph[level][from] = nullptr;
         return set_err(h, SPIN_ECUDA, "cudaGraphInstantiate: %s", cudaGetErrorString(e3));
     }
     return SPIN_OK;
+}
+
+// Replay 2^level intervals from the current state's buffer.
+int replay(spin_lattice* h, int level) {
+    if (!h->graph[level][h->cur]) {
+        const int rc = capture_interval(h, level, h->cur);
+        if (rc != SPIN_OK) return rc;
+    }
+    SPIN_CUDA(h, cudaGraphLaunch(h->graph[level][h->cur], h->st));
+    h->n += (long long)h->p.steps_per_pulse << level;
+    h->cur = h->graph_end[level][h->cur];
+    h->replayed += 1LL << level;
+    return SPIN_OK;
+}
+
+// The longest graph for a call that has nsteps left.
+int graph_level(const spin_lattice* h, long long nsteps) {
+    if (h->g.N() > kLongGraphSites || h->replayed < kLongGraphAfter) return 0;
+    int level = 0;
+    while (level + 1 < kGraphLevels && ((long long)h->p.steps_per_pulse << (level + 1)) <= std::min<long long>(nsteps, kGraphSteps))
+        ++level;
+    return level;
 }
 
 // While recording, copy the current state into checkpoint slot (n-n0)/K
@@ -418,15 +452,10 @@ int spin_step_pulse(spin_lattice* h, int64_t nsteps) {
             const long long d0 = h->n - h->rec_n0;
             const long long next_ckpt = (d0 / h->rec_K + 1) * h->rec_K;
             if (h->n % R == 0 && nsteps >= R && h->eager_intervals > 0 && d0 >= 0 && next_ckpt >= d0 + R) {
-                if (!h->graph[h->cur]) {
-                    int rc = capture_interval(h, h->cur);
-                    if (rc != SPIN_OK) return rc;
-                }
-                SPIN_CUDA(h, cudaGraphLaunch(h->graph[h->cur], h->st));
-                h->n += R;
-                h->cur = h->graph_end[h->cur];
+                int rc = replay(h, 0);
+                if (rc != SPIN_OK) return rc;
                 nsteps -= R;
-                int rc = record_if_due(h);
+                rc = record_if_due(h);
                 if (rc != SPIN_OK) return rc;
                 continue;
             }
@@ -439,14 +468,10 @@ int spin_step_pulse(spin_lattice* h, int64_t nsteps) {
             continue;
         }
         if (h->n % R == 0 && nsteps >= R && h->eager_intervals > 0) {
-            if (!h->graph[h->cur]) {
-                int rc = capture_interval(h, h->cur);
-                if (rc != SPIN_OK) return rc;
-            }
-            SPIN_CUDA(h, cudaGraphLaunch(h->graph[h->cur], h->st));
-            h->n += R;
-            h->cur = h->graph_end[h->cur];
-            nsteps -= R;
+            const int level = graph_level(h, nsteps);
+            const int rc = replay(h, level);
+            if (rc != SPIN_OK) return rc;
+            nsteps -= (int64_t)R << level;
             continue;
         }
         const bool interval_start = h->n % R == 0 && nsteps >= R;
@@ -470,11 +495,18 @@ int spin_step_pulse(spin_lattice* h, int64_t nsteps) {
 int spin_observables(spin_lattice* h, double M[3], double* E) {
     if (!h || !M || !E) return SPIN_EINVAL;
     SPIN_CUDA(h, observe(h, h->cur, false, h->st));
-    double o[5];
-    int status = 0;
-    SPIN_CUDA(h, cudaMemcpyAsync(o, h->out_obs, sizeof(o), cudaMemcpyDeviceToHost, h->st));
-    SPIN_CUDA(h, cudaMemcpyAsync(&status, h->d_status, sizeof(int), cudaMemcpyDeviceToHost, h->st));
+    // one copy from the observables to the status word (neighbours in the
+    // workspace): a small copy to the host costs 5 us or more
+    char host[1024];
+    const size_t span = reinterpret_cast<char*>(h->d_status) - reinterpret_cast<char*>(h->out_obs) + sizeof(int);
+    static_assert(4 * kAlign <= sizeof(host), "observables, interval, sample count and status");
+    if (span > sizeof(host)) return set_err(h, SPIN_EINVAL, "workspace layout");
+    SPIN_CUDA(h, cudaMemcpyAsync(host, h->out_obs, span, cudaMemcpyDeviceToHost, h->st));
     SPIN_CUDA(h, cudaStreamSynchronize(h->st));
+    double o[5];
+    int status;
+    memcpy(o, host, sizeof(o));
+    memcpy(&status, host + span - sizeof(int), sizeof(int));
     if (status & 1) return set_err(h, SPIN_ETIMEOUT, "a bounded wait in the fused step gave up; the state is invalid");
     M[0] = o[0];
     M[1] = o[1];
@@ -486,21 +518,30 @@ int spin_observables(spin_lattice* h, double M[3], double* E) {
 
 int spin_samples(spin_lattice* h, double* out, int64_t max_records, int64_t* count) {
     if (!h || !count || (max_records > 0 && !out) || max_records < 0) return SPIN_EINVAL;
-    long long total = 0;
-    int status = 0;
-    SPIN_CUDA(h, cudaMemcpyAsync(&total, h->d_sample_count, sizeof(total), cudaMemcpyDeviceToHost, h->st));
-    SPIN_CUDA(h, cudaMemcpyAsync(&status, h->d_status, sizeof(int), cudaMemcpyDeviceToHost, h->st));
+    // the count and the status word in one copy, then the records in one, or two
+    // where the ring wraps (one per record before: 10 records 80 us)
+    char host[2 * kAlign];
+    const size_t span = reinterpret_cast<char*>(h->d_status) - reinterpret_cast<char*>(h->d_sample_count) + sizeof(int);
+    if (span > sizeof(host)) return set_err(h, SPIN_EINVAL, "workspace layout");
+    SPIN_CUDA(h, cudaMemcpyAsync(host, h->d_sample_count, span, cudaMemcpyDeviceToHost, h->st));
     SPIN_CUDA(h, cudaStreamSynchronize(h->st));
+    long long total;
+    int status;
+    memcpy(&total, host, sizeof(total));
+    memcpy(&status, host + span - sizeof(int), sizeof(int));
     if (status & 1) return set_err(h, SPIN_ETIMEOUT, "a bounded wait in the fused step gave up; the state is invalid");
     long long first = h->samples_read;
     if (total - first > SPIN_SAMPLE_RING) first = total - SPIN_SAMPLE_RING;
     if (total - first > max_records) first = total - max_records;
     const long long n = total - first;
-    for (long long q = 0; q < n; ++q) {
+    for (long long q = 0; q < n;) {
         const long long slot = (first + q) % SPIN_SAMPLE_RING;
-        SPIN_CUDA(h, cudaMemcpyAsync(out + 5 * q, h->ring + 5 * slot, 5 * sizeof(double), cudaMemcpyDeviceToHost, h->st));
+        const long long m = std::min<long long>(n - q, SPIN_SAMPLE_RING - slot);
+        SPIN_CUDA(h, cudaMemcpyAsync(out + 5 * q, h->ring + 5 * slot, (size_t)m * 5 * sizeof(double),
+                                     cudaMemcpyDeviceToHost, h->st));
+        q += m;
     }
-    SPIN_CUDA(h, cudaStreamSynchronize(h->st));
+    if (n > 0) SPIN_CUDA(h, cudaStreamSynchronize(h->st));
     h->samples_read = total;
     *count = n;
     return SPIN_OK;
@@ -573,8 +614,9 @@ int spin_record_end(spin_lattice* h) {
 
 int spin_lattice_destroy(spin_lattice* h) {
     if (!h) return SPIN_EINVAL;
-    for (int b = 0; b < 2; ++b)
-        if (h->graph[b]) cudaGraphExecDestroy(h->graph[b]);
+    for (auto& level : h->graph)
+        for (cudaGraphExec_t g : level)
+            if (g) cudaGraphExecDestroy(g);
     if (h->capture_stream) cudaStreamDestroy(h->capture_stream);
     delete h;
     return SPIN_OK;

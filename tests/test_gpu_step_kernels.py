@@ -239,3 +239,21 @@ def test_fp32_stage_kernels_bitwise(gpu, integ, L):
 def test_fp32_stage_kernels_oracle(gpu, orc, integ, shape, precession, hsite, bc):
     _compare(gpu, orc, shape, 3 * 2e-6, hsite=hsite, precision=32, integrator=getattr(gpu, integ),
              precession=precession, bc=bc)
+
+
+def test_sample_ring_wraps_and_long_graphs(gpu):
+    """Samples read in portions across the ring's end, from intervals replayed
+    singly and several to a graph, equal the observables taken step by step."""
+    p = gpu.Params(6, 5, 4, J=1.0, D=0.1, H=(0.0, 0.0, 0.2), lam=0.1, T=0.5, dt=0.1, R=2, seed=3)
+    s0 = torch.from_numpy(spin_inputs.random_spins(6, 5, 4, seed=3))
+    a, b = gpu.Lattice(p, s0), gpu.Lattice(p, s0)
+    ring = gpu._binding.SPIN_SAMPLE_RING
+    a.step(2 * (ring - 3))
+    assert len(a.samples()) == ring - 3
+    a.step(2 * 11)
+    got = gpu.spin_samples(a.handle, 9)
+    for k in range(ring - 3 + 11):
+        b.step(2)
+    assert torch.equal(a.state, b.state)
+    want = b.samples()[-9:]
+    assert len(got) == 9 and got == want and got[-1][0] == 2.0 * (ring + 8)
