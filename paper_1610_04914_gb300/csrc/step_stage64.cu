@@ -1,5 +1,5 @@
 // FP64 step of the chain tableaus (RK4, RK2 midpoint, Heun): one kernel per
-// Runge-Kutta stage, one thread per site.
+// Runge-Kutta stage, one thread per site (four lanes on the smallest lattices).
 //
 // What bounds it: GB300's FP64 pipe, about two lanes per SM and cycle, so a
 // warp's FP64 instruction takes as long as some sixty other instructions and
@@ -11,8 +11,8 @@
 // computed exactly once, and the stage inputs X_j go through memory.  RK4,
 // one interval: 128^3 (4 steps, one pulse) 16.08 -> 3.60 ms, 16^3 (10 steps,
 // one pulse, observables) 2.09 -> 0.25 ms; with the sums below off the FP64
-// pipe and the cheaper noise draw 1.97 and 0.23 ms.  The pipe is then 85%
-// active.
+// pipe and the cheaper noise draw 1.97 and 0.23 ms; the pipe is then 85%
+// active at 128^3.  16^3 with four lanes per site: 0.18 ms.
 //
 // The accumulator of the tableau is not kept: with K_j = dt f(X_j) and
 // X_{j+1} = s + a_{j+1,j} K_j, every K_j but the last is (X_{j+1} - s)/a_{j+1,j},
@@ -109,8 +109,8 @@ __device__ __forceinline__ double rk4_sum(double x2, double x3, double x4, doubl
 enum StageRole { kFirst, kMiddle, kLast2, kLast4 };
 
 // WIDE: sums through the integer pipes, for lattices that fill the FP64 pipe
-// (the smallest ones wait on latencies instead, of which the integer form has
-// more: 16^3 242 against 250 us for 10 steps).  UNITX: J = 1 and the uniform
+// (smaller ones wait on latencies instead, of which the integer form has more:
+// 16^3 242 against 250 us for 10 steps).  UNITX: J = 1 and the uniform
 // field along z without site fields, so that H_x and H_y are the bare neighbour
 // sums (the products and sums with 1 and 0 would be two more instructions).
 template <int ROLE, bool PREC, bool HSITE, bool PULSE, bool WIDE, bool UNITX>
@@ -173,8 +173,91 @@ __global__ void __launch_bounds__(128) k_stage64(const __grid_constant__ Stage64
     for (int c = 0; c < 3; ++c) a.out[c][i] = o[c];
 }
 
+// The smallest lattices: four lanes per site, one component each (the fourth
+// repeats the third).  A warp's FP64 instruction takes 64 cycles of its
+// scheduler whatever its active lanes, and with a warp or two per scheduler a
+// stage lasts as long as the 37 FP64 instructions of one warp; split by
+// component a lane executes 13 (the pulse: half).  The other components' spins,
+// fields and cross products come by shuffles, the numbers are those of
+// k_stage64.  What is left is the launch and the loads: 2.5 us per stage.  Ten
+// RK4 steps with a pulse and one launch graph, one thread per site against four
+// lanes: 8^3 146 and 100 us, 16^3 150 and 109, 21^3 156 and 139, 22^3 162 and
+// 144, 24^3 158 and 166; two stages: 21^3 88 and 82, 24^3 88 and 98.
+constexpr int kLaneSites = 152 * 72;
+__device__ __forceinline__ double lane_get(double v, int lane) { return __shfl_sync(0xffffffffu, v, lane); }
+
+template <int ROLE, bool PREC, bool HSITE, bool PULSE>
+__global__ void __launch_bounds__(32) k_stage64_lanes(const __grid_constant__ Stage64Args a) {
+    pdl_go();
+    const int lane = (int)(threadIdx.x & 31), first = lane & ~3, c = min(lane & 3, 2);
+    const int l1 = first + (c + 1) % 3, l2 = first + (c + 2) % 3;   // lanes of the next two components
+    const int iu = (int)(blockIdx.x * 8 + (threadIdx.x >> 2));
+    const bool mine = iu < a.N && (lane & 3) < 3;
+    const int i = min(iu, a.N - 1);
+    const int row = i / a.nx, x = i - row * a.nx;
+    const int z = row / a.ny, y = row - z * a.ny;
+    const int P = a.nx * a.ny;
+    const int nb[6] = {x > 0 ? i - 1 : i + (a.nx - 1), x < a.nx - 1 ? i + 1 : i - (a.nx - 1),
+                       y > 0 ? i - a.nx : i + (P - a.nx), y < a.ny - 1 ? i + a.nx : i - (P - a.nx),
+                       z > 0 ? i - P : i + (a.nz - 1) * P, z < a.nz - 1 ? i + P : i - (a.nz - 1) * P};
+    const bool cut[6] = {a.bc && x == 0, a.bc && x == a.nx - 1, a.bc && y == 0,
+                         a.bc && y == a.ny - 1, a.bc && z == 0, a.bc && z == a.nz - 1};
+    auto pick = [c](const auto& p) { return c == 0 ? p[0] : c == 1 ? p[1] : p[2]; };
+    const double* q = pick(a.x);
+    const double* sp = pick(a.s);
+    const double Hc = pick(a.H);
+    pdl_wait();
+    double n[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) n[k] = cut[k] ? 0.0 : q[nb[k]];
+    const double v = q[i], s = ROLE == kFirst ? v : sp[i];
+    double x2 = 0, x3 = 0;
+    if (ROLE == kLast4) {
+        x2 = pick(a.q[0])[i];
+        x3 = pick(a.q[1])[i];
+    }
+    const double hs = HSITE ? pick(a.hs)[i] : 0.0;
+    double p = 0;
+    if (PULSE) {
+        // drawn while the loads above are in flight; components 0 and 1 of G
+        // share a radius and an angle, 2 has its own
+        const Words4 w = noise_words(a.seed, (uint64_t)i, (uint64_t)*a.interval, a.replica);
+        const double r = Gauss<double>::root(Gauss<double>::neg2log(Gauss<double>::u01(c == 2 ? w.w[2] : w.w[0])));
+        double cs, sn;
+        Gauss<double>::angle(c == 2 ? w.w[3] : w.w[1], cs, sn);
+        p = a.sigma * (r * (c == 1 ? sn : cs));
+    }
+    double h = a.J * (((n[0] + n[1]) + (n[2] + n[3])) + (n[4] + n[5])) + Hc;
+    if (HSITE) h += hs;
+    h += a.twoD * (c == 2 ? v : 0.0);
+    const double v1 = lane_get(v, l1), v2 = lane_get(v, l2);
+    const double A = v1 * lane_get(h, l2) - v2 * lane_get(h, l1);
+    const double B = v1 * lane_get(A, l2) - v2 * lane_get(A, l1);
+    const double f = PREC ? A - a.lambda * B : -a.lambda * B;
+    double o;
+    if (ROLE == kFirst || ROLE == kMiddle) {
+        o = s + a.c * f;
+    } else {
+        const double acc = ROLE == kLast4 ? (1.0 / 3.0) * ((x2 + 2.0 * x3) + (v - s)) : a.g0 * s + a.gx * v;
+        o = acc + a.c * f;
+        if (a.renorm) {
+            const double sq = o * o;
+            o *= rsqrt((lane_get(sq, first) + lane_get(sq, first + 1)) + lane_get(sq, first + 2));
+        }
+        if (PULSE) {
+            double s0 = lane_get(o, first), s1 = lane_get(o, first + 1), s2 = lane_get(o, first + 2);
+            pulse_rotate<double>(s0, s1, s2, lane_get(p, first), lane_get(p, first + 1), lane_get(p, first + 2), a.sigma);
+            o = c == 0 ? s0 : c == 1 ? s1 : s2;
+        }
+    }
+    if (mine) pick(a.out)[i] = o;
+}
+
 template <int ROLE, bool PREC, bool HSITE, bool PULSE>
 cudaError_t stage_launch(const Stage64Args& a, cudaStream_t st) {
+    if (a.N <= kLaneSites)
+        return launch_pdl(a.pdl != 0, k_stage64_lanes<ROLE, PREC, HSITE, PULSE>, dim3((unsigned)((a.N + 7) / 8)), dim3(32), 0,
+                          st, a);
     // up to one warp per scheduler: one warp per block, spread over the SMs
     const bool wide = a.N > 152 * 4 * 32;
     const dim3 block(wide ? 128 : 32), grid((unsigned)(((unsigned)a.N + block.x - 1) / block.x));

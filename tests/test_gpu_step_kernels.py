@@ -37,6 +37,17 @@ def test_fp64_stage_kernels(gpu, orc, integ, shape, precession, hsite, bc):
              precession=precession, bc=bc)
 
 
+# four lanes per site up to 10944 sites: a last block of one site, exactly the
+# line, one site beyond it; sides of 1, free faces, site fields
+@pytest.mark.parametrize("integ", ["RK4", "RK2_MIDPOINT", "HEUN"])
+@pytest.mark.parametrize("shape,precession,hsite,bc", [
+    ((1, 1, 1), 1, True, 0), ((3, 11, 1), 0, False, 1), ((5, 5, 5), 1, False, 1),
+    ((16, 18, 38), 1, True, 1), ((5, 11, 199), 0, True, 0)])
+def test_fp64_component_lanes(gpu, orc, integ, shape, precession, hsite, bc):
+    _compare(gpu, orc, shape, 1e-13, hsite=hsite, precision=64, integrator=getattr(gpu, integ),
+             precession=precession, bc=bc)
+
+
 # free spins (J = D = H = 0): three pulses with sigma at both sides of the
 # series limit 0.35, far above it (general form), and angles from ~0 to beyond
 # phi^2 = 4.  Per pulse the angle carries about four roundings of G, relative,
