@@ -13,6 +13,8 @@
 // term included).  The float-to-double conversions of the terms are done with
 // integer bit operations (exact for every finite float), because this GPU's
 // FP64 pipe, which would otherwise convert them, is ~1/76 of its FP32 rate.
+// Where the stages are stored (below), a step's terms stay floats until its last
+// stage and are added exactly, as 64-bit integers, before one FP64 addition each.
 //
 // Transposes used (f the right-hand side of Eq. LLL at fixed noise, a = s x H):
 //   w_i = (df_i/dH_i)^T v_i = -(s x v) - lambda s x (s x v)    [slow: without -(s x v)]
@@ -51,6 +53,11 @@ constexpr int kAW = kAT / 32;
 // blocks take 1.12 rounds of 152 SMs instead of 1.35; measured 4.5% faster
 // per backward step with the programmatic-dependent launches (8 blocks, 32
 // registers: 1%).
+// Without the FP64 arrays the stored-stage x/w-parts fit 32 registers: 8 blocks,
+// and 64^3 is one round.
+#ifndef SPIN_ADJ_LATEB
+#define SPIN_ADJ_LATEB 8
+#endif
 #ifndef SPIN_ADJ_MINB
 #define SPIN_ADJ_MINB 6
 #endif
@@ -211,20 +218,20 @@ struct StageIn {
 // site: on this GPU's narrow FP64 pipe a per-block tree reduction, at five
 // adds per warp and value, measured slower.)
 // Every load of the site is issued before the arithmetic.
-template <typename real, bool PREC, bool HSITE>
+template <typename real, bool PREC, bool HSITE, bool LATE>
 __device__ __forceinline__ void w_part(const StageIn<real>& in, const CV3<real>& hs, const Site<real>& st,
                                        const AdjGeom<real>& G, const real v[3], const V3<real>& w, const V3<real>& u,
-                                       const V3<double>& gh, double* __restrict__ gjd) {
+                                       const V3<double>& gh, double* __restrict__ gjd, real* __restrict__ tj) {
     const int i = st.i;
     real s[3], sn[3], hsv[3];
-    double g[3];
-    const double gj = gjd[i], gd = gjd[G.N + i];
+    double g[3] = {0, 0, 0};
+    const double gj = LATE ? 0.0 : gjd[i], gd = LATE ? 0.0 : gjd[G.N + i];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
         s[c] = in.x.c[c][i];
-        sn[c] = in.sn.c[0] ? in.sn.c[c][i] : nbsum<real>(in.x.c[c], st);
+        sn[c] = LATE || in.sn.c[0] ? in.sn.c[c][i] : nbsum<real>(in.x.c[c], st);
         hsv[c] = HSITE ? hs.c[c][i] : real(0);
-        g[c] = gh.c[c][i];
+        if (!LATE) g[c] = gh.c[c][i];
     }
     real hr[3];
 #pragma unroll
@@ -256,14 +263,79 @@ __device__ __forceinline__ void w_part(const StageIn<real>& in, const CV3<real>&
         if (st.valid) {
             w.c[c][i] = wi[c];
             u.c[c][i] = ui;
-            gh.c[c][i] = g[c] + to_f64(wi[c]);
+            if (!LATE) gh.c[c][i] = g[c] + to_f64(wi[c]);
         }
     }
     if (st.valid) {
-        gjd[i] = gj + to_f64(wi[0] * sn[0] + wi[1] * sn[1] + wi[2] * sn[2]);
-        gjd[G.N + i] = gd + to_f64(real(2) * s[2] * wi[2]);
+        const real tJ = wi[0] * sn[0] + wi[1] * sn[1] + wi[2] * sn[2], tD = real(2) * s[2] * wi[2];
+        if (LATE) {
+            tj[i] = tJ;
+            tj[G.N + i] = tD;
+        } else {
+            gjd[i] = gj + to_f64(tJ);
+            gjd[G.N + i] = gd + to_f64(tD);
+        }
     }
 }
+
+// The sum of a step's S terms (S = 2 or 4; the others zero) as a double,
+// rounded once: the mantissas, shifted to the largest exponent, add as 64-bit
+// integers; what lies 2^-60 below the largest term is lost.
+__device__ __noinline__ double plain_sum4(float a, float b, float c, float d) {
+    return (((double)a + (double)b) + (double)c) + (double)d;
+}
+__device__ __forceinline__ double sum4(const float (&v)[4]) {
+    unsigned emax = 1u;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) emax = max(emax, (__float_as_uint(v[k]) >> 23) & 0xFFu);
+    if (emax == 0xFFu) return plain_sum4(v[0], v[1], v[2], v[3]);
+    long long S = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const unsigned b = __float_as_uint(v[k]), e = (b >> 23) & 0xFFu;
+        const unsigned m = (b & 0x7FFFFFu) | (e ? 0x800000u : 0u);
+        const long long x = (long long)(((unsigned long long)m << 36) >> min(emax - max(e, 1u), 63u));
+        const long long sg = (long long)((int)b >> 31);
+        S += (x ^ sg) - sg;
+    }
+    return from_fixed(S, emax + 896u);   // units of 2^(emax - 186)
+}
+
+// A step's terms of the FP64 gradient arrays, in one go after its last stage
+// (stored stages): w of every stage is kept until here, as are the products
+// that the stages' w-parts wrote.  Added stage by stage, the read and write of
+// five doubles a site was 40% of a stage's traffic.  64^3, RK4, cold: the three
+// inner stages 11.6 -> 8.0 us, this one with the sums 11.9 -> 18.5; a gradient
+// over 20 steps 1560 -> 1525 us.  (Spread over the next step's stages instead,
+// w and terms in two sets of arrays: 1560, out of L2.)
+template <typename real>
+struct StepTerms {
+    CV3<real> w[4];        // w of each stage
+    const real* t[4];      // dL/dJ (N) and dL/dD (N) terms of each stage
+    int stages;            // 2 or 4
+    V3<double> gh;
+    double* gjd;
+};
+__device__ __forceinline__ void add_terms(const StepTerms<float>& a, const Site<float>& st, long long N) {
+    const int i = st.i;
+    float v[5][4];
+    double g[5];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const bool on = k < a.stages;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) v[c][k] = on ? a.w[k].c[c][i] : 0.0f;
+        v[3][k] = on ? a.t[k][i] : 0.0f;
+        v[4][k] = on ? a.t[k][N + i] : 0.0f;
+    }
+#pragma unroll
+    for (int c = 0; c < 5; ++c) {
+        double* const q = c < 3 ? a.gh.c[c] + i : a.gjd + (c - 3) * N + i;
+        g[c] = *q + sum4(v[c]);
+        if (st.valid) *q = g[c];
+    }
+}
+__device__ __forceinline__ void add_terms(const StepTerms<double>&, const Site<double>&, long long) {}   // never stored
 
 // Top of the transposed step: pulse and renormalisation transposes, lam_s =
 // lam_y, lam_K_j = b_j lam_y (stored for j < S-1; for chain tableaus lam_y
@@ -288,10 +360,11 @@ struct TopArgs {
     V3<real> w, u;       // w, u of stage S-1
     V3<double> gh;       // FP64 field gradient
     double* gjd;         // FP64 per-site dL/dJ (N) and dL/dD (N) terms
+    real* tj;            // stored stages: the stage's terms of those, added after the step
 };
 
 // The top at a site, given the adjoint (l0, l1, l2) of the step's output.
-template <typename real, bool PREC, bool HSITE, int S, bool CHAIN>
+template <typename real, bool PREC, bool HSITE, int S, bool CHAIN, bool LATE>
 __device__ __forceinline__ void top_body(const TopArgs<real>& a, const AdjGeom<real>& G, const Site<real>& st, real l0,
                                          real l1, real l2) {
     const int i = st.i;
@@ -303,7 +376,7 @@ __device__ __forceinline__ void top_body(const TopArgs<real>& a, const AdjGeom<r
     }
     if (a.renorm) {
         real y0, y1, y2;
-        if (a.ystored.c[0]) {
+        if (LATE || a.ystored.c[0]) {
             y0 = a.ystored.c[0][i];
             y1 = a.ystored.c[1][i];
             y2 = a.ystored.c[2][i];
@@ -338,15 +411,15 @@ __device__ __forceinline__ void top_body(const TopArgs<real>& a, const AdjGeom<r
     }
     const real bl = a.b[S - 1] * G.dt;
     const real v[3] = {bl * l0, bl * l1, bl * l2};
-    w_part<real, PREC, HSITE>(a.last, a.hs, st, G, v, a.w, a.u, a.gh, a.gjd);
+    w_part<real, PREC, HSITE, LATE>(a.last, a.hs, st, G, v, a.w, a.u, a.gh, a.gjd, a.tj);
 }
 
-template <typename real, bool PREC, bool HSITE, int S, bool CHAIN>
+template <typename real, bool PREC, bool HSITE, int S, bool CHAIN, bool LATE>
 __global__ void __launch_bounds__(kAT) k_adj_top_w(TopArgs<real> a, AdjGeom<real> G) {
     pdl_wait();
     const Site<real> st = site_here<real>(G.nx, G.ny, G.nz, G.bc);
     const int i = st.i;
-    top_body<real, PREC, HSITE, S, CHAIN>(a, G, st, a.lam.c[0][i], a.lam.c[1][i], a.lam.c[2][i]);
+    top_body<real, PREC, HSITE, S, CHAIN, LATE>(a, G, st, a.lam.c[0][i], a.lam.c[1][i], a.lam.c[2][i]);
     pdl_go();
 }
 
@@ -370,12 +443,15 @@ struct XWArgs {
     V3<real> wn, un;     // w, u of stage j-1
     V3<double> gh;       // FP64 field gradient
     double* gjd;         // FP64 per-site dL/dJ (N) and dL/dD (N) terms
+    real* tj;            // stored stages: the stage's terms of those, added after the step
 };
 
-template <typename real, bool PREC, bool HSITE, int NL, bool W, bool CHAIN>
-__global__ void __launch_bounds__(kAT, CHAIN ? SPIN_ADJ_MINB : 1) k_adj_xw(XWArgs<real> a, AdjGeom<real> G) {
+template <typename real, bool PREC, bool HSITE, int NL, bool W, bool CHAIN, bool LATE>
+__global__ void __launch_bounds__(kAT, LATE && W ? SPIN_ADJ_LATEB : CHAIN ? SPIN_ADJ_MINB : 1)
+    k_adj_xw(XWArgs<real> a, StepTerms<real> terms, AdjGeom<real> G) {
     pdl_wait();
     const Site<real> st = site_here<real>(G.nx, G.ny, G.nz, G.bc);
+    if (LATE && NL == 0) add_terms(terms, st, G.N);
     const int i = st.i;
     constexpr int NLOAD = CHAIN ? 1 : (NL > 0 ? NL : 1);
     real ux[3], lm[3], wz, nsum[3], lkv[NLOAD][3];
@@ -418,7 +494,7 @@ __global__ void __launch_bounds__(kAT, CHAIN ? SPIN_ADJ_MINB : 1) k_adj_xw(XWArg
     }
     if (W) {
         const real v[3] = {G.dt * lk[0], G.dt * lk[1], G.dt * lk[2]};
-        w_part<real, PREC, HSITE>(a.prev, a.hs, st, G, v, a.wn, a.un, a.gh, a.gjd);
+        w_part<real, PREC, HSITE, LATE>(a.prev, a.hs, st, G, v, a.wn, a.un, a.gh, a.gjd, a.tj);
     }
     pdl_go();
 }
@@ -429,9 +505,10 @@ __global__ void __launch_bounds__(kAT, CHAIN ? SPIN_ADJ_MINB : 1) k_adj_xw(XWArg
 // step.  For steps whose stages were stored (the top then reads only stored
 // arrays of step m-1).
 template <typename real, bool PREC, bool HSITE, int S, bool CHAIN>
-__global__ void __launch_bounds__(kAT, CHAIN ? SPIN_ADJ_MINB : 1) k_adj_x0_top(XWArgs<real> a, TopArgs<real> ta, AdjGeom<real> G) {
+__global__ void __launch_bounds__(kAT, CHAIN ? SPIN_ADJ_MINB : 1) k_adj_x0_top(XWArgs<real> a, TopArgs<real> ta, StepTerms<real> terms, AdjGeom<real> G) {
     pdl_wait();
     const Site<real> st = site_here<real>(G.nx, G.ny, G.nz, G.bc);
+    add_terms(terms, st, G.N);   // step m's w of the last stage is overwritten below, at this site only
     const int i = st.i;
     real ux[3], lm[3], nsum[3];
 #pragma unroll
@@ -448,7 +525,7 @@ __global__ void __launch_bounds__(kAT, CHAIN ? SPIN_ADJ_MINB : 1) k_adj_x0_top(X
         if (c == 2) lx += G.twoD * wz;
         l[c] = lm[c] + lx;
     }
-    top_body<real, PREC, HSITE, S, CHAIN>(ta, G, st, l[0], l[1], l[2]);
+    top_body<real, PREC, HSITE, S, CHAIN, true>(ta, G, st, l[0], l[1], l[2]);
     pdl_go();
 }
 
@@ -582,82 +659,94 @@ void launch_lincomb(int nk, real* out, const real* s, const LinComb<real>& lc, l
 inline bool adj_tableau_supported(int S, bool chain) { return chain ? (S == 2 || S == 4) : S == 6; }
 
 template <typename real, bool PREC, bool HSITE>
-cudaError_t launch_xw_t(int j, int S, bool chain, const XWArgs<real>& a, const AdjGeom<real>& G, dim3 gb,
-                        cudaStream_t st) {
+cudaError_t launch_xw_t(int j, int S, bool chain, bool late, const XWArgs<real>& a, const StepTerms<real>& t,
+                        const AdjGeom<real>& G, dim3 gb, cudaStream_t st) {
     if (!adj_tableau_supported(S, chain)) return cudaErrorInvalidValue;
-    if (chain) {
-        switch (j) {
-            case 0: return adj_launch(k_adj_xw<real, PREC, HSITE, 0, false, true>, gb, st, a, G);
-            case 1: return adj_launch(k_adj_xw<real, PREC, HSITE, 1, true, true>, gb, st, a, G);
-            case 2: return adj_launch(k_adj_xw<real, PREC, HSITE, 2, true, true>, gb, st, a, G);
-            case 3: return adj_launch(k_adj_xw<real, PREC, HSITE, 3, true, true>, gb, st, a, G);
+    if constexpr (sizeof(real) == 4) {
+        if (late) switch (j) {
+            case 0: return adj_launch(k_adj_xw<real, PREC, HSITE, 0, false, true, true>, gb, st, a, t, G);
+            case 1: return adj_launch(k_adj_xw<real, PREC, HSITE, 1, true, true, true>, gb, st, a, t, G);
+            case 2: return adj_launch(k_adj_xw<real, PREC, HSITE, 2, true, true, true>, gb, st, a, t, G);
+            case 3: return adj_launch(k_adj_xw<real, PREC, HSITE, 3, true, true, true>, gb, st, a, t, G);
             default: return cudaErrorInvalidValue;
         }
-        return cudaSuccess;
     }
-    switch (j) {
-        case 0: return adj_launch(k_adj_xw<real, PREC, HSITE, 0, false, false>, gb, st, a, G);
-        case 1: return adj_launch(k_adj_xw<real, PREC, HSITE, 1, true, false>, gb, st, a, G);
-        case 2: return adj_launch(k_adj_xw<real, PREC, HSITE, 2, true, false>, gb, st, a, G);
-        case 3: return adj_launch(k_adj_xw<real, PREC, HSITE, 3, true, false>, gb, st, a, G);
-        case 4: return adj_launch(k_adj_xw<real, PREC, HSITE, 4, true, false>, gb, st, a, G);
-        case 5: return adj_launch(k_adj_xw<real, PREC, HSITE, 5, true, false>, gb, st, a, G);
+    if (late) return cudaErrorInvalidValue;
+    if (chain) switch (j) {
+        case 0: return adj_launch(k_adj_xw<real, PREC, HSITE, 0, false, true, false>, gb, st, a, t, G);
+        case 1: return adj_launch(k_adj_xw<real, PREC, HSITE, 1, true, true, false>, gb, st, a, t, G);
+        case 2: return adj_launch(k_adj_xw<real, PREC, HSITE, 2, true, true, false>, gb, st, a, t, G);
+        case 3: return adj_launch(k_adj_xw<real, PREC, HSITE, 3, true, true, false>, gb, st, a, t, G);
         default: return cudaErrorInvalidValue;
     }
-    return cudaSuccess;
+    switch (j) {
+        case 0: return adj_launch(k_adj_xw<real, PREC, HSITE, 0, false, false, false>, gb, st, a, t, G);
+        case 1: return adj_launch(k_adj_xw<real, PREC, HSITE, 1, true, false, false>, gb, st, a, t, G);
+        case 2: return adj_launch(k_adj_xw<real, PREC, HSITE, 2, true, false, false>, gb, st, a, t, G);
+        case 3: return adj_launch(k_adj_xw<real, PREC, HSITE, 3, true, false, false>, gb, st, a, t, G);
+        case 4: return adj_launch(k_adj_xw<real, PREC, HSITE, 4, true, false, false>, gb, st, a, t, G);
+        case 5: return adj_launch(k_adj_xw<real, PREC, HSITE, 5, true, false, false>, gb, st, a, t, G);
+        default: return cudaErrorInvalidValue;
+    }
 }
 
 // x-part of stage j and (j > 0) w-part of stage j-1.
 template <typename real>
-cudaError_t launch_xw(bool prec, bool hsite, int j, int S, bool chain, const XWArgs<real>& a, const AdjGeom<real>& G,
-                      dim3 gb, cudaStream_t st) {
+cudaError_t launch_xw(bool prec, bool hsite, int j, int S, bool chain, bool late, const XWArgs<real>& a,
+                      const StepTerms<real>& t, const AdjGeom<real>& G, dim3 gb, cudaStream_t st) {
     if (prec) {
-        if (hsite) return launch_xw_t<real, true, true>(j, S, chain, a, G, gb, st);
-        return launch_xw_t<real, true, false>(j, S, chain, a, G, gb, st);
+        if (hsite) return launch_xw_t<real, true, true>(j, S, chain, late, a, t, G, gb, st);
+        return launch_xw_t<real, true, false>(j, S, chain, late, a, t, G, gb, st);
     }
-    if (hsite) return launch_xw_t<real, false, true>(j, S, chain, a, G, gb, st);
-    return launch_xw_t<real, false, false>(j, S, chain, a, G, gb, st);
+    if (hsite) return launch_xw_t<real, false, true>(j, S, chain, late, a, t, G, gb, st);
+    return launch_xw_t<real, false, false>(j, S, chain, late, a, t, G, gb, st);
 }
 
+// Stored stages (single precision) only.
 template <typename real, bool PREC, bool HSITE>
-cudaError_t launch_x0_top_t(int S, bool chain, const XWArgs<real>& xa, const TopArgs<real>& ta, const AdjGeom<real>& G,
-                            dim3 gb, cudaStream_t st) {
-    if (chain && S == 2) return adj_launch(k_adj_x0_top<real, PREC, HSITE, 2, true>, gb, st, xa, ta, G);
-    else if (chain && S == 4) return adj_launch(k_adj_x0_top<real, PREC, HSITE, 4, true>, gb, st, xa, ta, G);
-    else return cudaErrorInvalidValue;
-    return cudaSuccess;
+cudaError_t launch_x0_top_t(int S, const XWArgs<real>& xa, const TopArgs<real>& ta, const StepTerms<real>& t,
+                            const AdjGeom<real>& G, dim3 gb, cudaStream_t st) {
+    if constexpr (sizeof(real) == 4) {
+        if (S == 2) return adj_launch(k_adj_x0_top<real, PREC, HSITE, 2, true>, gb, st, xa, ta, t, G);
+        if (S == 4) return adj_launch(k_adj_x0_top<real, PREC, HSITE, 4, true>, gb, st, xa, ta, t, G);
+    }
+    return cudaErrorInvalidValue;
 }
 
 template <typename real>
-cudaError_t launch_x0_top(bool prec, bool hsite, int S, bool chain, const XWArgs<real>& xa, const TopArgs<real>& ta,
-                          const AdjGeom<real>& G, dim3 gb, cudaStream_t st) {
+cudaError_t launch_x0_top(bool prec, bool hsite, int S, const XWArgs<real>& xa, const TopArgs<real>& ta,
+                          const StepTerms<real>& t, const AdjGeom<real>& G, dim3 gb, cudaStream_t st) {
     if (prec) {
-        if (hsite) return launch_x0_top_t<real, true, true>(S, chain, xa, ta, G, gb, st);
-        return launch_x0_top_t<real, true, false>(S, chain, xa, ta, G, gb, st);
+        if (hsite) return launch_x0_top_t<real, true, true>(S, xa, ta, t, G, gb, st);
+        return launch_x0_top_t<real, true, false>(S, xa, ta, t, G, gb, st);
     }
-    if (hsite) return launch_x0_top_t<real, false, true>(S, chain, xa, ta, G, gb, st);
-    return launch_x0_top_t<real, false, false>(S, chain, xa, ta, G, gb, st);
+    if (hsite) return launch_x0_top_t<real, false, true>(S, xa, ta, t, G, gb, st);
+    return launch_x0_top_t<real, false, false>(S, xa, ta, t, G, gb, st);
 }
 
 template <typename real, bool PREC, bool HSITE>
-cudaError_t launch_top_w_t(int S, bool chain, const TopArgs<real>& a, const AdjGeom<real>& G, dim3 gb,
+cudaError_t launch_top_w_t(int S, bool chain, bool late, const TopArgs<real>& a, const AdjGeom<real>& G, dim3 gb,
                            cudaStream_t st) {
-    if (chain && S == 2) return adj_launch(k_adj_top_w<real, PREC, HSITE, 2, true>, gb, st, a, G);
-    else if (chain && S == 4) return adj_launch(k_adj_top_w<real, PREC, HSITE, 4, true>, gb, st, a, G);
-    else if (!chain && S == 6) return adj_launch(k_adj_top_w<real, PREC, HSITE, 6, false>, gb, st, a, G);
-    else return cudaErrorInvalidValue;
-    return cudaSuccess;
+    if constexpr (sizeof(real) == 4) {
+        if (late && chain && S == 2) return adj_launch(k_adj_top_w<real, PREC, HSITE, 2, true, true>, gb, st, a, G);
+        if (late && chain && S == 4) return adj_launch(k_adj_top_w<real, PREC, HSITE, 4, true, true>, gb, st, a, G);
+    }
+    if (late) return cudaErrorInvalidValue;
+    if (chain && S == 2) return adj_launch(k_adj_top_w<real, PREC, HSITE, 2, true, false>, gb, st, a, G);
+    if (chain && S == 4) return adj_launch(k_adj_top_w<real, PREC, HSITE, 4, true, false>, gb, st, a, G);
+    if (!chain && S == 6) return adj_launch(k_adj_top_w<real, PREC, HSITE, 6, false, false>, gb, st, a, G);
+    return cudaErrorInvalidValue;
 }
 
 template <typename real>
-cudaError_t launch_top_w(bool prec, bool hsite, int S, bool chain, const TopArgs<real>& a, const AdjGeom<real>& G,
-                         dim3 gb, cudaStream_t st) {
+cudaError_t launch_top_w(bool prec, bool hsite, int S, bool chain, bool late, const TopArgs<real>& a,
+                         const AdjGeom<real>& G, dim3 gb, cudaStream_t st) {
     if (prec) {
-        if (hsite) return launch_top_w_t<real, true, true>(S, chain, a, G, gb, st);
-        return launch_top_w_t<real, true, false>(S, chain, a, G, gb, st);
+        if (hsite) return launch_top_w_t<real, true, true>(S, chain, late, a, G, gb, st);
+        return launch_top_w_t<real, true, false>(S, chain, late, a, G, gb, st);
     }
-    if (hsite) return launch_top_w_t<real, false, true>(S, chain, a, G, gb, st);
-    return launch_top_w_t<real, false, false>(S, chain, a, G, gb, st);
+    if (hsite) return launch_top_w_t<real, false, true>(S, chain, late, a, G, gb, st);
+    return launch_top_w_t<real, false, false>(S, chain, late, a, G, gb, st);
 }
 
 template <typename real>
@@ -735,6 +824,11 @@ cudaError_t adjoint_run(const AdjointRun<real>& A) {
     auto stage_x = [&](int j, int m) { return slot_arr(m, j - 2); };           // X_j, j = 2..S
     auto stage_sn = [&](int j, int m) { return slot_arr(m, S - 1 + j - 1); };  // sum_nn X_j, j = 1..S
     auto stage_y = [&](int m) { return slot_arr(m, 2 * S - 1); };
+    // stored stages: w of every stage and its dL/dJ and dL/dD terms stay until
+    // the step's end (w in the first pair's arrays and in the lam_K ones that
+    // chain tableaus leave free, the terms in the unused K_j)
+    const bool late = stored && tb.chain;
+    auto wbuf = [&](int j) { return late ? (j < 2 ? wb[j] : LK[j - 1]) : wb[j & 1]; };
     cudaStream_t st = A.stream;
     const real* hs = A.h_site;
     const bool HS = hs != nullptr;
@@ -753,6 +847,14 @@ cudaError_t adjoint_run(const AdjointRun<real>& A) {
     G.H[2] = (real)A.H[2];
     G.lambda = (real)A.lambda;
     G.dt = (real)A.dt;
+    StepTerms<real> terms{};
+    for (int j = 0; late && j < S; ++j) {
+        terms.w[j] = cv3<real>(wbuf(j), N);
+        terms.t[j] = Kst[j];
+    }
+    terms.stages = S;
+    terms.gh = gh3;
+    terms.gjd = gjd;
     cudaError_t e;
 
     // seed from the final state (component arrays of the caller)
@@ -839,7 +941,8 @@ cudaError_t adjoint_run(const AdjointRun<real>& A) {
             ta.sigma = (real)A.sigma;
             ta.last = in[S - 1];
             ta.hs = hs3;
-            ta.w = v3<real>(wb[(S - 1) & 1], N);
+            ta.w = v3<real>(wbuf(S - 1), N);
+            ta.tj = late ? Kst[S - 1] : nullptr;
             ta.u = v3<real>(ub[(S - 1) & 1], N);
             ta.gh = gh3;
             ta.gjd = gjd;
@@ -847,7 +950,7 @@ cudaError_t adjoint_run(const AdjointRun<real>& A) {
         };
         auto xw_args = [&](int j, const StageIn<real>* in) {
             XWArgs<real> xa{};
-            xa.w = cv3<real>(wb[j & 1], N);
+            xa.w = cv3<real>(wbuf(j), N);
             xa.u = cv3<real>(ub[j & 1], N);
             xa.lam = v3<real>(lam, N);
             for (int l = 0; l < j; ++l) {
@@ -858,7 +961,8 @@ cudaError_t adjoint_run(const AdjointRun<real>& A) {
             xa.bl = j > 0 ? (real)tb.b[j - 1] : real(0);
             if (j > 0) {
                 xa.prev = in[j - 1];
-                xa.wn = v3<real>(wb[(j - 1) & 1], N);
+                xa.wn = v3<real>(wbuf(j - 1), N);
+                xa.tj = late ? Kst[j - 1] : nullptr;
                 xa.un = v3<real>(ub[(j - 1) & 1], N);
             }
             xa.hs = hs3;
@@ -866,7 +970,6 @@ cudaError_t adjoint_run(const AdjointRun<real>& A) {
             xa.gjd = gjd;
             return xa;
         };
-        const bool fuse_top = stored && tb.chain;
         for (int m = seglen; m >= 1; --m) {
             const real* s = seg + (size_t)(m - 1) * len;
             StageIn<real> in[6];
@@ -890,20 +993,21 @@ cudaError_t adjoint_run(const AdjointRun<real>& A) {
                     else k_adj_rhs<real, false, false><<<gb, kAT, 0, st>>>(in[j].x, hs3, K3, G);
                 }
             }
-            if (!fuse_top || m == seglen) {
+            if (!late || m == seglen) {
                 const TopArgs<real> ta = top_args(m, in);
-                if ((e = launch_top_w<real>(A.precession != 0, HS, S, tb.chain, ta, G, gb, st)) != cudaSuccess)
+                if ((e = launch_top_w<real>(A.precession != 0, HS, S, tb.chain, late, ta, G, gb, st)) != cudaSuccess)
                     return e;
             }
             for (int j = S - 1; j >= 0; --j) {
                 const XWArgs<real> xa = xw_args(j, in);
-                if (j == 0 && fuse_top && m > 1) {
+                if (j == 0 && late && m > 1) {
                     StageIn<real> inp[6];
                     stage_inputs(m - 1, inp);
                     const TopArgs<real> ta = top_args(m - 1, inp);
-                    if ((e = launch_x0_top<real>(A.precession != 0, HS, S, tb.chain, xa, ta, G, gb, st)) != cudaSuccess)
+                    if ((e = launch_x0_top<real>(A.precession != 0, HS, S, xa, ta, terms, G, gb, st)) != cudaSuccess)
                         return e;
-                } else if ((e = launch_xw<real>(A.precession != 0, HS, j, S, tb.chain, xa, G, gb, st)) != cudaSuccess) {
+                } else if ((e = launch_xw<real>(A.precession != 0, HS, j, S, tb.chain, late, xa, terms, G, gb, st)) !=
+                           cudaSuccess) {
                     return e;
                 }
             }

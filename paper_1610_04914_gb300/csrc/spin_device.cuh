@@ -206,6 +206,24 @@ struct Math<double> {
     __device__ __forceinline__ static void sincos_(double x, double* s, double* c) { sincos(x, s, c); }
 };
 
+// S 2^(emax - 1082) rounded once to nearest, with integer operations (an FP64
+// instruction or conversion takes as long as some sixty of them); emax is such
+// that the result is a normal number.
+__device__ __forceinline__ double from_fixed(long long S, unsigned emax) {
+    const long long sg = S >> 63;
+    const unsigned long long a = (unsigned long long)((S ^ sg) - sg);
+    const int lz = __clzll((long long)a);
+    const unsigned long long n = a << lz;      // leading bit at 63
+    unsigned long long r = n >> 11;
+    const unsigned rem = (unsigned)n & 0x7FFu;
+    r += (rem > 0x400u || (rem == 0x400u && (r & 1ULL))) ? 1ULL : 0ULL;
+    // leading bit of a at bit 63 - lz: biased exponent emax + 4 - lz, of which
+    // the mantissa's leading bit adds one
+    r += (unsigned long long)(emax + 3u - (unsigned)lz) << 52;
+    r |= (unsigned long long)sg & 0x8000000000000000ULL;
+    return a == 0ULL ? 0.0 : __longlong_as_double((long long)r);
+}
+
 // sin(phi)/phi and (1 - cos(phi))/phi^2 for p = phi^2 <= kSmallPhi2: the Taylor
 // series in p, truncated below the type's rounding (the first omitted terms are
 // p^7/15! = 1.3e-8 and p^11/23! = 1.6e-16 at p = 4).

@@ -67,20 +67,6 @@ __device__ __forceinline__ long long fixed(double v, unsigned emax) {
     const long long sg = (long long)((int)h >> 31);
     return (x ^ sg) - sg;
 }
-__device__ __forceinline__ double from_fixed(long long S, unsigned emax) {
-    const long long sg = S >> 63;
-    const unsigned long long a = (unsigned long long)((S ^ sg) - sg);
-    const int lz = __clzll((long long)a);
-    const unsigned long long n = a << lz;      // leading bit at 63
-    unsigned long long r = n >> 11;
-    const unsigned rem = (unsigned)n & 0x7FFu;
-    r += (rem > 0x400u || (rem == 0x400u && (r & 1ULL))) ? 1ULL : 0ULL;
-    // leading bit of a at bit 63 - lz: biased exponent emax + 4 - lz, of which
-    // the mantissa's leading bit adds one
-    r += (unsigned long long)(emax + 3u - (unsigned)lz) << 52;
-    r |= (unsigned long long)sg & 0x8000000000000000ULL;
-    return a == 0ULL ? 0.0 : __longlong_as_double((long long)r);
-}
 // Kept out of line: inlined, the compiler would execute it for every site.
 __device__ __noinline__ double plain_sum6(double a, double b, double c, double d, double e, double f) {
     return ((a + b) + (c + d)) + (e + f);

@@ -6,7 +6,7 @@ import pytest
 import torch
 
 import spin_inputs
-from gpu_helpers import run_gpu, run_oracle
+from gpu_helpers import as_input, orc_params, run_gpu, run_oracle
 
 pytestmark = pytest.mark.gpu
 
@@ -268,3 +268,42 @@ def test_sample_ring_wraps_and_long_graphs(gpu):
     assert torch.equal(a.state, b.state)
     want = b.samples()[-9:]
     assert len(got) == 9 and got == want and got[-1][0] == 2.0 * (ring + 8)
+
+
+# FP32 gradients whose step terms are added once per step: the order of the
+# additions does not depend on the segments, so every K gives the same bits
+# (segments of one step, a short last segment, one segment); against the oracle
+# with the bounds of test_gpu_adjoint.py; terms of very different size and
+# underflowing ones (a loss scaled by 1e-34); a lattice of several blocks with
+# idle lanes and rows
+@pytest.mark.parametrize("integ,precession", [("RK4", 1), ("RK2_MIDPOINT", 1), ("HEUN", 0)])
+def test_adjoint_step_terms(gpu, orc, integ, precession):
+    shape, nsteps = (33, 9, 3), 7
+    p = gpu.Params(*shape, J=0.9, D=0.25, H=(0.05, -0.1, 0.2), lam=0.1, T=0.8, dt=0.1, R=3, seed=12, precision=32,
+                   integrator=getattr(gpu, integ), precession=precession)
+    s0 = spin_inputs.random_spins(*shape, seed=11)
+    hs = spin_inputs.site_fields(*shape, 0.1, seed=13)
+
+    def grad(K, scale=1.0):
+        lat = gpu.Lattice(p, torch.from_numpy(s0), h_site=torch.from_numpy(hs))
+        lat.record(K, nsteps)
+        lat.step(nsteps)
+        g = lat.backward([0.3 * scale, -0.2 * scale, 0.7 * scale], scale, field_grad=True, state_grad=True)
+        return np.concatenate([[g["J"], g["D"]], g["H"], g["h"].cpu().numpy().ravel(),
+                               g["s0"].double().cpu().numpy().ravel()])
+
+    got = grad(3)
+    assert np.array_equal(got, grad(1)) and np.array_equal(got, grad(7))
+    ref = orc.adjoint(orc_params(orc, p), as_input(p, s0), nsteps, [0.3, -0.2, 0.7], 1.0, h_site=as_input(p, hs))
+    parts = [[ref["J"], ref["D"]], ref["H"], ref["h"], ref["s0"]]
+    at = 0
+    for r in parts:
+        r = np.asarray(r, float).ravel()
+        d = got[at:at + r.size] - r
+        assert np.max(np.abs(d)) < 1e-5 * np.max(np.abs(r))
+        at += r.size
+    # scaled by 1e-34 the per-site terms lie below 2^-126 (subnormal, spacing
+    # 2^-149): each of the adjoint's roundings is then absolute
+    tiny = grad(3, 1e-34)
+    n = 5 + 3 * 33 * 9 * 3
+    assert np.max(np.abs(tiny[5:n] - 1e-34 * got[5:n])) < 1e-5 * np.max(np.abs(1e-34 * got[5:n])) + 400 * 2.0 ** -149
