@@ -76,7 +76,9 @@ typedef struct spin_params {
                                  SPIN_EUNSUPPORTED) */
     int32_t replica;          /* replica number, third word of the noise counter */
     int32_t path;             /* 0: fused single-kernel step where the tableau allows
-                                 (RK4, RK2 midpoint, Heun), else per-stage kernels;
+                                 (RK4, RK2 midpoint, Heun; FP64 and small FP32
+                                 lattices: one kernel per stage, the same states
+                                 bit for bit in FP32), else per-stage kernels;
                                  1: per-stage kernels always (cross-check path) */
     int32_t bc;               /* 0: periodic boundaries; 1: free boundaries (the paper's
                                  particle, Sec. IV): a site on a face has no neighbour
@@ -95,8 +97,9 @@ typedef struct spin_lattice spin_lattice;
 
 /*
  * Bytes of workspace a handle for *p needs.  Layout (internal): a second state
- * buffer for the out-of-place stencil update, stage temporaries for
- * multi-kernel integrators, FP64 reduction partials, the device-resident
+ * buffer for the out-of-place stencil update, stage temporaries where a step
+ * is several kernels (FP64: 6N values for RK4, 3N for the two-stage tableaus;
+ * small FP32 lattices; RK5), FP64 reduction partials, the device-resident
  * interval counter and the sample ring.
  * Errors: SPIN_EINVAL for a null pointer or invalid parameters.
  */
@@ -127,8 +130,8 @@ int spin_lattice_create(const spin_params* p, void* sx, void* sy, void* sz,
  * the pulse number floor((n-1)/R) is applied when n mod R == floor(R/2)
  * (Eq. ST-expansion: mid-interval; every step when R = 1), and the
  * observables are sampled into the sample ring when n mod R == 0 (Sec. III.A:
- * values at the end of each Delta t).  Full intervals are replayed from a
- * cached CUDA graph.  On return (stream-ordered) the caller's arrays hold the
+ * values at the end of each Delta t).  Full intervals are replayed from cached
+ * CUDA graphs, on lattices of up to 2^20 sites several intervals per graph.  On return (stream-ordered) the caller's arrays hold the
  * state after the last step.
  * Kernel choice for FP32 RK4 steps (all give bitwise the same states): the
  * register-ring fused step, or, where its wave-cost estimate is lower (large
@@ -195,9 +198,9 @@ int spin_record_end(spin_lattice* h);
  * The backward pass restores each checkpoint, recomputes its K steps with
  * the forward kernels and runs the transposed steps backwards.  For FP32
  * states with a chain tableau (RK4, RK2 midpoint, Heun) on the fused path the
- * recomputing steps also write every stage's input and increment, which the
- * transposed steps read instead of recomputing them; the workspace then holds
- * (2 x stages - 1) x K extra arrays of 3N values (taken only while they come
+ * recomputing steps also write every stage's input and neighbour sum and the
+ * unnormalised result, which the transposed steps read instead of recomputing
+ * them; the workspace then holds 2 x stages x K extra arrays of 3N values (taken only while they come
  * to at most 8 GiB; otherwise the stages are recomputed per step).
  *   dLdM, dLdE   host seeds of the loss
  *   workspace    device, >= spin_backward_workspace_size(p, K) bytes, 256-aligned
@@ -207,8 +210,9 @@ int spin_record_end(spin_lattice* h);
  *   g_s0         nullable device array of 3N (state type): dL/ds_{n0}
  * Parameter gradients accumulate in FP64: every site's term of every stage of
  * every step is formed in the state precision and added in FP64 (dL/dh_i
- * straight into g_h_site; dL/dJ, dL/dD, dL/dH through FP64 per-thread sums
- * reduced in FP64).  The adjoint state is kept in the state precision.
+ * straight into g_h_site; dL/dJ, dL/dD per site, all three then summed over the
+ * sites in FP64; where stages are stored, the terms of one step are first added
+ * to each other without rounding).  The adjoint state is kept in the state precision.
  * Synchronises the stream.
  * Errors: SPIN_EINVAL (no recording, range mismatch), SPIN_ENOSPACE, SPIN_ECUDA.
  */

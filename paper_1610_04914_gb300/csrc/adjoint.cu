@@ -109,11 +109,6 @@ __device__ __forceinline__ Site<real> site_here(int nx, int ny, int nz, int bc) 
     return s;
 }
 
-// Record of this block in the per-block partial sums.
-__device__ __forceinline__ int block_record() {
-    return (int)(blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z));
-}
-
 // Component arrays (x, y, z blocks of a 3N array).
 template <typename real>
 struct V3 {
