@@ -206,6 +206,19 @@ struct Math<double> {
     __device__ __forceinline__ static void sincos_(double x, double* s, double* c) { sincos(x, s, c); }
 };
 
+// 1/sqrt(x) from the FP32 reciprocal root of x cut to 24 bits and one
+// third-order step, as in Gauss<double>::root: five FP64 instructions.  Outside
+// the normal floats' range (zero, infinite and NaN arguments among it) the
+// library's, out of line so that it is not executed for every site.
+static __device__ __noinline__ double plain_rsqrt(double x) { return rsqrt(x); }
+__device__ __forceinline__ double inv_root(double x) {
+    const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x);
+    if (h - 0x38100000u >= 0x0FE00000u) return plain_rsqrt(x);
+    const double g = to_f64(rsqrtf(__uint_as_float(((h - 0x38000000u) << 3) | (l >> 29))));
+    const double d = fma(-(x * g), g, 1.0);
+    return fma(g * d, fma(0.375, d, 0.5), g);
+}
+
 // S 2^(emax - 1082) rounded once to nearest, with integer operations (an FP64
 // instruction or conversion takes as long as some sixty of them); emax is such
 // that the result is a normal number.

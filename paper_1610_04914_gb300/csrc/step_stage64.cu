@@ -11,8 +11,9 @@
 // computed exactly once, and the stage inputs X_j go through memory.  RK4,
 // one interval: 128^3 (4 steps, one pulse) 16.08 -> 3.60 ms, 16^3 (10 steps,
 // one pulse, observables) 2.09 -> 0.25 ms; with the sums below off the FP64
-// pipe and the cheaper noise draw 1.97 and 0.23 ms; the pipe is then 85%
-// active at 128^3.  16^3 with four lanes per site: 0.18 ms.
+// pipe and the cheaper noise draw 1.97 and 0.23 ms, with the products
+// folded into the update and a short reciprocal root 1.86 ms; the pipe is then
+// 85% active at 128^3.  16^3 with four lanes per site: 0.175 ms.
 //
 // The accumulator of the tableau is not kept: with K_j = dt f(X_j) and
 // X_{j+1} = s + a_{j+1,j} K_j, every K_j but the last is (X_{j+1} - s)/a_{j+1,j},
@@ -39,8 +40,10 @@ struct Stage64Args {
     const double* hs[3];
     double* out[3];        // X_{j+1}, or the new state
     int nx, ny, nz, N;
-    double J, twoD, H[3], lambda;
-    double c;              // dt a_{j+1,j}; last stage: dt b_S
+    // J, 2D, H and the factor of h_i times c = dt a_{j+1,j} (last stage: dt b_S,
+    // of S = 4 thrice that), slow equation: times -c lambda
+    double J, twoD, H[3], hc, lambda;
+    double unscale;        // last stage without renormalisation: factor of the result
     double g0, gx;         // last stage of S = 2: weights of s and X_2
     int bc, renorm;
     int pdl;   // host: launch as a programmatic dependent
@@ -94,12 +97,15 @@ __device__ __forceinline__ double rk4_sum(double x2, double x3, double x4, doubl
 
 enum StageRole { kFirst, kMiddle, kLast2, kLast4 };
 
-// WIDE: sums through the integer pipes, for lattices that fill the FP64 pipe
+// With h = c H_eff (c folded into the constants), c f = v x (h - lambda v x h),
+// c f = v x (v x h) for the slow equation, and the second product is added to
+// the state by its own multiply-adds: 15 FP64 instructions after the field, 18
+// when the two products, their sum and the update are taken one by one.
+
+// WIDE: neighbour sums through the integer pipes, for lattices that fill the FP64 pipe
 // (smaller ones wait on latencies instead, of which the integer form has more:
-// 16^3 242 against 250 us for 10 steps).  UNITX: J = 1 and the uniform
-// field along z without site fields, so that H_x and H_y are the bare neighbour
-// sums (the products and sums with 1 and 0 would be two more instructions).
-template <int ROLE, bool PREC, bool HSITE, bool PULSE, bool WIDE, bool UNITX>
+// 16^3 242 against 250 us for 10 steps).
+template <int ROLE, bool PREC, bool HSITE, bool PULSE, bool WIDE>
 __global__ void __launch_bounds__(128) k_stage64(const __grid_constant__ Stage64Args a) {
     pdl_go();
     const unsigned iu = blockIdx.x * blockDim.x + threadIdx.x;   // N < 2^31, the last block may pass it
@@ -125,33 +131,32 @@ __global__ void __launch_bounds__(128) k_stage64(const __grid_constant__ Stage64
                               fy1 ? 0.0 : q[yp], fz0 ? 0.0 : q[zm], fz1 ? 0.0 : q[zp]};
         s[c] = ROLE == kFirst ? v[c] : a.s[c][i];
         const double sum = WIDE ? sum6(nb) : ((nb[0] + nb[1]) + (nb[2] + nb[3])) + (nb[4] + nb[5]);
-        h[c] = UNITX && c < 2 ? sum : a.J * sum + a.H[c];
-        if (HSITE) h[c] += a.hs[c][i];
+        h[c] = fma(a.J, sum, a.H[c]);
+        if (HSITE) h[c] = fma(a.hc, a.hs[c][i], h[c]);
     }
-    h[2] += a.twoD * v[2];
-    double f[3];
-    llg_rhs<double, PREC>(v[0], v[1], v[2], h[0], h[1], h[2], a.lambda, f[0], f[1], f[2]);
+    h[2] = fma(a.twoD, v[2], h[2]);
+    double g[3] = {v[1] * h[2] - v[2] * h[1], v[2] * h[0] - v[0] * h[2], v[0] * h[1] - v[1] * h[0]};
+    if (PREC) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) g[c] = fma(-a.lambda, g[c], h[c]);
+    }
     double o[3];
-    if (ROLE == kFirst || ROLE == kMiddle) {
 #pragma unroll
-        for (int c = 0; c < 3; ++c) o[c] = s[c] + a.c * f[c];
-    } else {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            double acc;
-            if (ROLE == kLast4) {
-                const double x2 = a.q[0][c][i], x3 = a.q[1][c][i];
-                acc = (1.0 / 3.0) * (WIDE ? rk4_sum(x2, x3, v[c], s[c]) : (x2 + 2.0 * x3) + (v[c] - s[c]));
-            } else {
-                acc = a.g0 * s[c] + a.gx * v[c];
-            }
-            o[c] = acc + a.c * f[c];
+    for (int c = 0; c < 3; ++c) {
+        double base = s[c];
+        if (ROLE == kLast4) {   // three times the result
+            const double x2 = a.q[0][c][i], x3 = a.q[1][c][i];
+            base = rk4_sum(x2, x3, v[c], s[c]);
+        } else if (ROLE == kLast2) {
+            base = a.g0 * s[c] + a.gx * v[c];
         }
-        if (a.renorm) {
-            const double inv = rsqrt(o[0] * o[0] + o[1] * o[1] + o[2] * o[2]);
+        const int d = (c + 1) % 3, e = (c + 2) % 3;
+        o[c] = fma(v[d], g[e], fma(-v[e], g[d], base));
+    }
+    if (ROLE == kLast2 || ROLE == kLast4) {
+        const double inv = a.renorm ? inv_root(o[0] * o[0] + o[1] * o[1] + o[2] * o[2]) : a.unscale;
 #pragma unroll
-            for (int c = 0; c < 3; ++c) o[c] *= inv;
-        }
+        for (int c = 0; c < 3; ++c) o[c] *= inv;
         if (PULSE)
             pulse_site<double>(o[0], o[1], o[2], a.seed, (uint64_t)i, (uint64_t)*a.interval, a.replica, a.sigma);
     }
@@ -162,13 +167,13 @@ __global__ void __launch_bounds__(128) k_stage64(const __grid_constant__ Stage64
 // The smallest lattices: four lanes per site, one component each (the fourth
 // repeats the third).  A warp's FP64 instruction takes 64 cycles of its
 // scheduler whatever its active lanes, and with a warp or two per scheduler a
-// stage lasts as long as the 37 FP64 instructions of one warp; split by
-// component a lane executes 13 (the pulse: half).  The other components' spins,
-// fields and cross products come by shuffles, the numbers are those of
+// stage lasts as long as the FP64 instructions of one warp, 34 with plain sums;
+// split by component a lane executes 12 (the pulse: half).  The other components' spins,
+// fields and cross products come by shuffles, the arithmetic is that of
 // k_stage64.  What is left is the launch and the loads: 2.5 us per stage.  Ten
 // RK4 steps with a pulse and one launch graph, one thread per site against four
-// lanes: 8^3 146 and 100 us, 16^3 150 and 109, 21^3 156 and 139, 22^3 162 and
-// 144, 24^3 158 and 166; two stages: 21^3 88 and 82, 24^3 88 and 98.
+// lanes: 8^3 146 and 99 us, 16^3 150 and 107, 21^3 156 and 135, 22^3 162 and
+// 137, 24^3 156 and 166; two stages: 21^3 88 and 80, 24^3 87 and 98.
 constexpr int kLaneSites = 152 * 72;
 __device__ __forceinline__ double lane_get(double v, int lane) { return __shfl_sync(0xffffffffu, v, lane); }
 
@@ -213,23 +218,20 @@ __global__ void __launch_bounds__(32) k_stage64_lanes(const __grid_constant__ St
         Gauss<double>::angle(c == 2 ? w.w[3] : w.w[1], cs, sn);
         p = a.sigma * (r * (c == 1 ? sn : cs));
     }
-    double h = a.J * (((n[0] + n[1]) + (n[2] + n[3])) + (n[4] + n[5])) + Hc;
-    if (HSITE) h += hs;
-    h += a.twoD * (c == 2 ? v : 0.0);
+    double h = fma(a.J, ((n[0] + n[1]) + (n[2] + n[3])) + (n[4] + n[5]), Hc);
+    if (HSITE) h = fma(a.hc, hs, h);
+    h = fma(a.twoD, c == 2 ? v : 0.0, h);
     const double v1 = lane_get(v, l1), v2 = lane_get(v, l2);
-    const double A = v1 * lane_get(h, l2) - v2 * lane_get(h, l1);
-    const double B = v1 * lane_get(A, l2) - v2 * lane_get(A, l1);
-    const double f = PREC ? A - a.lambda * B : -a.lambda * B;
-    double o;
-    if (ROLE == kFirst || ROLE == kMiddle) {
-        o = s + a.c * f;
-    } else {
-        const double acc = ROLE == kLast4 ? (1.0 / 3.0) * ((x2 + 2.0 * x3) + (v - s)) : a.g0 * s + a.gx * v;
-        o = acc + a.c * f;
-        if (a.renorm) {
-            const double sq = o * o;
-            o *= rsqrt((lane_get(sq, first) + lane_get(sq, first + 1)) + lane_get(sq, first + 2));
-        }
+    double g = v1 * lane_get(h, l2) - v2 * lane_get(h, l1);
+    if (PREC) g = fma(-a.lambda, g, h);
+    double base = s;
+    if (ROLE == kLast4) base = rk4_sum(x2, x3, v, s);
+    if (ROLE == kLast2) base = a.g0 * s + a.gx * v;
+    double o = fma(v1, lane_get(g, l2), fma(-v2, lane_get(g, l1), base));
+    if (ROLE == kLast2 || ROLE == kLast4) {
+        const double sq = o * o;
+        const double n2 = (lane_get(sq, first) + lane_get(sq, first + 1)) + lane_get(sq, first + 2);
+        o *= a.renorm ? inv_root(n2) : a.unscale;
         if (PULSE) {
             double s0 = lane_get(o, first), s1 = lane_get(o, first + 1), s2 = lane_get(o, first + 2);
             pulse_rotate<double>(s0, s1, s2, lane_get(p, first), lane_get(p, first + 1), lane_get(p, first + 2), a.sigma);
@@ -247,12 +249,8 @@ cudaError_t stage_launch(const Stage64Args& a, cudaStream_t st) {
     // up to one warp per scheduler: one warp per block, spread over the SMs
     const bool wide = a.N > 152 * 4 * 32;
     const dim3 block(wide ? 128 : 32), grid((unsigned)(((unsigned)a.N + block.x - 1) / block.x));
-    const bool unitx = !HSITE && a.J == 1.0 && a.H[0] == 0.0 && a.H[1] == 0.0;
-    if (wide)
-        return unitx ? launch_pdl(a.pdl != 0, k_stage64<ROLE, PREC, HSITE, PULSE, true, !HSITE>, grid, block, 0, st, a)
-                     : launch_pdl(a.pdl != 0, k_stage64<ROLE, PREC, HSITE, PULSE, true, false>, grid, block, 0, st, a);
-    return unitx ? launch_pdl(a.pdl != 0, k_stage64<ROLE, PREC, HSITE, PULSE, false, !HSITE>, grid, block, 0, st, a)
-                 : launch_pdl(a.pdl != 0, k_stage64<ROLE, PREC, HSITE, PULSE, false, false>, grid, block, 0, st, a);
+    return wide ? launch_pdl(a.pdl != 0, k_stage64<ROLE, PREC, HSITE, PULSE, true>, grid, block, 0, st, a)
+                : launch_pdl(a.pdl != 0, k_stage64<ROLE, PREC, HSITE, PULSE, false>, grid, block, 0, st, a);
 }
 
 template <int ROLE, bool PULSE>
@@ -283,8 +281,6 @@ cudaError_t launch_step_stage64(const StepLaunch<double>& L) {
     a.ny = L.g.ny;
     a.nz = L.g.nz;
     a.N = (int)N;
-    a.J = L.ph.J;
-    a.twoD = L.ph.twoD;
     a.lambda = L.ph.lambda;
     a.bc = L.bc;
     a.renorm = L.renorm;
@@ -294,11 +290,17 @@ cudaError_t launch_step_stage64(const StepLaunch<double>& L) {
     a.sigma = L.sigma;
     a.interval = L.d_interval;
     for (int c = 0; c < 3; ++c) {
-        a.H[c] = L.ph.H[c];
         a.hs[c] = L.hs[c];
         a.s[c] = L.in[c];
     }
     const bool prec = L.precession != 0, hs = L.hs[0] != nullptr;
+    auto scale = [&](double c) {
+        const double k = prec ? c : -c * L.ph.lambda;
+        a.J = k * L.ph.J;
+        a.twoD = k * L.ph.twoD;
+        for (int q = 0; q < 3; ++q) a.H[q] = k * L.ph.H[q];
+        a.hc = k;
+    };
     if (S == 4 && !rk4_weights(tb)) return cudaErrorInvalidValue;
     // stage 1 .. S-1 write X_2 .. X_S, of S = 4 the first into the output array
     auto scratch = [&](int q, int c) { return L.tmp + ((size_t)q * 3 + c) * N; };
@@ -310,11 +312,12 @@ cudaError_t launch_step_stage64(const StepLaunch<double>& L) {
         }
         cudaError_t e;
         if (j < S) {
-            a.c = tb.a[j][j - 1] * L.dt;
+            scale(tb.a[j][j - 1] * L.dt);
             e = j == 1 ? stage_dispatch<kFirst, false>(a, L.stream, prec, hs)
                        : stage_dispatch<kMiddle, false>(a, L.stream, prec, hs);
         } else {
-            a.c = tb.b[S - 1] * L.dt;
+            scale((S == 4 ? 3.0 : 1.0) * tb.b[S - 1] * L.dt);
+            a.unscale = S == 4 ? 1.0 / 3.0 : 1.0;
             a.gx = tb.b[0] / tb.a[1][0];
             a.g0 = 1.0 - a.gx;
             if (S == 4) {

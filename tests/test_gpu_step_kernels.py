@@ -48,6 +48,21 @@ def test_fp64_component_lanes(gpu, orc, integ, shape, precession, hsite, bc):
              precession=precession, bc=bc)
 
 
+# the last FP64 stage without renormalisation (its result scaled back), and
+# spins of 1e-30, whose squared length lies outside the range of the short
+# reciprocal root; four lanes, one thread per site, and the integer sums
+@pytest.mark.parametrize("integ,precession", [("RK4", 1), ("RK2_MIDPOINT", 0)])
+@pytest.mark.parametrize("shape", [(7, 6, 5), (23, 22, 24), (28, 27, 26)])
+@pytest.mark.parametrize("renorm,scale", [(0, 1.0), (1, 1e-30)])
+def test_fp64_last_stage_forms(gpu, orc, integ, precession, shape, renorm, scale):
+    p = gpu.Params(*shape, J=0.9, D=0.15, H=(0.05, -0.1, 0.2), lam=0.1, T=0.7, dt=0.07, R=3, seed=77, replica=2,
+                   precision=64, renorm=renorm, integrator=getattr(gpu, integ), precession=precession)
+    s0 = scale * spin_inputs.random_spins(*shape, seed=3)
+    got, _ = run_gpu(gpu, p, s0, 3)
+    ref, _ = run_oracle(orc, p, s0, 3)
+    assert np.max(np.abs(got - ref)) < 1e-13
+
+
 # free spins (J = D = H = 0): three pulses with sigma at both sides of the
 # series limit 0.35, far above it (general form), and angles from ~0 to beyond
 # phi^2 = 4.  Per pulse the angle carries about four roundings of G, relative,
