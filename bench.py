@@ -718,7 +718,7 @@ def fp64_step_timing(sp, torch, dev, flush, stream):
     torch.cuda.synchronize()
     ms = float(np.mean([a.elapsed_time(c) for a, c in ev]))
     lat.close()
-    return {"lattice": "128^3 FP64 RK4 (fused FP64 kernel)", "kernel_ms_per_launch": ms,
+    return {"lattice": "128^3 FP64 RK4 (one kernel per stage)", "kernel_ms_per_launch": ms,
             "spin_steps_per_s": p.N / (ms / 1e3)}
 
 
