@@ -2,9 +2,10 @@
 // while the kernel before it on the stream drains (or, where that one calls
 // pdl_go, as soon as all of its blocks have started); it calls pdl_wait before
 // it touches memory that an earlier kernel writes or reads.  pdl_wait returns
-// when the kernel before has finished and its writes are visible.  A kernel
-// that calls pdl_go after its own pdl_wait also promises its successor that
-// everything before it has finished.
+// when the kernel before has finished and its writes are visible.  Nothing that
+// an earlier kernel on the stream writes may be relied on before that, not even
+// what the kernel before the last one wrote (some kernels call pdl_go before
+// their own pdl_wait).
 //
 // In interval graphs the kernels get ordinary edges, with one exception.
 // Programmatic edges between graph nodes gained nothing or cost time (an interval of 96 replicas 2048 -> 2133 us, RK5 at 128^3 1108 -> 1148,
@@ -21,6 +22,14 @@ namespace spin {
 
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 __device__ __forceinline__ void pdl_go() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+
+// A word that an earlier kernel on the stream writes, read without the
+// non-coherent cache.  Before pdl_wait its value may be an old one.
+__device__ __forceinline__ unsigned long long load_shared_word(const long long* p) {
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];\n" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
 
 constexpr long long kPdlGraphSites = 1LL << 20;
 

@@ -187,19 +187,28 @@ cudaError_t patch_dispatch(const PatchArgs& a, dim3 grid, cudaStream_t st, bool 
 //
 // The draw does not depend on the state: the kernel is launched while the step
 // before it drains and each thread draws for its first site before it waits.
+// The pulse number it draws with then is a guess, loaded where nothing yet
+// promises that an earlier kernel's write of it is visible; the number counts
+// as read only after the wait, and a draw made with another one is made again.
 // The state may go to other arrays (odd intervals, spin_api.cu).
 __global__ void __launch_bounds__(256) k_pulse_f32(const float* sx, const float* sy, const float* sz, float* ox, float* oy,
-                                                   float* oz, unsigned N, uint64_t seed,
-                                                   const long long* __restrict__ interval, uint64_t replica,
-                                                   float sigma) {
-    const uint64_t k = (uint64_t)*interval;   // written at the last interval's end, before the step before this
+                                                   float* oz, unsigned N, uint64_t seed, const long long* interval,
+                                                   uint64_t replica, float sigma) {
+    uint64_t k = load_shared_word(interval);
     // N < 2^31 and the stride is far below 2^31, so the index cannot wrap
     for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
-        float g0, g1, g2;
-        Gauss<float>::draw(noise_words(seed, (uint64_t)i, k, replica), g0, g1, g2);
-        pdl_wait();   // returns at once after the first time
-        pdl_go();
-        float x = sx[i], y = sy[i], z = sz[i];
+        float g0, g1, g2, x, y, z;
+        for (;;) {
+            Gauss<float>::draw(noise_words(seed, (uint64_t)i, k, replica), g0, g1, g2);
+            pdl_wait();   // returns at once after the first time
+            pdl_go();
+            const uint64_t now = load_shared_word(interval);
+            x = sx[i];
+            y = sy[i];
+            z = sz[i];
+            if (now == k) break;
+            k = now;
+        }
         pulse_rotate<float>(x, y, z, mul_rn(sigma, g0), mul_rn(sigma, g1), mul_rn(sigma, g2), sigma);
         ox[i] = x;
         oy[i] = y;

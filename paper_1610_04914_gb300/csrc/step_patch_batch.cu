@@ -90,9 +90,9 @@ __global__ void __launch_bounds__(256) k_pulse_batch(float* __restrict__ sx, flo
                                                      const long long* __restrict__ interval) {
     const ObsBlock ob = blocks[blockIdx.x];
     const BatchRep rp = reps[ob.rep];
-    const uint64_t k = (uint64_t)*interval;
     pdl_wait();
     pdl_go();
+    const uint64_t k = (uint64_t)*interval;
     const unsigned first = (unsigned)ob.row0 * rp.L;
     const unsigned count = (unsigned)ob.nrows * rp.L;
     for (unsigned q = threadIdx.x; q < count; q += blockDim.x) {
