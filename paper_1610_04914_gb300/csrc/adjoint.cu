@@ -529,7 +529,7 @@ __global__ void __launch_bounds__(kAT, CHAIN ? SPIN_ADJ_MINB : 1) k_adj_x0_top(X
 // gradient, whose sum is dL/dH): block (p, c) writes parts[c kSumParts + p];
 // fixed order (deterministic), four chains of additions per thread.
 constexpr int kSumParts = 152;
-__global__ void __launch_bounds__(kAT) k_adj_sum_parts(const double* __restrict__ gjd, const double* __restrict__ gh,
+__global__ void __launch_bounds__(kAT) k_adj_sum_parts(const double* gjd, const double* gh,
                                                        long long N, double* __restrict__ parts) {
     __shared__ double red[kAW];
     pdl_wait();
@@ -549,7 +549,7 @@ __global__ void __launch_bounds__(kAT) k_adj_sum_parts(const double* __restrict_
 
 // acc[c] = the FP64 sum of parts[c kSumParts ...] (one block per array, fixed
 // order).
-__global__ void __launch_bounds__(kAT) k_adj_sum_final(const double* __restrict__ parts, double* __restrict__ acc) {
+__global__ void __launch_bounds__(kAT) k_adj_sum_final(const double* parts, double* __restrict__ acc) {
     __shared__ double red[kAW];
     pdl_wait();
     const double* g = parts + (long long)blockIdx.x * kSumParts;

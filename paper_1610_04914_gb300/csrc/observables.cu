@@ -47,10 +47,9 @@ struct ObsLane {
 // FP32, then added in FP64.  FP64: the sums of bonds and s_z^2 are kept apart
 // and combined once per row, 13 FP64 operations a site.
 template <typename real, bool HSITE>
-__device__ __forceinline__ void obs_row(ObsLane& o, const real* __restrict__ sx, const real* __restrict__ sy,
-                                        const real* __restrict__ sz, const real* __restrict__ hx,
-                                        const real* __restrict__ hy, const real* __restrict__ hz, long long rb,
-                                        long long rby, long long rbz, int nx, bool openx, bool openy, bool openz,
+__device__ __forceinline__ void obs_row(ObsLane& o, const real* sx, const real* sy, const real* sz, const real* hx,
+                                        const real* hy, const real* hz, long long rb, long long rby,
+                                        long long rbz, int nx, bool openx, bool openy, bool openz,
                                         double J, double D, double H0, double H1, double H2, int lane) {
     real m0 = 0, m1 = 0, m2 = 0, e = 0, sq = 0, hs = 0;
     const real Jr = (real)J, Dr = (real)D, H0r = (real)H0, H1r = (real)H1, H2r = (real)H2;
@@ -126,9 +125,8 @@ __device__ __forceinline__ void obs_block(const ObsLane& o, double* __restrict__
 
 template <typename real, bool HSITE>
 __global__ void __launch_bounds__(kObsThreads, 2)
-    k_obs_partial(const real* __restrict__ sx, const real* __restrict__ sy, const real* __restrict__ sz,
-                  const real* __restrict__ hx, const real* __restrict__ hy, const real* __restrict__ hz, int nx,
-                  int ny, int nz, double J, double D, double H0, double H1, double H2, double* __restrict__ partials,
+    k_obs_partial(const real* sx, const real* sy, const real* sz, const real* hx, const real* hy, const real* hz,
+                  int nx, int ny, int nz, double J, double D, double H0, double H1, double H2, double* __restrict__ partials,
                   int bc) {
     // one warp per lattice row (y, z); lanes stride along x, so no per-site
     // index division and the row's loads are coalesced
@@ -148,10 +146,9 @@ __global__ void __launch_bounds__(kObsThreads, 2)
     obs_block(o, partials + (long long)blockIdx.x * 5);
 }
 
-__global__ void __launch_bounds__(kObsThreads) k_obs_final(const double* __restrict__ partials, int nblocks, double invN,
+__global__ void __launch_bounds__(kObsThreads) k_obs_final(const double* partials, int nblocks, double invN,
                                                            double* __restrict__ out5, double* __restrict__ ring, int ring_len,
-                                                           long long* __restrict__ interval,
-                                                           long long* __restrict__ sample_count, int R) {
+                                                           long long* interval, long long* sample_count, int R) {
     __shared__ double tot[5];
     pdl_wait();
     long long m = 0, count = 0;
@@ -193,7 +190,7 @@ __global__ void __launch_bounds__(kObsThreads) k_obs_final(const double* __restr
 // Batched replicas: the same row-wise reduction, each block on a row range
 // of one replica; the final pass gives one record per replica.
 __global__ void __launch_bounds__(kObsThreads, 2)
-    k_obs_batch_partial(const float* __restrict__ sx, const float* __restrict__ sy, const float* __restrict__ sz,
+    k_obs_batch_partial(const float* sx, const float* sy, const float* sz,
                         const BatchRep* __restrict__ reps, const ObsBlock* __restrict__ blocks, double J, double D,
                         double H0, double H1, double H2, double* __restrict__ partials) {
     pdl_wait();
@@ -216,12 +213,12 @@ __global__ void __launch_bounds__(kObsThreads, 2)
 
 // one warp per replica at a time, 32 warps
 constexpr int kObsFinalThreads = 1024;
-__global__ void __launch_bounds__(kObsFinalThreads) k_obs_batch_final(const double* __restrict__ partials,
+__global__ void __launch_bounds__(kObsFinalThreads) k_obs_batch_final(const double* partials,
                                                                       const int* __restrict__ first_block,
                                                                       const BatchRep* __restrict__ reps, int nrep,
                                                                       double* __restrict__ out, double* __restrict__ ring,
-                                                                      int ring_len, long long* __restrict__ interval,
-                                                                      long long* __restrict__ sample_count, int R) {
+                                                                      int ring_len, long long* interval,
+                                                                      long long* sample_count, int R) {
     pdl_wait();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const long long m = ring ? *interval : 0;

@@ -76,15 +76,15 @@ struct PatchShape<2, 2> {
 constexpr int kTileVariants = 3;
 
 struct PatchArgs {
-    const float* __restrict__ in0;
-    const float* __restrict__ in1;
-    const float* __restrict__ in2;
+    const float* in0;
+    const float* in1;
+    const float* in2;
     float* __restrict__ out0;
     float* __restrict__ out1;
     float* __restrict__ out2;
-    const float* __restrict__ hs0;
-    const float* __restrict__ hs1;
-    const float* __restrict__ hs2;
+    const float* hs0;
+    const float* hs1;
+    const float* hs2;
     int nx, ny, nz, tz, n_iter;
     float J, twoD, Hx, Hy, Hz, lambda;
     float cdt[4];
@@ -312,9 +312,9 @@ __device__ __forceinline__ void patch_iteration(const PatchArgs& a, PRings<S, HS
 #pragma unroll
             for (int rr = 0; rr < PY; ++rr) {
                 const int o0 = bh + th.col[rr][0], o1 = bh + th.col[rr][1];
-                r.h[sl][rr][0] = make_float2(__ldg(a.hs0 + o0), __ldg(a.hs0 + o1));
-                r.h[sl][rr][1] = make_float2(__ldg(a.hs1 + o0), __ldg(a.hs1 + o1));
-                r.h[sl][rr][2] = make_float2(__ldg(a.hs2 + o0), __ldg(a.hs2 + o1));
+                r.h[sl][rr][0] = make_float2(a.hs0[o0], a.hs0[o1]);
+                r.h[sl][rr][1] = make_float2(a.hs1[o0], a.hs1[o1]);
+                r.h[sl][rr][2] = make_float2(a.hs2[o0], a.hs2[o1]);
             }
         }
     }
@@ -583,9 +583,9 @@ __device__ __forceinline__ void patch_tile(const PatchArgs& a, int bx, int by, i
 #pragma unroll
         for (int rr = 0; rr < PY; ++rr) {
             const int o0 = base + th.col[rr][0], o1 = base + th.col[rr][1];
-            r.s[L & 3][rr][0] = make_float2(__ldg(a.in0 + o0), __ldg(a.in0 + o1));
-            r.s[L & 3][rr][1] = make_float2(__ldg(a.in1 + o0), __ldg(a.in1 + o1));
-            r.s[L & 3][rr][2] = make_float2(__ldg(a.in2 + o0), __ldg(a.in2 + o1));
+            r.s[L & 3][rr][0] = make_float2(a.in0[o0], a.in0[o1]);
+            r.s[L & 3][rr][1] = make_float2(a.in1[o0], a.in1[o1]);
+            r.s[L & 3][rr][2] = make_float2(a.in2[o0], a.in2[o1]);
             if (a.bc) {
                 const float zin = (t0 + L >= 0 && t0 + L < a.nz) ? 1.f : 0.f;
                 const f2 m = make_float2(th.cmask[rr].x * zin, th.cmask[rr].y * zin);

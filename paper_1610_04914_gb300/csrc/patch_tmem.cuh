@@ -279,12 +279,12 @@ __device__ __forceinline__ void tm_tile(const PatchArgs& a, int bx, int by, int 
         f2 s2[3];
         const int b2 = wrapi(t0 + 2, a.nz) * th.plane, b3 = wrapi(t0 + 3, a.nz) * th.plane;
         const int o0 = th.col[0][0], o1 = th.col[0][1];
-        s2[0] = make_float2(__ldg(a.in0 + b2 + o0), __ldg(a.in0 + b2 + o1));
-        s2[1] = make_float2(__ldg(a.in1 + b2 + o0), __ldg(a.in1 + b2 + o1));
-        s2[2] = make_float2(__ldg(a.in2 + b2 + o0), __ldg(a.in2 + b2 + o1));
-        sc[0] = make_float2(__ldg(a.in0 + b3 + o0), __ldg(a.in0 + b3 + o1));
-        sc[1] = make_float2(__ldg(a.in1 + b3 + o0), __ldg(a.in1 + b3 + o1));
-        sc[2] = make_float2(__ldg(a.in2 + b3 + o0), __ldg(a.in2 + b3 + o1));
+        s2[0] = make_float2(a.in0[b2 + o0], a.in0[b2 + o1]);
+        s2[1] = make_float2(a.in1[b2 + o0], a.in1[b2 + o1]);
+        s2[2] = make_float2(a.in2[b2 + o0], a.in2[b2 + o1]);
+        sc[0] = make_float2(a.in0[b3 + o0], a.in0[b3 + o1]);
+        sc[1] = make_float2(a.in1[b3 + o0], a.in1[b3 + o1]);
+        sc[2] = make_float2(a.in2[b3 + o0], a.in2[b3 + o1]);
         if (a.bc) {
             const float z2 = (t0 + 2 >= 0 && t0 + 2 < a.nz) ? 1.f : 0.f;
             const float z3 = (t0 + 3 >= 0 && t0 + 3 < a.nz) ? 1.f : 0.f;

@@ -5,7 +5,9 @@
 // when the kernel before has finished and its writes are visible.  Nothing that
 // an earlier kernel on the stream writes may be relied on before that, not even
 // what the kernel before the last one wrote (some kernels call pdl_go before
-// their own pdl_wait).
+// their own pdl_wait).  Such data is read by plain loads: __ldg and
+// const __restrict__ parameters tell the compiler that it does not change while
+// the kernel runs, so that a load may move ahead of the wait.
 //
 // In interval graphs the kernels get ordinary edges, with one exception.
 // Programmatic edges between graph nodes gained nothing or cost time (an interval of 96 replicas 2048 -> 2133 us, RK5 at 128^3 1108 -> 1148,

@@ -87,7 +87,7 @@ cudaError_t batch_dispatch(const PatchArgs& a, const BatchItem* items, int nitem
 __global__ void __launch_bounds__(256) k_pulse_batch(float* __restrict__ sx, float* __restrict__ sy,
                                                      float* __restrict__ sz, const BatchRep* __restrict__ reps,
                                                      const ObsBlock* __restrict__ blocks, uint64_t seed,
-                                                     const long long* __restrict__ interval) {
+                                                     const long long* interval) {
     const ObsBlock ob = blocks[blockIdx.x];
     const BatchRep rp = reps[ob.rep];
     pdl_wait();

@@ -58,9 +58,9 @@ constexpr int kSlotBytes = kTY * kRowBytes;            // one plane of the tile 
 constexpr int kOutBufFloats = kOutY * kOutX * kRec;    // A's output records of one plane
 
 struct Rk5Args {
-    const float* __restrict__ in0;   // A: the state s
-    const float* __restrict__ in1;
-    const float* __restrict__ in2;
+    const float* in0;   // A: the state s
+    const float* in1;
+    const float* in2;
     float* __restrict__ out0;        // B: the new state
     float* __restrict__ out1;
     float* __restrict__ out2;
@@ -424,15 +424,15 @@ __global__ void __launch_bounds__(kNT, 1) k_step_rk5(Rk5Args a) {
         const int base = wrapi(t0 + L, a.nz) * th.plane;
         const int o0 = base + th.col[0], o1 = base + th.col[1];
         if (SEG == 0) {
-            r.x[0][L][0] = make_float2(__ldg(a.in0 + o0), __ldg(a.in0 + o1));
-            r.x[0][L][1] = make_float2(__ldg(a.in1 + o0), __ldg(a.in1 + o1));
-            r.x[0][L][2] = make_float2(__ldg(a.in2 + o0), __ldg(a.in2 + o1));
+            r.x[0][L][0] = make_float2(a.in0[o0], a.in0[o1]);
+            r.x[0][L][1] = make_float2(a.in1[o0], a.in1[o1]);
+            r.x[0][L][2] = make_float2(a.in2[o0], a.in2[o1]);
         } else {
             const float* c0 = a.car + (size_t)kRec * (unsigned)o0;
             const float* c1 = a.car + (size_t)kRec * (unsigned)o1;
-            r.x[0][L][0] = make_float2(__ldg(c0 + 0), __ldg(c1 + 0));
-            r.x[0][L][1] = make_float2(__ldg(c0 + 1), __ldg(c1 + 1));
-            r.x[0][L][2] = make_float2(__ldg(c0 + 2), __ldg(c1 + 2));
+            r.x[0][L][0] = make_float2(c0[0], c1[0]);
+            r.x[0][L][1] = make_float2(c0[1], c1[1]);
+            r.x[0][L][2] = make_float2(c0[2], c1[2]);
         }
         if (a.bc) {
             const f2 m = r5_mask(th, t0 + L, a.nz);

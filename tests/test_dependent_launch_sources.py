@@ -5,8 +5,6 @@ import glob
 import os
 import re
 
-import pytest
-
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1610_04914_gb300", "csrc")
 
 
@@ -41,3 +39,16 @@ def test_pulse_number_is_read_after_the_wait():
         assert not re.search(r"\*\s*(a\.)?interval\b", before), name
         if "load_shared_word" in before:
             assert "load_shared_word" in after, name
+
+
+def test_data_of_earlier_kernels_is_read_by_plain_loads():
+    """A load that the compiler takes for one of unchanging data may move ahead
+    of the wait: only the constant tables are read that way."""
+    for name, params, _ in kernels():
+        assert not re.search(r"const\s+(real|float|double|long long)\s*\*\s*__restrict__", params), name
+    for path in glob.glob(os.path.join(CSRC, "*.cu*")):
+        text = re.sub(r"//[^\n]*", "", open(path).read())
+        assert all(t.startswith("&k") for t in re.findall(r"__ldg\(([^)]*)", text)), path
+    for header in ("patch_tile.cuh", "step_rk5.cu"):
+        text = open(os.path.join(CSRC, header)).read()
+        assert not re.search(r"const float\*\s*__restrict__", text), header
