@@ -568,12 +568,21 @@ cudaError_t upload_scales(const spin_params* p, int nrep, const double* T, const
     return e;
 }
 
-// Lanes per replica of a rectangular-noise run: while the launch leaves most
-// schedulers with a warp or less.  Heun, R = 1, 200 steps with 1 / 2 / 4 / 8
-// lanes: 1000 replicas 154 / 117 / 82 / 69 us, 8192 157 / 119 / 99 / 116, 16384
-// 156 / 142 / 145 / 184; RK5, R = 4: 1000 80 / 71 / 64 / 62, 8192 82 / 72 / 87 /
-// 142, 16384 82 / 94 / 149 / 228.
-int rect_lanes(int nrep) { return nrep <= 2048 ? 8 : nrep <= 6144 ? 4 : nrep <= 10240 ? 2 : 1; }
+// Lanes per replica of a rectangular-noise run: as many as leave one warp per
+// scheduler (152 SMs with a block of four warps each).  Up to there the lanes'
+// repeated steps cost nothing and the draws of 8, 4 or 2 intervals run side by
+// side; a second warp on a scheduler doubles the steps' share where the
+// arithmetic pipe is the limit, in FP64 always (limits of 2048, 6144 and 10240
+// replicas for all runs, against one lane: 6144 and 10240 FP64 replicas took 1.7
+// to 1.9 times as long, RK5 with R = 40 in FP32 1.06 times).  120 steps, us, one
+// lane before / 8 lanes at 2432 / 4 at 4864 / 2 at 9728 / 1 at 9729 replicas:
+// Heun R = 1 107 / 48 / 56 / 77 / 96, FP64 1062 / 422 / 462 / 548 / 714; RK5
+// R = 40 49 / 38 / 38 / 39 / 41, FP64 1022 / 982 / 980 / 986 / 1006.
+int rect_lanes(int nrep) {
+    for (int lanes = 8; lanes > 1; lanes >>= 1)
+        if (nrep <= 152 * 128 / lanes) return lanes;
+    return 1;
+}
 
 template <typename real, int INTEG>
 cudaError_t rect_launch(int nrep, int lanes, const RunArgs<real>& A, cudaStream_t st) {
