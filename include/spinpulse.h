@@ -133,13 +133,17 @@ int spin_lattice_create(const spin_params* p, void* sx, void* sy, void* sz,
  * values at the end of each Delta t).  Full intervals are replayed from cached
  * CUDA graphs, on lattices of up to 2^20 sites several intervals per graph.  On return (stream-ordered) the caller's arrays hold the
  * state after the last step.
- * Kernel choice for FP32 RK4 steps (all give bitwise the same states): the
- * register-ring fused step, or, where its wave-cost estimate is lower (large
- * lattices, no per-site field), the step that keeps its older planes in
- * tensor memory; the environment variable SPIN_TMEM=0 / =1, read when a step
- * is launched or captured, forbids / forces the latter, and SPIN_TMA=1
- * stages the spin planes by tensor-map bulk copies instead of cp.async
- * (slower on GB300; kept for measurement).
+ * Kernel choice for FP32 steps of the chain tableaus (all give bitwise the same
+ * states): on small lattices (48^3 sites and fewer for RK4, 64^3 for the
+ * two-stage tableaus, 56^3 and 72^3 with site fields) one kernel per stage, else
+ * the register-ring fused step, or, for RK4 where its wave-cost estimate is lower
+ * (large lattices, no per-site field), the step that keeps its older planes in
+ * tensor memory.  Environment variables, read when a step is launched or
+ * captured: SPIN_TMEM=0 forbids and SPIN_TMEM=1 forces the last of these for
+ * RK4 without site fields, and SPIN_TMA=1 stages the spin planes of RK4 steps by
+ * tensor-map bulk copies instead of cp.async where the lattice's sides allow it
+ * (slower on GB300; kept for measurement); either at 1 takes the fused step, not
+ * the stage kernels, at every size.
  * Errors: SPIN_EINVAL (null handle, nsteps < 0), SPIN_ECUDA.
  */
 int spin_step_pulse(spin_lattice* h, int64_t nsteps);

@@ -12,6 +12,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cstdlib>
 
 #include "spin_device.cuh"
 #include "spin_internal.h"
@@ -255,12 +256,22 @@ static cudaError_t launch_generic(const StepLaunch<real>& L) {
     return cudaGetLastError();
 }
 
+// SPIN_TMA=1 and SPIN_TMEM=1 choose a form of the fused tile, at every size.
+static bool tile_forced() {
+    for (const char* name : {"SPIN_TMA", "SPIN_TMEM"}) {
+        const char* env = std::getenv(name);
+        if (env && env[0] == '1') return true;
+    }
+    return false;
+}
+
 template <typename real>
 cudaError_t launch_step(const StepLaunch<real>& L) {
     if (L.tab->chain && !L.force_generic && (L.tab->stages == 4 || L.tab->stages == 2)) {
         if (sizeof(real) == 4) {
             const StepLaunch<float>& F = reinterpret_cast<const StepLaunch<float>&>(L);
-            if (!stage32_small(L.g, L.tab->stages, F.hs[0] != nullptr, F.st_n[0][0] != nullptr)) return launch_step_patch(F);
+            if (!stage32_small(L.g, L.tab->stages, F.hs[0] != nullptr, F.st_n[0][0] != nullptr) || tile_forced())
+                return launch_step_patch(F);
             const cudaError_t e = launch_step_stage32(F);
             return e != cudaSuccess || !L.pulse ? e : launch_pulse_lattice(F);
         }
