@@ -108,8 +108,9 @@ Layout layout_for(const spin_params* p) {
     if (generic) off += align_up(elt * (size_t)(tb.stages + 1) * 3 * (size_t)g.N());
     else if (elt == 8) off += align_up(elt * (size_t)stage64_scratch(tb.stages) * (size_t)g.N());
     // stage inputs of the small-lattice FP32 stage kernels, with site fields or
-    // without
-    if (elt == 4 && stage32_small(g, tb.stages == 4 ? 4 : 2, true, false)) {
+    // without (RK5, which does not take them, has the room too: callers may count
+    // on its workspace being the RK4 one and its own stage arrays)
+    if (elt == 4 && p->path != 1 && stage32_small(g, tb.stages == 4 ? 4 : 2, true, false)) {
         if (!generic) L.tmp = off;
         off += align_up(elt * (size_t)stage32_scratch(tb.stages) * (size_t)g.N());
     }
