@@ -131,8 +131,11 @@ int spin_lattice_create(const spin_params* p, void* sx, void* sy, void* sz,
  * (Eq. ST-expansion: mid-interval; every step when R = 1), and the
  * observables are sampled into the sample ring when n mod R == 0 (Sec. III.A:
  * values at the end of each Delta t).  Full intervals are replayed from cached
- * CUDA graphs, on lattices of up to 2^20 sites several intervals per graph.  On return (stream-ordered) the caller's arrays hold the
- * state after the last step.
+ * CUDA graphs, on lattices of up to 2^20 sites several intervals per graph.  On
+ * a stream that the caller captures, the kernels of every step are captured, as
+ * ordinary launches (the handle's step count then counts the captured steps; the
+ * pulse number and the samples follow the replays).  On return (stream-ordered)
+ * the caller's arrays hold the state after the last step.
  * Kernel choice for FP32 steps of the chain tableaus (all give bitwise the same
  * states): on small lattices (48^3 sites and fewer for RK4, 64^3 for the
  * two-stage tableaus, 56^3 and 72^3 with site fields) one kernel per stage, else

@@ -17,6 +17,7 @@
 #include <vector>
 
 #include "../../include/spinpulse.h"
+#include "pdl.cuh"
 #include "spin_internal.h"
 
 using namespace spin;
@@ -239,12 +240,15 @@ Phys<double> bphys(const spin_batch* b) {
     return ph;
 }
 
+int into(const spin_batch* b, cudaStream_t st) {
+    return b->capture_stream && st == b->capture_stream ? kIntervalGraph : launch_into(st);
+}
+
 cudaError_t batch_observe(spin_batch* b, int buf, bool sample, cudaStream_t st) {
     const float* s[3] = {(const float*)b->buf[buf][0], (const float*)b->buf[buf][1], (const float*)b->buf[buf][2]};
     return launch_observables_batch(s, b->reps, b->oblocks, b->nblocks_obs, b->first_block, b->nrep, bphys(b),
                                     b->partials, b->out, sample ? b->ring : nullptr, SPIN_BATCH_SAMPLE_RING,
-                                    b->d_interval, b->d_sample_count, b->p.steps_per_pulse, st,
-                                    b->capture_stream && st == b->capture_stream);
+                                    b->d_interval, b->d_sample_count, b->p.steps_per_pulse, st, into(b, st));
 }
 
 // One launch per tile variant in use, each over its slice of the item table.
@@ -268,7 +272,7 @@ cudaError_t batch_one_step(spin_batch* b, int from, long long n_next, cudaStream
     if (pulse) {
         float* s[3] = {(float*)b->buf[from ^ 1][0], (float*)b->buf[from ^ 1][1], (float*)b->buf[from ^ 1][2]};
         e = launch_pulse_batch(s, b->reps, b->oblocks, b->nblocks_obs, b->p.seed, b->d_interval, st,
-                               b->capture_stream && st == b->capture_stream);
+                               into(b, st));
         if (e != cudaSuccess) return e;
     }
     if (n_next % R == 0) e = batch_observe(b, from ^ 1, true, st);
@@ -586,8 +590,9 @@ int spin_batch_autotune(spin_batch* b) {
 int spin_batch_step_pulse(spin_batch* b, int64_t nsteps) {
     if (!b || nsteps < 0) return SPIN_EINVAL;
     const int R = b->p.steps_per_pulse;
+    const bool replays = launch_into(b->st) == kStream;   // a caller's capture gets the steps' kernels themselves
     while (nsteps > 0) {
-        if (b->n % R == 0 && nsteps >= R && b->eager_intervals > 0) {
+        if (replays && b->n % R == 0 && nsteps >= R && b->eager_intervals > 0) {
             if (!b->graph[b->cur]) {
                 int rc = capture_batch_interval(b, b->cur);
                 if (rc != SPIN_OK) return rc;

@@ -176,14 +176,15 @@ cudaError_t sweeps_t(const spin_params* p, void* s, const void* h_site, uint64_t
     A.accepted = accepted;
     const long long threads = (long long)p->ny * p->nz * ((p->nx + 1) / 2);
     const unsigned blocks = (unsigned)((threads + 255) / 256);
+    const bool pdl = launch_into(st) == kStream;
     for (long long w = sweep0; w < sweep0 + nsweeps; ++w) {
         A.sweep = w;
         for (int c = 0; c < 2; ++c) {
             if (only_color >= 0 && c != only_color) continue;
             A.color = c;
             const cudaError_t e =
-                h_site ? launch_pdl(true, k_metropolis<real, true>, dim3(blocks), dim3(256), 0, st, A)
-                       : launch_pdl(true, k_metropolis<real, false>, dim3(blocks), dim3(256), 0, st, A);
+                h_site ? launch_pdl(pdl, k_metropolis<real, true>, dim3(blocks), dim3(256), 0, st, A)
+                       : launch_pdl(pdl, k_metropolis<real, false>, dim3(blocks), dim3(256), 0, st, A);
             if (e != cudaSuccess) return e;
         }
     }

@@ -259,10 +259,10 @@ int observables_blocks(Geom g) {
 template <typename real>
 cudaError_t launch_observables(const real* s[3], const real* hs[3], Geom g, Phys<double> ph, double* partials,
                                int nblocks, double* out5, double* sample_ring, int ring, long long* d_interval,
-                               long long* d_sample_count, int R, cudaStream_t stream, int bc, bool graph) {
+                               long long* d_sample_count, int R, cudaStream_t stream, int bc, int into) {
     const double D = 0.5 * ph.twoD;
     const dim3 grid(nblocks), block(kObsThreads);
-    const bool pdl = !graph || (sizeof(real) == 4 && g.N() <= kPdlGraphSites);
+    const bool pdl = pdl_after_step(into, (int)sizeof(real), g.N());
     const cudaError_t e =
         hs[0] ? launch_pdl(pdl, k_obs_partial<real, true>, grid, block, 0, stream, s[0], s[1], s[2], hs[0], hs[1], hs[2], g.nx,
                            g.ny, g.nz, ph.J, D, ph.H[0], ph.H[1], ph.H[2], partials, bc)
@@ -276,19 +276,19 @@ cudaError_t launch_observables(const real* s[3], const real* hs[3], Geom g, Phys
 cudaError_t launch_observables_batch(const float* s[3], const BatchRep* reps, const ObsBlock* blocks, int nblocks,
                                      const int* first_block, int nrep, Phys<double> ph, double* partials,
                                      double* out, double* ring, int ring_len, long long* d_interval,
-                                     long long* d_sample_count, int R, cudaStream_t stream, bool graph) {
-    const cudaError_t e = launch_pdl(!graph, k_obs_batch_partial, dim3(nblocks), dim3(kObsThreads), 0, stream, s[0], s[1], s[2], reps,
+                                     long long* d_sample_count, int R, cudaStream_t stream, int into) {
+    const cudaError_t e = launch_pdl(into == kStream, k_obs_batch_partial, dim3(nblocks), dim3(kObsThreads), 0, stream, s[0], s[1], s[2], reps,
                                      blocks, ph.J, 0.5 * ph.twoD, ph.H[0], ph.H[1], ph.H[2], partials);
     if (e != cudaSuccess) return e;
-    return launch_pdl(!graph, k_obs_batch_final, dim3(1), dim3(kObsFinalThreads), 0, stream, (const double*)partials, first_block, reps, nrep, out,
+    return launch_pdl(into == kStream, k_obs_batch_final, dim3(1), dim3(kObsFinalThreads), 0, stream, (const double*)partials, first_block, reps, nrep, out,
                         ring, ring_len, d_interval, d_sample_count, R);
 }
 
 template cudaError_t launch_observables<float>(const float* s[3], const float* hs[3], Geom, Phys<double>, double*, int,
-                                               double*, double*, int, long long*, long long*, int, cudaStream_t, int, bool);
+                                               double*, double*, int, long long*, long long*, int, cudaStream_t, int, int);
 template cudaError_t launch_observables<double>(const double* s[3], const double* hs[3], Geom, Phys<double>, double*,
                                                 int, double*, double*, int, long long*, long long*, int, cudaStream_t,
-                                                int, bool);
+                                                int, int);
 
 }  // namespace spin
 
@@ -373,19 +373,20 @@ extern "C" int spin_observables_noalloc(int32_t precision, const void* sx, const
     ph.H[1] = H[1];
     ph.H[2] = H[2];
     const size_t comp = (size_t)(precision == 64 ? 8 : 4) * (size_t)g.N();
+    const int into = launch_into(st) == kStream ? kIntervalGraph : kCallersGraph;   // large lattices: ordinary launches
     cudaError_t e;
     if (precision == 32) {
         const float* s[3] = {(const float*)sx, (const float*)sy, (const float*)sz};
         const float* hs[3] = {nullptr, nullptr, nullptr};
         if (h_site)
             for (int c = 0; c < 3; ++c) hs[c] = (const float*)((const char*)h_site + c * comp);
-        e = launch_observables<float>(s, hs, g, ph, scratch, nblocks, out5, nullptr, 0, nullptr, nullptr, 1, st, bc, true);
+        e = launch_observables<float>(s, hs, g, ph, scratch, nblocks, out5, nullptr, 0, nullptr, nullptr, 1, st, bc, into);
     } else {
         const double* s[3] = {(const double*)sx, (const double*)sy, (const double*)sz};
         const double* hs[3] = {nullptr, nullptr, nullptr};
         if (h_site)
             for (int c = 0; c < 3; ++c) hs[c] = (const double*)((const char*)h_site + c * comp);
-        e = launch_observables<double>(s, hs, g, ph, scratch, nblocks, out5, nullptr, 0, nullptr, nullptr, 1, st, bc, true);
+        e = launch_observables<double>(s, hs, g, ph, scratch, nblocks, out5, nullptr, 0, nullptr, nullptr, 1, st, bc, into);
     }
     return e == cudaSuccess ? SPIN_OK : SPIN_ECUDA;
 }

@@ -677,7 +677,7 @@ inline PatchArgs patch_args_common(const StepLaunch<float>& L) {
     a.sigma = L.sigma;
     a.interval = L.d_interval;
     a.bc = L.bc;
-    a.pdl = L.graph ? 0 : 1;
+    a.pdl = L.into == kStream;
     a.err = L.d_status;
     return a;
 }

@@ -35,6 +35,20 @@ __device__ __forceinline__ unsigned long long load_shared_word(const long long* 
 
 constexpr long long kPdlGraphSites = 1LL << 20;
 
+// Where a launch goes: to a stream, into a handle's own interval graph, or into
+// a graph that the caller captures.  The last gets ordinary launches only: a
+// caller may ask for the edges of its graph, or add to the capture, by calls
+// that refuse edges with data.
+enum LaunchInto { kStream = 0, kIntervalGraph = 1, kCallersGraph = 2 };
+inline int launch_into(cudaStream_t st) {
+    cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+    return cudaStreamIsCapturing(st, &s) == cudaSuccess && s != cudaStreamCaptureStatusNone ? kCallersGraph : kStream;
+}
+// The pulse and the observables (elt: bytes of a component).
+inline bool pdl_after_step(int into, int elt, long long N) {
+    return into == kStream || (into == kIntervalGraph && elt == 4 && N <= kPdlGraphSites);
+}
+
 // pdl = false: an ordinary launch.
 template <typename Kern, typename... Args>
 cudaError_t launch_pdl(bool pdl, Kern kernel, dim3 grid, dim3 block, size_t smem, cudaStream_t st, const Args&... args) {

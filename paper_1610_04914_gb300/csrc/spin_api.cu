@@ -11,6 +11,7 @@
 #include <new>
 
 #include "../../include/spinpulse.h"
+#include "pdl.cuh"
 #include "spin_internal.h"
 
 using namespace spin;
@@ -190,7 +191,9 @@ Phys<double> phys64(const spin_lattice* h) {
 }
 
 // Work on the handle's capture stream goes into an interval graph.
-bool captured(const spin_lattice* h, cudaStream_t st) { return h->capture_stream && st == h->capture_stream; }
+int into(const spin_lattice* h, cudaStream_t st) {
+    return h->capture_stream && st == h->capture_stream ? kIntervalGraph : launch_into(st);
+}
 
 // Launch observables of buffer b; sample=true records into the ring.
 cudaError_t observe(spin_lattice* h, int b, bool sample, cudaStream_t st) {
@@ -200,14 +203,14 @@ cudaError_t observe(spin_lattice* h, int b, bool sample, cudaStream_t st) {
         return launch_observables<float>(s, hs, h->g, phys64(h), h->partials, h->nblocks_obs,
                                          sample ? h->out_sample : h->out_obs, sample ? h->ring : nullptr,
                                          SPIN_SAMPLE_RING, h->d_interval, h->d_sample_count, h->p.steps_per_pulse, st,
-                                         h->p.bc, captured(h, st));
+                                         h->p.bc, into(h, st));
     }
     const double* s[3] = {(const double*)h->buf[b][0], (const double*)h->buf[b][1], (const double*)h->buf[b][2]};
     const double* hs[3] = {(const double*)h->hs[0], (const double*)h->hs[1], (const double*)h->hs[2]};
     return launch_observables<double>(s, hs, h->g, phys64(h), h->partials, h->nblocks_obs,
                                       sample ? h->out_sample : h->out_obs, sample ? h->ring : nullptr,
                                       SPIN_SAMPLE_RING, h->d_interval, h->d_sample_count, h->p.steps_per_pulse, st,
-                                      h->p.bc, captured(h, st));
+                                      h->p.bc, into(h, st));
 }
 
 // One step n -> n+1 from buffer *buf on stream st, which becomes the buffer of
@@ -224,7 +227,7 @@ cudaError_t launch_one_step(spin_lattice* h, int* buf, long long n_next, cudaStr
     if (h->elt == 4) {
         StepLaunch<float> L = make_launch<float>(h, from, pulse);
         L.stream = st;
-        L.graph = captured(h, st);
+        L.into = into(h, st);
         if (pulse && (R & 1) && !L.force_generic && (h->tab.chain || rk5_fused_supports(L))) {
             to = from;
             for (int c = 0; c < 3; ++c) L.pulse_out[c] = static_cast<float*>(h->buf[to][c]);
@@ -233,7 +236,7 @@ cudaError_t launch_one_step(spin_lattice* h, int* buf, long long n_next, cudaStr
     } else {
         StepLaunch<double> L = make_launch<double>(h, from, pulse);
         L.stream = st;
-        L.graph = captured(h, st);
+        L.into = into(h, st);
         e = launch_step<double>(L);
     }
     if (e != cudaSuccess) return e;
@@ -444,6 +447,8 @@ int spin_lattice_create(const spin_params* p, void* sx, void* sy, void* sz, cons
 int spin_step_pulse(spin_lattice* h, int64_t nsteps) {
     if (!h || nsteps < 0) return SPIN_EINVAL;
     const int R = h->p.steps_per_pulse;
+    // a caller's capture gets the steps' kernels themselves
+    const bool replays = launch_into(h->st) == kStream;
     while (nsteps > 0) {
         if (h->rec_active) {
             // recording: a whole noise interval is replayed from the graph when
@@ -452,7 +457,7 @@ int spin_step_pulse(spin_lattice* h, int64_t nsteps) {
             // checkpoint step is seen
             const long long d0 = h->n - h->rec_n0;
             const long long next_ckpt = (d0 / h->rec_K + 1) * h->rec_K;
-            if (h->n % R == 0 && nsteps >= R && h->eager_intervals > 0 && d0 >= 0 && next_ckpt >= d0 + R) {
+            if (replays && h->n % R == 0 && nsteps >= R && h->eager_intervals > 0 && d0 >= 0 && next_ckpt >= d0 + R) {
                 int rc = replay(h, 0);
                 if (rc != SPIN_OK) return rc;
                 nsteps -= R;
@@ -468,7 +473,7 @@ int spin_step_pulse(spin_lattice* h, int64_t nsteps) {
             if (rc != SPIN_OK) return rc;
             continue;
         }
-        if (h->n % R == 0 && nsteps >= R && h->eager_intervals > 0) {
+        if (replays && h->n % R == 0 && nsteps >= R && h->eager_intervals > 0) {
             const int level = graph_level(h, nsteps);
             const int rc = replay(h, level);
             if (rc != SPIN_OK) return rc;

@@ -52,7 +52,7 @@ struct StepLaunch {
     cudaStream_t stream;
     int force_generic;
     int bc;                // 0 periodic, 1 free boundaries
-    int graph;             // 1: captured into an interval graph (kernels get ordinary edges)
+    int into;              // LaunchInto (pdl.cuh); graphs get ordinary launches
     // FP32 fused path only: if st_n[0][0] is set, the step also writes, at
     // every site, the stage inputs X_j (j = 2..S, st_x[j-2]), the neighbour
     // sums sum_nn X_j of every stage (j = 1..S, st_n[j-1]) and the
@@ -118,11 +118,11 @@ struct ObsBlock {
 };
 // Pulse rotation of every site of every replica (block table as above).
 cudaError_t launch_pulse_batch(float* s[3], const BatchRep* reps, const ObsBlock* blocks, int nblocks, uint64_t seed,
-                               const long long* d_interval, cudaStream_t st, bool graph);
+                               const long long* d_interval, cudaStream_t st, int into);
 cudaError_t launch_observables_batch(const float* s[3], const BatchRep* reps, const ObsBlock* blocks, int nblocks,
                                      const int* first_block, int nrep, Phys<double> ph, double* partials,
                                      double* out, double* ring, int ring_len, long long* d_interval,
-                                     long long* d_sample_count, int R, cudaStream_t stream, bool graph);
+                                     long long* d_sample_count, int R, cudaStream_t stream, int into);
 
 // FP64 observables: per-block partials, then a one-block deterministic sum.
 // out5 = (M_x, M_y, M_z, E, nonfinite count); if sample_ring != null the
@@ -132,7 +132,7 @@ template <typename real>
 cudaError_t launch_observables(const real* s[3], const real* hs[3], Geom g, Phys<double> ph,
                                double* partials, int nblocks, double* out5, double* sample_ring,
                                int ring, long long* d_interval, long long* d_sample_count, int R,
-                               cudaStream_t stream, int bc, bool graph);
+                               cudaStream_t stream, int bc, int into);
 int observables_blocks(Geom g);
 
 cudaError_t launch_noise_draw(uint64_t seed, long long k, long long replica, long long n, int precision,

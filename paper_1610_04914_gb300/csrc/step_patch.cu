@@ -355,7 +355,7 @@ cudaError_t launch_pulse_lattice(const StepLaunch<float>& L) {
     const long long N = L.g.N();
     const int blocks = (int)std::max<long long>(1, std::min<long long>((N + 255) / 256, 152LL * 32));
     float* const* o = L.pulse_out[0] ? L.pulse_out : L.out;
-    return launch_pdl(!L.graph || N <= kPdlGraphSites, k_pulse_f32, dim3(blocks), dim3(256), 0, L.stream, (const float*)L.out[0], (const float*)L.out[1],
+    return launch_pdl(pdl_after_step(L.into, 4, N), k_pulse_f32, dim3(blocks), dim3(256), 0, L.stream, (const float*)L.out[0], (const float*)L.out[1],
                       (const float*)L.out[2], o[0], o[1], o[2], (unsigned)N, L.seed, L.d_interval, L.replica, L.sigma);
 }
 

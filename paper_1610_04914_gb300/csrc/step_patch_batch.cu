@@ -110,8 +110,8 @@ __global__ void __launch_bounds__(256) k_pulse_batch(float* __restrict__ sx, flo
 }  // namespace
 
 cudaError_t launch_pulse_batch(float* s[3], const BatchRep* reps, const ObsBlock* blocks, int nblocks, uint64_t seed,
-                               const long long* d_interval, cudaStream_t st, bool graph) {
-    return launch_pdl(!graph, k_pulse_batch, dim3(nblocks), dim3(256), 0, st, s[0], s[1], s[2], reps, blocks, seed, d_interval);
+                               const long long* d_interval, cudaStream_t st, int into) {
+    return launch_pdl(into == kStream, k_pulse_batch, dim3(nblocks), dim3(256), 0, st, s[0], s[1], s[2], reps, blocks, seed, d_interval);
 }
 int patch_out_x(int stages) { return kPC - 2 * stages; }
 int patch_rows(int stages, int variant) {

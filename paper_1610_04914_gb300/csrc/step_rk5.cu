@@ -552,7 +552,7 @@ cudaError_t launch_step_rk5(const StepLaunch<float>& L) {
     a.b6 = c(tb.b[5]);
     a.renorm = L.renorm;
     a.bc = L.bc;
-    a.pdl = L.graph ? 0 : 1;
+    a.pdl = L.into == kStream;
     a.car = L.tmp;   // 12 floats per site in the step scratch
     a.err = L.d_status;
     a.pair8 = pairs_aligned(a.nx, L.in[0], L.in[1], L.in[2]) && pairs_aligned(a.nx, L.out[0], L.out[1], L.out[2]);

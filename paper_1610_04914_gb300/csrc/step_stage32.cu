@@ -114,7 +114,7 @@ cudaError_t run_stages(const StepLaunch<float>& L) {
     a.nlambda = -L.ph.lambda;
     a.bc = L.bc;
     a.renorm = L.renorm;
-    a.pdl = L.graph ? 0 : 1;
+    a.pdl = L.into == kStream;
     for (int c = 0; c < 3; ++c) {
         a.H[c] = L.ph.H[c];
         a.hs[c] = L.hs[c];

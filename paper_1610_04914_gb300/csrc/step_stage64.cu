@@ -284,7 +284,7 @@ cudaError_t launch_step_stage64(const StepLaunch<double>& L) {
     a.lambda = L.ph.lambda;
     a.bc = L.bc;
     a.renorm = L.renorm;
-    a.pdl = L.graph ? 0 : 1;
+    a.pdl = L.into == kStream;
     a.seed = L.seed;
     a.replica = L.replica;
     a.sigma = L.sigma;
