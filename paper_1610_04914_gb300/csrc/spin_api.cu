@@ -16,11 +16,12 @@
 
 using namespace spin;
 
-// Small lattices replay several intervals as one graph: the GPU idles for a few
-// microseconds between two graph launches, and an interval of a few small kernels
-// takes only tens (64^3, RK2, R = 2, ten intervals of a call 477 -> 452 us).
-// A longer graph is captured once enough intervals have been replayed to pay for
-// it, and holds at most kGraphSteps steps.
+// Small lattices replay several intervals as one graph: the GPU idles for two to
+// two and a half microseconds between two graph launches, and an interval of a
+// few small kernels takes only tens.  To capture and instantiate a graph costs
+// the host about 1.9 us a kernel, as long as the kernel takes the GPU or less; so
+// a longer graph is captured only while the GPU still works on at least as many
+// intervals of the same call, and holds at most kGraphSteps steps.
 constexpr int kGraphLevels = 4;
 constexpr int kGraphSteps = 32;
 constexpr long long kLongGraphSites = 1LL << 20;
@@ -288,12 +289,25 @@ int replay(spin_lattice* h, int level) {
     return SPIN_OK;
 }
 
-// The longest graph for a call that has nsteps left.
-int graph_level(const spin_lattice* h, long long nsteps) {
+// The level of the longest graph that n steps fill.
+int longest_level(const spin_lattice* h, long long n) {
     if (h->g.N() > kLongGraphSites || h->replayed < kLongGraphAfter) return 0;
     int level = 0;
-    while (level + 1 < kGraphLevels && ((long long)h->p.steps_per_pulse << (level + 1)) <= std::min<long long>(nsteps, kGraphSteps))
+    while (level + 1 < kGraphLevels && ((long long)h->p.steps_per_pulse << (level + 1)) <= std::min<long long>(n, kGraphSteps))
         ++level;
+    return level;
+}
+
+// The graph for a call that has nsteps left and *ahead intervals queued behind
+// which no graph has been captured yet: the longest that there is, or that can be
+// captured behind them.
+int next_level(const spin_lattice* h, long long nsteps, long long* ahead) {
+    int level = longest_level(h, nsteps);
+    for (; level > 0 && !h->graph[level][h->cur]; --level)
+        if (*ahead >= (1LL << level)) {
+            *ahead -= 1LL << level;
+            break;
+        }
     return level;
 }
 
@@ -449,6 +463,7 @@ int spin_step_pulse(spin_lattice* h, int64_t nsteps) {
     const int R = h->p.steps_per_pulse;
     // a caller's capture gets the steps' kernels themselves
     const bool replays = launch_into(h->st) == kStream;
+    long long intervals = 0, ahead = 0;   // replayed by this call; of those, not yet captured behind
     while (nsteps > 0) {
         if (h->rec_active) {
             // recording: a whole noise interval is replayed from the graph when
@@ -474,10 +489,12 @@ int spin_step_pulse(spin_lattice* h, int64_t nsteps) {
             continue;
         }
         if (replays && h->n % R == 0 && nsteps >= R && h->eager_intervals > 0) {
-            const int level = graph_level(h, nsteps);
+            const int level = next_level(h, nsteps, &ahead);
             const int rc = replay(h, level);
             if (rc != SPIN_OK) return rc;
             nsteps -= (int64_t)R << level;
+            intervals += 1LL << level;
+            ahead += 1LL << level;
             continue;
         }
         const bool interval_start = h->n % R == 0 && nsteps >= R;
@@ -495,6 +512,9 @@ int spin_step_pulse(spin_lattice* h, int64_t nsteps) {
             SPIN_CUDA(h, cudaMemcpyAsync(h->buf[0][c], h->buf[1][c], bytes, cudaMemcpyDeviceToDevice, h->st));
         h->cur = 0;
     }
+    // the graph that a call like this one would begin with
+    const int level = longest_level(h, intervals * R);
+    if (level > 0 && !h->graph[level][0] && ahead >= (1LL << level)) return capture_interval(h, level, 0);
     return SPIN_OK;
 }
 
