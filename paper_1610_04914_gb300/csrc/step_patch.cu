@@ -185,22 +185,37 @@ cudaError_t patch_dispatch(const PatchArgs& a, dim3 grid, cudaStream_t st, bool 
 // rotation and this kernel rotates the finished state in place.  The
 // arithmetic per site is the fused epilogue's, so the results are identical.
 //
-// The draw does not depend on the state: the kernel is launched while the step
-// before it drains and each thread draws for its first site before it waits.
-// The pulse number it draws with then is a guess, loaded where nothing yet
-// promises that an earlier kernel's write of it is visible; the number counts
-// as read only after the wait, and a draw made with another one is made again.
-// The state may go to other arrays (odd intervals, spin_api.cu).
+// The draw does not depend on the state.  AHEAD, on lattices of one site per
+// thread: the kernel is launched while the step before it drains, and each thread
+// draws before it waits.  The pulse number it draws with then is a guess, loaded
+// where nothing yet promises that an earlier kernel's write of it is visible; the
+// number counts as read only after the wait, and a draw made with another one is
+// made again.  Larger lattices, of many sites per thread, wait first: with the
+// second reading in every turn of their loop a replayed pulse took 36.9 us at
+// 128^3 and 281 at 256^3, so 34.9 and 262.  The state may go to
+// other arrays (odd intervals, spin_api.cu).
+__device__ __forceinline__ void pulse_draw(uint64_t seed, unsigned i, uint64_t k, uint64_t replica, float (&g)[3]) {
+    Gauss<float>::draw(noise_words(seed, (uint64_t)i, k, replica), g[0], g[1], g[2]);
+}
+template <bool AHEAD>
 __global__ void __launch_bounds__(256) k_pulse_f32(const float* sx, const float* sy, const float* sz, float* ox, float* oy,
                                                    float* oz, unsigned N, uint64_t seed, const long long* interval,
                                                    uint64_t replica, float sigma) {
-    uint64_t k = load_shared_word(interval);
-    // N < 2^31 and the stride is far below 2^31, so the index cannot wrap
-    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
-        float g0, g1, g2, x, y, z;
+    auto turn = [&](unsigned i, float x, float y, float z, const float (&g)[3]) {
+        pulse_rotate<float>(x, y, z, mul_rn(sigma, g[0]), mul_rn(sigma, g[1]), mul_rn(sigma, g[2]), sigma);
+        ox[i] = x;
+        oy[i] = y;
+        oz[i] = z;
+    };
+    unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+    float g[3];
+    if (AHEAD) {
+        if (i >= N) return;
+        uint64_t k = load_shared_word(interval);
+        float x, y, z;
         for (;;) {
-            Gauss<float>::draw(noise_words(seed, (uint64_t)i, k, replica), g0, g1, g2);
-            pdl_wait();   // returns at once after the first time
+            pulse_draw(seed, i, k, replica, g);
+            pdl_wait();
             pdl_go();
             const uint64_t now = load_shared_word(interval);
             x = sx[i];
@@ -209,10 +224,16 @@ __global__ void __launch_bounds__(256) k_pulse_f32(const float* sx, const float*
             if (now == k) break;
             k = now;
         }
-        pulse_rotate<float>(x, y, z, mul_rn(sigma, g0), mul_rn(sigma, g1), mul_rn(sigma, g2), sigma);
-        ox[i] = x;
-        oy[i] = y;
-        oz[i] = z;
+        turn(i, x, y, z, g);
+        return;
+    }
+    pdl_wait();
+    pdl_go();
+    const uint64_t k = load_shared_word(interval);
+    // N < 2^31 and the stride is far below 2^31, so the index cannot wrap
+    for (; i < N; i += gridDim.x * blockDim.x) {
+        pulse_draw(seed, i, k, replica, g);
+        turn(i, sx[i], sy[i], sz[i], g);
     }
 }
 
@@ -355,8 +376,9 @@ cudaError_t launch_pulse_lattice(const StepLaunch<float>& L) {
     const long long N = L.g.N();
     const int blocks = (int)std::max<long long>(1, std::min<long long>((N + 255) / 256, 152LL * 32));
     float* const* o = L.pulse_out[0] ? L.pulse_out : L.out;
-    return launch_pdl(pdl_after_step(L.into, 4, N), k_pulse_f32, dim3(blocks), dim3(256), 0, L.stream, (const float*)L.out[0], (const float*)L.out[1],
-                      (const float*)L.out[2], o[0], o[1], o[2], (unsigned)N, L.seed, L.d_interval, L.replica, L.sigma);
+    return launch_pdl(pdl_after_step(L.into, 4, N), N <= blocks * 256LL ? k_pulse_f32<true> : k_pulse_f32<false>, dim3(blocks),
+                      dim3(256), 0, L.stream, (const float*)L.out[0], (const float*)L.out[1], (const float*)L.out[2], o[0],
+                      o[1], o[2], (unsigned)N, L.seed, L.d_interval, L.replica, L.sigma);
 }
 
 }  // namespace spin
