@@ -187,8 +187,8 @@ int spin_set_step(spin_lattice* h, int64_t n);
  * Trajectory recording for the adjoint (checkpointing).  From the handle's
  * current step n0, spin_step_pulse copies the state into `store` every K steps
  * (slot c holds the state after step n0 + c*K, component-major: 3N values of
- * the state type), for at most nsteps steps; while recording, steps launch one
- * by one (no graph replay).  store: caller-owned device memory of at least
+ * the state type), for at most nsteps steps; while recording, a whole interval is
+ * replayed from its graph unless a checkpoint falls inside it.  store: caller-owned device memory of at least
  * spin_record_store_size() bytes, borrowed until spin_record_end.
  * Errors: SPIN_EINVAL (K < 1, nsteps < 1, null), SPIN_ENOSPACE, SPIN_ECUDA.
  */
@@ -219,7 +219,9 @@ int spin_record_end(spin_lattice* h);
  * every step is formed in the state precision and added in FP64 (dL/dh_i
  * straight into g_h_site; dL/dJ, dL/dD per site, all three then summed over the
  * sites in FP64; where stages are stored, the terms of one step are first added
- * to each other without rounding).  The adjoint state is kept in the state precision.
+ * to each other: each counts down to 2^-59 of the power of two of the largest, and
+ * the sum is rounded once to double).  The adjoint state is kept in the state
+ * precision.
  * Synchronises the stream.
  * Errors: SPIN_EINVAL (no recording, range mismatch), SPIN_ENOSPACE, SPIN_ECUDA.
  */

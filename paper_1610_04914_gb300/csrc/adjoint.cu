@@ -14,7 +14,7 @@
 // integer bit operations (exact for every finite float), because this GPU's
 // FP64 pipe, which would otherwise convert them, is ~1/76 of its FP32 rate.
 // Where the stages are stored (below), a step's terms stay floats until its last
-// stage and are added exactly, as 64-bit integers, before one FP64 addition each.
+// stage and are added as 64-bit integers (sum4), before one FP64 addition each.
 //
 // Transposes used (f the right-hand side of Eq. LLL at fixed noise, a = s x H):
 //   w_i = (df_i/dH_i)^T v_i = -(s x v) - lambda s x (s x v)    [slow: without -(s x v)]
@@ -273,9 +273,11 @@ __device__ __forceinline__ void w_part(const StageIn<real>& in, const CV3<real>&
     }
 }
 
-// The sum of a step's S terms (S = 2 or 4; the others zero) as a double,
-// rounded once: the mantissas, shifted to the largest exponent, add as 64-bit
-// integers; what lies 2^-60 below the largest term is lost.
+// The sum of a step's S terms (S = 2 or 4; the others zero) as a double: the
+// mantissas, shifted to the largest exponent, add as 64-bit integers, and the sum
+// is rounded once.  A term loses what lies below 2^-59 of the largest one's power of
+// two (nothing, if it is within 36 binades of it); where the terms cancel beyond
+// that, FP64 additions in a row would keep more.
 __device__ __noinline__ double plain_sum4(float a, float b, float c, float d) {
     return (((double)a + (double)b) + (double)c) + (double)d;
 }

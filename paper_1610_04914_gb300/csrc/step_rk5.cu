@@ -71,7 +71,7 @@ struct Rk5Args {
     float a21, a31, a32, a42, a43, a51, a54, a61, a62, a63, a64, a65;
     float b1, b3, b4, b5, b6;
     int renorm;
-    int bc;
+    int bc;                          // 1: free boundaries
     int pdl;                         // host: launch as a programmatic dependent
     int pair8;                       // 1: column pairs are aligned 8-byte words of the state arrays
     int* err;                        // device status word: bit 0 set when a bounded wait gave up

@@ -53,11 +53,12 @@ struct Stage64Args {
 };
 
 // Fixed-point sums of doubles without the FP64 pipe: the mantissas, shifted to
-// the largest exponent of the terms, add exactly as 64-bit integers and the sum
-// is rounded once to nearest.  A term loses only what lies 2^-60 below the
-// largest, so a sum is at least as exact as the additions in a row would be;
-// those are 5 of a component's 12 FP64 instructions per stage, and the integer
-// pipes are idle.  Magnitudes below 2^-923 count as zero; where a term is above
+// the largest exponent of the terms, add as 64-bit integers and the sum is rounded
+// once to nearest.  A term loses what lies below 2^-59 of the largest one's power of
+// two, 64 times less than the first rounding of the additions in a row may cost;
+// only where the terms cancel to below that do the additions keep more ({1, -1,
+// 2^-70} gives 0 here).  Those are 5 of a component's 12 FP64 instructions per
+// stage, and the integer pipes are idle.  Magnitudes below 2^-923 count as zero; where a term is above
 // 2^977, infinite or NaN (emax > kMaxExp) the caller takes the plain sum.
 constexpr unsigned kMinExp = 100u, kMaxExp = 2000u;
 __device__ __forceinline__ unsigned exponent(double v) { return ((unsigned)__double2hiint(v) >> 20) & 0x7FFu; }
@@ -102,9 +103,10 @@ enum StageRole { kFirst, kMiddle, kLast2, kLast4 };
 // the state by its own multiply-adds: 15 FP64 instructions after the field, 18
 // when the two products, their sum and the update are taken one by one.
 
-// WIDE: neighbour sums through the integer pipes, for lattices that fill the FP64 pipe
-// (smaller ones wait on latencies instead, of which the integer form has more:
-// 16^3 242 against 250 us for 10 steps).
+// WIDE: neighbour sums through the integer pipes, for lattices that fill the FP64
+// pipe (up to one warp per scheduler, 19456 sites, latencies count instead, of which
+// the integer form has more: RK4 us per step, plain / integer sums, 23^3 15.8 / 16.0,
+// 24^3 15.3 / 15.8, 26^3 16.3 / 16.2, 27x27x26 16.2 / 16.4).
 template <int ROLE, bool PREC, bool HSITE, bool PULSE, bool WIDE>
 __global__ void __launch_bounds__(128) k_stage64(const __grid_constant__ Stage64Args a) {
     pdl_go();
