@@ -240,15 +240,11 @@ Phys<double> bphys(const spin_batch* b) {
     return ph;
 }
 
-int into(const spin_batch* b, cudaStream_t st) {
-    return b->capture_stream && st == b->capture_stream ? kIntervalGraph : launch_into(st);
-}
-
-cudaError_t batch_observe(spin_batch* b, int buf, bool sample, cudaStream_t st) {
+cudaError_t batch_observe(spin_batch* b, int buf, bool sample, cudaStream_t st, int into) {
     const float* s[3] = {(const float*)b->buf[buf][0], (const float*)b->buf[buf][1], (const float*)b->buf[buf][2]};
     return launch_observables_batch(s, b->reps, b->oblocks, b->nblocks_obs, b->first_block, b->nrep, bphys(b),
                                     b->partials, b->out, sample ? b->ring : nullptr, SPIN_BATCH_SAMPLE_RING,
-                                    b->d_interval, b->d_sample_count, b->p.steps_per_pulse, st, into(b, st));
+                                    b->d_interval, b->d_sample_count, b->p.steps_per_pulse, st, into);
 }
 
 // One launch per tile variant in use, each over its slice of the item table.
@@ -262,7 +258,7 @@ cudaError_t batch_step_kernels(spin_batch* b, const StepLaunch<float>& Ls) {
     return cudaSuccess;
 }
 
-cudaError_t batch_one_step(spin_batch* b, int from, long long n_next, cudaStream_t st) {
+cudaError_t batch_one_step(spin_batch* b, int from, long long n_next, cudaStream_t st, int into) {
     const int R = b->p.steps_per_pulse;
     const bool pulse = b->p.noise && (n_next % R) == (R / 2);
     // the step kernel without its epilogue rotation, then the pulse over all
@@ -272,10 +268,10 @@ cudaError_t batch_one_step(spin_batch* b, int from, long long n_next, cudaStream
     if (pulse) {
         float* s[3] = {(float*)b->buf[from ^ 1][0], (float*)b->buf[from ^ 1][1], (float*)b->buf[from ^ 1][2]};
         e = launch_pulse_batch(s, b->reps, b->oblocks, b->nblocks_obs, b->p.seed, b->d_interval, st,
-                               into(b, st));
+                               into);
         if (e != cudaSuccess) return e;
     }
-    if (n_next % R == 0) e = batch_observe(b, from ^ 1, true, st);
+    if (n_next % R == 0) e = batch_observe(b, from ^ 1, true, st, into);
     return e;
 }
 
@@ -411,7 +407,7 @@ int capture_batch_interval(spin_batch* b, int from) {
     int bb = from;
     cudaError_t e = cudaSuccess;
     for (int q = 1; q <= b->p.steps_per_pulse && e == cudaSuccess; ++q) {
-        e = batch_one_step(b, bb, q, cs);
+        e = batch_one_step(b, bb, q, cs, kIntervalGraph);
         bb ^= 1;
     }
     cudaGraph_t g = nullptr;
@@ -590,7 +586,8 @@ int spin_batch_autotune(spin_batch* b) {
 int spin_batch_step_pulse(spin_batch* b, int64_t nsteps) {
     if (!b || nsteps < 0) return SPIN_EINVAL;
     const int R = b->p.steps_per_pulse;
-    const bool replays = launch_into(b->st) == kStream;   // a caller's capture gets the steps' kernels themselves
+    const int into = launch_into(b->st);
+    const bool replays = into == kStream;   // a caller's capture gets the steps' kernels themselves
     while (nsteps > 0) {
         if (replays && b->n % R == 0 && nsteps >= R && b->eager_intervals > 0) {
             if (!b->graph[b->cur]) {
@@ -606,7 +603,7 @@ int spin_batch_step_pulse(spin_batch* b, int64_t nsteps) {
         const bool interval_start = b->n % R == 0 && nsteps >= R;
         const int steps = interval_start ? R : 1;
         for (int q = 0; q < steps; ++q) {
-            BATCH_CUDA(b, batch_one_step(b, b->cur, b->n + 1, b->st));
+            BATCH_CUDA(b, batch_one_step(b, b->cur, b->n + 1, b->st, into));
             b->cur ^= 1;
             b->n += 1;
         }
@@ -624,7 +621,7 @@ int spin_batch_step_pulse(spin_batch* b, int64_t nsteps) {
 
 int spin_batch_observables(spin_batch* b, double* out) {
     if (!b || !out) return SPIN_EINVAL;
-    BATCH_CUDA(b, batch_observe(b, b->cur, false, b->st));
+    BATCH_CUDA(b, batch_observe(b, b->cur, false, b->st, launch_into(b->st)));
     int status = 0;
     BATCH_CUDA(b, cudaMemcpyAsync(out, b->out, sizeof(double) * 5 * (size_t)b->nrep, cudaMemcpyDeviceToHost, b->st));
     BATCH_CUDA(b, cudaMemcpyAsync(&status, b->d_status, sizeof(int), cudaMemcpyDeviceToHost, b->st));

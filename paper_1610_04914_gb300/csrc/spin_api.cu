@@ -191,27 +191,22 @@ Phys<double> phys64(const spin_lattice* h) {
     return ph;
 }
 
-// Work on the handle's capture stream goes into an interval graph.
-int into(const spin_lattice* h, cudaStream_t st) {
-    return h->capture_stream && st == h->capture_stream ? kIntervalGraph : launch_into(st);
-}
-
 // Launch observables of buffer b; sample=true records into the ring.
-cudaError_t observe(spin_lattice* h, int b, bool sample, cudaStream_t st) {
+cudaError_t observe(spin_lattice* h, int b, bool sample, cudaStream_t st, int into) {
     if (h->elt == 4) {
         const float* s[3] = {(const float*)h->buf[b][0], (const float*)h->buf[b][1], (const float*)h->buf[b][2]};
         const float* hs[3] = {(const float*)h->hs[0], (const float*)h->hs[1], (const float*)h->hs[2]};
         return launch_observables<float>(s, hs, h->g, phys64(h), h->partials, h->nblocks_obs,
                                          sample ? h->out_sample : h->out_obs, sample ? h->ring : nullptr,
                                          SPIN_SAMPLE_RING, h->d_interval, h->d_sample_count, h->p.steps_per_pulse, st,
-                                         h->p.bc, into(h, st));
+                                         h->p.bc, into);
     }
     const double* s[3] = {(const double*)h->buf[b][0], (const double*)h->buf[b][1], (const double*)h->buf[b][2]};
     const double* hs[3] = {(const double*)h->hs[0], (const double*)h->hs[1], (const double*)h->hs[2]};
     return launch_observables<double>(s, hs, h->g, phys64(h), h->partials, h->nblocks_obs,
                                       sample ? h->out_sample : h->out_obs, sample ? h->ring : nullptr,
                                       SPIN_SAMPLE_RING, h->d_interval, h->d_sample_count, h->p.steps_per_pulse, st,
-                                      h->p.bc, into(h, st));
+                                      h->p.bc, into);
 }
 
 // One step n -> n+1 from buffer *buf on stream st, which becomes the buffer of
@@ -219,7 +214,7 @@ cudaError_t observe(spin_lattice* h, int b, bool sample, cudaStream_t st) {
 // the other; with an odd number of steps per interval the pulse of the FP32
 // fused paths, a kernel of its own, goes back, so that an interval ends where
 // it began and the state needs no copy to the caller's arrays (256^3: 60 us).
-cudaError_t launch_one_step(spin_lattice* h, int* buf, long long n_next, cudaStream_t st) {
+cudaError_t launch_one_step(spin_lattice* h, int* buf, long long n_next, cudaStream_t st, int into) {
     const int R = h->p.steps_per_pulse;
     const bool pulse = h->p.noise && is_pulse_step(n_next, R);
     const int from = *buf;
@@ -228,7 +223,7 @@ cudaError_t launch_one_step(spin_lattice* h, int* buf, long long n_next, cudaStr
     if (h->elt == 4) {
         StepLaunch<float> L = make_launch<float>(h, from, pulse);
         L.stream = st;
-        L.into = into(h, st);
+        L.into = into;
         if (pulse && (R & 1) && !L.force_generic && (h->tab.chain || rk5_fused_supports(L))) {
             to = from;
             for (int c = 0; c < 3; ++c) L.pulse_out[c] = static_cast<float*>(h->buf[to][c]);
@@ -237,12 +232,12 @@ cudaError_t launch_one_step(spin_lattice* h, int* buf, long long n_next, cudaStr
     } else {
         StepLaunch<double> L = make_launch<double>(h, from, pulse);
         L.stream = st;
-        L.into = into(h, st);
+        L.into = into;
         e = launch_step<double>(L);
     }
     if (e != cudaSuccess) return e;
     *buf = to;
-    if (n_next % R == 0) e = observe(h, to, true, st);
+    if (n_next % R == 0) e = observe(h, to, true, st, into);
     return e;
 }
 
@@ -257,7 +252,7 @@ int capture_interval(spin_lattice* h, int level, int from) {
     // the graph covers steps mR+1 .. (m+2^level)R; pulse and sample positions
     // depend only on n mod R, so step numbers from 1 on describe every interval
     for (int q = 1; q <= (R << level) && e == cudaSuccess; ++q) {
-        e = launch_one_step(h, &b, q, cs);
+        e = launch_one_step(h, &b, q, cs, kIntervalGraph);
     }
     h->graph_end[level][from] = b;
     cudaGraph_t graph = nullptr;
@@ -462,7 +457,8 @@ int spin_step_pulse(spin_lattice* h, int64_t nsteps) {
     if (!h || nsteps < 0) return SPIN_EINVAL;
     const int R = h->p.steps_per_pulse;
     // a caller's capture gets the steps' kernels themselves
-    const bool replays = launch_into(h->st) == kStream;
+    const int into = launch_into(h->st);
+    const bool replays = into == kStream;
     long long intervals = 0, ahead = 0;   // replayed by this call; of those, not yet captured behind
     while (nsteps > 0) {
         if (h->rec_active) {
@@ -481,7 +477,7 @@ int spin_step_pulse(spin_lattice* h, int64_t nsteps) {
                 continue;
             }
             if (h->n % R == 0 && nsteps >= R) h->eager_intervals++;
-            SPIN_CUDA(h, launch_one_step(h, &h->cur, h->n + 1, h->st));
+            SPIN_CUDA(h, launch_one_step(h, &h->cur, h->n + 1, h->st, into));
             h->n += 1;
             nsteps -= 1;
             int rc = record_if_due(h);
@@ -500,7 +496,7 @@ int spin_step_pulse(spin_lattice* h, int64_t nsteps) {
         const bool interval_start = h->n % R == 0 && nsteps >= R;
         const int steps = interval_start ? R : 1;
         for (int q = 0; q < steps; ++q) {
-            SPIN_CUDA(h, launch_one_step(h, &h->cur, h->n + 1, h->st));
+            SPIN_CUDA(h, launch_one_step(h, &h->cur, h->n + 1, h->st, into));
             h->n += 1;
         }
         nsteps -= steps;
@@ -520,7 +516,7 @@ int spin_step_pulse(spin_lattice* h, int64_t nsteps) {
 
 int spin_observables(spin_lattice* h, double M[3], double* E) {
     if (!h || !M || !E) return SPIN_EINVAL;
-    SPIN_CUDA(h, observe(h, h->cur, false, h->st));
+    SPIN_CUDA(h, observe(h, h->cur, false, h->st, launch_into(h->st)));
     // one copy from the observables to the status word (neighbours in the
     // workspace): a small copy to the host costs 5 us or more
     char host[1024];
